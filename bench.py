@@ -64,8 +64,8 @@ def workload(name):
 
 def kernel_name(w, prec_name):
     """The fused line-pass kernel the default launch shape runs for this grid."""
-    if prec_name == "c64" and min(w.nx, w.ny) >= 1024:
-        return "line_pass_persistent"
+    if prec_name == "c64" and min(w.nx, w.ny) >= 256:
+        return "line_pass_team"
     return "line_pass_kernel"
 
 
@@ -94,7 +94,7 @@ def fft_flops_per_point_step(nx, ny):
     return 20.0 * (np.log2(nx) + np.log2(ny)) + 76.0
 
 
-KERNEL_SOURCES = ("line_pass.cuh", "persist_pass.cuh", "launch_impl.cuh", "common.cuh")
+KERNEL_SOURCES = ("line_pass.cuh", "team_pass.cuh", "launch_impl.cuh", "common.cuh")
 
 
 def kernel_hash():

@@ -202,12 +202,12 @@ long dirac_krylov_iterations(const dirac_ctx *ctx);
 /* CTA shape of the two fused passes (each pass: FFT along a line, k-space multiply,
  * inverse FFT, combine, transposed store): 256 selects the smaller and 512 the larger of
  * the pass's two shapes for its line length (complex64: about 256 and 512 threads per
- * CTA; complex128: 1 to 4 lines per CTA, 32 to 512 threads), 1024 the persistent
- * prefetching variant (complex64, lines of 256..4096 points; one CTA per SM streams the
- * next lines into shared memory while it transforms the current ones); 0 = the default
- * (complex64: persistent for lines of 1024 points or more, the smaller shape for 128-
- * and 256-point lines, else the larger; complex128: the smaller shape for 1024-point
- * lines and lines of 128 points or fewer, else the larger). 64- and 128-point lines take
+ * CTA; complex128: 1 to 4 lines per CTA, 32 to 512 threads), 1024 the radix-16 team pass
+ * (complex64, lines of 256..4096 points; L/16 threads per line, the next lines stream into
+ * shared memory while the current ones are finished); 0 = the default (complex64: the team
+ * pass for lines of 256 points or more, the smaller shape for 128-point lines, else the
+ * larger; complex128: the smaller shape for 1024-point lines and lines of 128 points or
+ * fewer, else the larger). 64- and 128-point lines take
  * 2 or 16 lines per CTA; lines of 32 points or fewer and 4096-point lines have one shape
  * only. 256 or 512 plus
  * DIRAC_LAUNCH_ALT_RADIX selects the other radix schedule of the FFT passes, where the line
@@ -226,7 +226,7 @@ dirac_status dirac_set_launch(dirac_ctx *ctx, int threads_x_pass, int threads_y_
 dirac_status dirac_autotune(dirac_ctx *ctx, int reps, int *threads_x, int *threads_y);
 
 /* Test hook for failure detection: in the next dirac_step -- or, for a context submitted
- * to a batch, in the first tick that steps it -- the persistent pass's bulk-copy waits
+ * to a batch, in the first tick that steps it -- the team pass's bulk-copy waits
  * expect 16 bytes that never arrive, so each wait runs out after its bound (about 1.5 s),
  * the kernel returns early and the next synchronising call (dirac_synchronize, or
  * dirac_batch_poll / dirac_batch_synchronize) reports DIRAC_ETIMEOUT; the context stays
@@ -249,14 +249,10 @@ size_t dirac_footprint_bytes(const dirac_grid *grid, dirac_precision precision);
 /* ---- Batched stepping of many independent contexts (any mix of grid sizes).
  * Contexts of the same grid size form a class; one tick advances every active context
  * by up to steps_per_tick steps: per step and class, one x-pass and one y-pass launch
- * over all of that class's active contexts. With the environment variable
- * DIRAC_BATCH_TICK=1 set at dirac_batch_create, a class of square complex64 grids with
- * 256..2048-point lines whose passes run the persistent pass takes its whole tick in ONE
- * persistent launch instead: work items (step, pass, context, line group) come from a
- * queue, and each waits -- bounded, DIRAC_ETIMEOUT when the bound runs out -- until the
- * context's previous pass is finished (the same results; 4-8% slower per class on the
- * 256-instance mix, hence not the default). The classes run on parallel branches of a
- * CUDA graph captured once per class layout and replayed. Each context computes
+ * over all of that class's active contexts. The classes run on parallel branches of a
+ * CUDA graph captured once per class layout and replayed. (The environment variable
+ * DIRAC_BATCH_TICK of earlier versions, one slower launch per tick with the same results, has
+ * no effect.) Each context computes
  * exactly what dirac_step(ctx, n_steps, dt) computes (Sec. 5.2 Scheme II); a submitted
  * context belongs to the batch until it is released and must not be stepped, read or
  * destroyed meanwhile. Contexts must have the batch's precision. */
@@ -307,7 +303,7 @@ dirac_status dirac_batch_autotune(dirac_batch *batch, int reps);
 /* The CTA shapes, in dirac_set_launch terms (256, 512, 1024 threads, possibly with
  * DIRAC_LAUNCH_ALT_RADIX), that the class of
  * nx x ny contexts runs in this batch: the autotuner's choice, else the batch default
- * (complex64 lines of 256 points or more: the persistent pass; otherwise 512).
+ * (complex64 lines of 256 points or more: the team pass; otherwise 512).
  * DIRAC_EINVAL if the batch has no such class. */
 dirac_status dirac_batch_launch_shape(const dirac_batch *batch, int nx, int ny, int *threads_x,
                                       int *threads_y);

@@ -3,10 +3,7 @@
 // Contexts of the same grid size and precision form a class. One tick advances every
 // active context by up to K steps through a device table of per-instance pointers
 // [K steps][2 passes][capacity]. Each class launches, for each step, one x-pass and one
-// y-pass over all its active contexts; with DIRAC_BATCH_TICK=1, a class of square
-// complex64 grids whose passes run the persistent pass takes the whole tick in one
-// persistent launch instead (work items with per-instance dependencies,
-// line_pass_persistent's TICK mode). The classes run on parallel branches of a CUDA graph
+// y-pass over all its active contexts. The classes run on parallel branches of a CUDA graph
 // so that their work overlaps on the device. The graph of a tick is captured once per
 // class layout (classes present and their table capacities) and replayed; between
 // ticks only the tables and the active counts (device memory) change, so contexts are
@@ -20,7 +17,6 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
-#include <cstdlib>
 #include <map>
 #include <new>
 #include <string>
@@ -48,8 +44,9 @@ struct Class {
   void* tw_y = nullptr;
   void* tw_x_alt = nullptr;  // the same for the alternative radix schedule (if any)
   void* tw_y_alt = nullptr;
+  void* tw_x_team = nullptr;  // twiddles of the team pass (complex64)
+  void* tw_y_team = nullptr;
   int opt[2] = {-1, -1};  // CTA shape of the x / y pass chosen by the autotuner (-1: default)
-  int* d_sync = nullptr;  // batched tick launch: per-slot done counters [capacity], queue
 };
 
 struct Slot {
@@ -82,10 +79,6 @@ struct dirac_batch {
   unsigned long long ticks = 0, ticks_done_seen = 0;
   int* d_err = nullptr;
   long launches = 0;
-  // DIRAC_BATCH_TICK=1: one persistent launch per tick for the eligible classes (measured
-  // 4-8% slower per class than per-step launches on the 256-instance mix, so not the
-  // default)
-  bool tick_launch = false;
   std::string err;
 };
 
@@ -122,7 +115,8 @@ static void free_class(Class& c) {
   if (c.tw_y) cudaFree(c.tw_y);
   if (c.tw_x_alt) cudaFree(c.tw_x_alt);
   if (c.tw_y_alt) cudaFree(c.tw_y_alt);
-  if (c.d_sync) cudaFree(c.d_sync);
+  if (c.tw_x_team) cudaFree(c.tw_x_team);
+  if (c.tw_y_team) cudaFree(c.tw_y_team);
   c = Class();
 }
 
@@ -131,24 +125,21 @@ static dirac_status grow_class(dirac_batch* b, Class& c, int need) {
   int cap = c.capacity ? c.capacity : 4;
   while (cap < need) cap *= 2;
   void *h = nullptr, *d = nullptr;
-  int *hc = nullptr, *dc = nullptr, *ds = nullptr;
+  int *hc = nullptr, *dc = nullptr;
   BCK(cudaMallocHost(&h, tab_bytes(b, cap)), "batch tables");
   BCK(cudaMalloc(&d, tab_bytes(b, cap)), "batch tables");
   BCK(cudaMallocHost((void**)&hc, b->steps_per_tick * sizeof(int)), "batch counts");
   BCK(cudaMalloc((void**)&dc, b->steps_per_tick * sizeof(int)), "batch counts");
-  BCK(cudaMalloc((void**)&ds, (cap + 1) * sizeof(int)), "batch tick counters");
   // the previous tables may still be read by an enqueued tick
   BCK(cudaStreamSynchronize(b->stream), "batch grow");
   if (c.h_tab) cudaFreeHost(c.h_tab);
   if (c.d_tab) cudaFree(c.d_tab);
   if (c.h_count) cudaFreeHost(c.h_count);
   if (c.d_count) cudaFree(c.d_count);
-  if (c.d_sync) cudaFree(c.d_sync);
   c.h_tab = h;
   c.d_tab = d;
   c.h_count = hc;
   c.d_count = dc;
-  c.d_sync = ds;
   c.capacity = cap;
   return DIRAC_OK;
 }
@@ -230,49 +221,18 @@ static dirac_status launch_class_step(dirac_batch* b, Class& c, int k, cudaStrea
     a.sigma = pass;
     a.tw = (const Cx<T>*)(pass == 0 ? c.tw_x : c.tw_y);
     a.tw_alt = (const Cx<T>*)(pass == 0 ? c.tw_x_alt : c.tw_y_alt);
+    a.tw_team = (const Cx<T>*)(pass == 0 ? c.tw_x_team : c.tw_y_team);
     a.err = b->d_err;
     a.inst = (const InstPtrs<T>*)c.d_tab + ((size_t)k * 2 + pass) * c.capacity;
     a.n_inst = c.d_count + k;
     a.inst_capacity = c.capacity;
-    // the autotuner's choice, else: complex64 lines of 256 points or more the persistent
+    // the autotuner's choice, else: complex64 lines of 256 points or more the team
     // pass (its grid does not depend on the number of active instances), otherwise the
     // larger shape
     const int opt = c.opt[pass] >= 0 ? c.opt[pass] : (sizeof(T) == 4 && a.L >= 256) ? 2 : 1;
     BCK(launch_line_pass<T>(a, MODE_STEP, opt, st), "batched pass");
     b->launches += 1;
   }
-  return DIRAC_OK;
-}
-
-// A class whose passes both run the persistent pass on square complex64 grids of
-// 256..2048-point lines takes the whole tick in one persistent launch (work items with
-// per-instance dependencies); the others launch each step's x and y passes.
-template <typename T>
-static bool class_tick_launch(const dirac_batch* b, const Class& c) {
-  if (sizeof(T) != 4 || !b->tick_launch || c.nx != c.ny) return false;
-  if (c.nx < 256 || c.nx > 2048) return false;
-  for (int p = 0; p < 2; ++p)
-    if (c.opt[p] != -1 && c.opt[p] != 2) return false;
-  return true;
-}
-
-template <typename T>
-static dirac_status launch_class_tick(dirac_batch* b, Class& c, int K, cudaStream_t st) {
-  BCK(cudaMemsetAsync(c.d_sync, 0, (c.capacity + 1) * sizeof(int), st), "tick counters");
-  LinePassArgs<T> a{};
-  a.L = c.nx;
-  a.n_lines = c.ny;
-  a.sigma = 0;  // per work item
-  a.tw = (const Cx<T>*)c.tw_x;  // the same table serves both passes (nx == ny)
-  a.err = b->d_err;
-  a.inst = (const InstPtrs<T>*)c.d_tab;
-  a.n_inst = c.d_count;
-  a.inst_capacity = c.capacity;
-  a.tick_k = K;
-  a.tick_done = c.d_sync;
-  a.tick_queue = c.d_sync + c.capacity;
-  BCK(launch_line_pass_tick<T>(a, st), "batched tick");
-  b->launches += 1;
   return DIRAC_OK;
 }
 
@@ -296,12 +256,8 @@ static dirac_status tick_graph(dirac_batch* b, int K) {
     Class& c = kv.second;
     if (e != cudaSuccess || st != DIRAC_OK) break;
     e = cudaStreamWaitEvent(c.stream, b->fork, 0);
-    if (e == cudaSuccess && class_tick_launch<T>(b, c)) {
-      st = launch_class_tick<T>(b, c, K, c.stream);
-    } else {
-      for (int k = 0; k < K && e == cudaSuccess && st == DIRAC_OK; ++k)
-        st = launch_class_step<T>(b, c, k, c.stream);
-    }
+    for (int k = 0; k < K && e == cudaSuccess && st == DIRAC_OK; ++k)
+      st = launch_class_step<T>(b, c, k, c.stream);
     cudaEvent_t j = nullptr;
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&j, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(j, c.stream);
@@ -383,7 +339,7 @@ static dirac_status run_tick(dirac_batch* b, int K) {
 }
 
 // Shapes worth timing for a pass over lines of L points (the launcher maps the others onto
-// these): complex64 256..4096 points also the persistent pass; lines of 32 points or
+// these): complex64 256..4096 points also the team pass; lines of 32 points or
 // fewer and 4096-point lines have one non-persistent shape.
 template <typename T>
 static std::vector<int> shape_candidates(int L) {
@@ -450,6 +406,7 @@ static dirac_status autotune_class(dirac_batch* b, Class& c, int reps, bool* cha
     a.sigma = pass;
     a.tw = (const Cx<T>*)(pass == 0 ? c.tw_x : c.tw_y);
     a.tw_alt = (const Cx<T>*)(pass == 0 ? c.tw_x_alt : c.tw_y_alt);
+    a.tw_team = (const Cx<T>*)(pass == 0 ? c.tw_x_team : c.tw_y_team);
     a.err = b->d_err;
     a.inst = d_tab + (size_t)pass * n;
     a.n_inst = d_cnt;
@@ -496,10 +453,6 @@ dirac_status dirac_batch_create(size_t hbm_budget_bytes, dirac_precision precisi
   if (!b) return DIRAC_ENOMEM;
   b->prec = precision;
   b->budget = hbm_budget_bytes;
-  {
-    const char* t = getenv("DIRAC_BATCH_TICK");
-    b->tick_launch = t && t[0] == '1' && t[1] == '\0';
-  }
   b->steps_per_tick = steps_per_tick;
   cudaError_t e = cudaSuccess;
   if (cuda_stream) {
@@ -590,6 +543,14 @@ dirac_status dirac_batch_submit(dirac_batch* b, dirac_ctx* inst, long n_steps, d
     } else {
       if (ax) BCK(launch_twiddles<double>(c.nx, ax, (Cx<double>*)c.tw_x_alt, b->stream), "twiddles");
       if (ay) BCK(launch_twiddles<double>(c.ny, ay, (Cx<double>*)c.tw_y_alt, b->stream), "twiddles");
+    }
+    if (b->prec == DIRAC_C64 && team_length(c.nx)) {
+      BCK(cudaMalloc(&c.tw_x_team, c.nx * cx), "class twiddles");
+      BCK(launch_team_twiddles<float>(c.nx, (Cx<float>*)c.tw_x_team, b->stream), "twiddles");
+    }
+    if (b->prec == DIRAC_C64 && team_length(c.ny)) {
+      BCK(cudaMalloc(&c.tw_y_team, c.ny * cx), "class twiddles");
+      BCK(launch_team_twiddles<float>(c.ny, (Cx<float>*)c.tw_y_team, b->stream), "twiddles");
     }
     BCK(cudaStreamSynchronize(b->stream), "class twiddles");
   }

@@ -27,6 +27,11 @@ __device__ __forceinline__ bool dbg_in(size_t idx, size_t bound) {
   return true;
 }
 
+// idx, or 0 when a debug build finds it out of bounds (a harmless slot of the same array)
+__device__ __forceinline__ size_t dbg_at(size_t idx, size_t bound) {
+  return dbg_in(idx, bound) ? idx : 0;
+}
+
 // Complex number in registers / shared memory.
 template <typename T>
 struct __align__(2 * sizeof(T)) Cx {
@@ -142,7 +147,7 @@ __device__ __forceinline__ Q4<T> apply_u(Q4<T> u, Q4<T> p) {
 
 namespace dgb {
 
-// ---- asynchronous bulk copies and mbarriers (sm_90+ PTX), used by the persistent pass
+// ---- asynchronous bulk copies and mbarriers (sm_90+ PTX), used by the team pass
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -174,9 +179,6 @@ __device__ __forceinline__ void bulk_copy_g2s(void* dst, const void* src, uint32
       "l"(src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }
-__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
 __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -201,75 +203,24 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
   return true;
 }
 
-// GPU-scope acquire load and release increment of a global counter (cross-CTA ordering of
-// the batched tick's work items).
-__device__ __forceinline__ int ld_acquire_gpu(const int* p) {
-  int v;
-  asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+// Position of frequency k in the multiplier tables of the radix-16 team pass (lines of L =
+// 256..4096 points, team_pass.cuh): thread j = R2 k0 + v of the line's L/16 (R2 = L/256)
+// holds frequency k0 + 16 (v + R2 q) + 256 k2 in element e = q R2 + k2, and entry e of thread
+// j sits at e L/16 + j, so that a warp reads consecutive entries.
+__host__ __device__ constexpr int team_perm(int L, int k) {
+  return (((k >> 4) & 15) / (L / 256) * (L / 256) + (k >> 8)) * (L / 16) + (k & 15) * (L / 256) +
+         ((k >> 4) & 15) % (L / 256);
 }
-__device__ __forceinline__ void red_release_gpu_add(int* p, int v) {
-  asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-// Orders this thread's earlier generic-proxy accesses of global memory before its later
-// async-proxy (bulk copy) accesses.
-__device__ __forceinline__ void fence_proxy_async_global() {
-  asm volatile("fence.proxy.async.global;" ::: "memory");
-}
+__host__ __device__ constexpr bool team_length(int L) { return L >= 256 && L <= 4096; }
 
-// Position of frequency k (< 1024) in the step-multiplier table of 1024-point lines that
-// the 1024-point persistent pass reads: its digit-swap FFT leaves frequency
-// s + 8 l4 + 64 m + 512 v0 in element m of the thread with warp slice s and lane bits
-// l4 = lane >> 2, v0 = (lane >> 1) & 1, so the table is ordered (m, v0, s, l4) and the 16
-// entries a warp reads for one m are two runs of 8 consecutive entries.
-__host__ __device__ constexpr int perm1024(int k) {
-  return ((k >> 6) & 7) * 128 + ((k >> 9) & 1) * 64 + (k & 7) * 8 + ((k >> 3) & 7);
+// Programmatic dependent launch: waits until the kernels this one depends on have completed
+// and their writes are visible (at once when launched without the attribute), and lets the
+// next kernel of the stream be scheduled (it waits here in turn).
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
-
-// ---- asynchronous stores from shared memory (bulk-group completion)
-// Tiled tensor store of one 2D box from shared memory (128-B aligned) to global memory,
-// at element coordinates (x, y) of the tensor map; x times the element size a multiple of
-// 16 bytes, neither coordinate negative.
-__device__ __forceinline__ void tma_store_2d(const void* tmap, uint32_t smem, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%2, %3}], [%1];" ::"l"(tmap),
-      "r"(smem), "r"(x), "r"(y)
-      : "memory");
-}
-// Bulk store of `bytes` (a multiple of 16) from shared to global memory, both 16-B aligned.
-__device__ __forceinline__ void bulk_copy_s2g(void* dst, uint32_t smem, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst),
-               "r"(smem), "r"(bytes)
-               : "memory");
-}
-__device__ __forceinline__ void bulk_commit() {
-  asm volatile("cp.async.bulk.commit_group;" ::: "memory");
-}
-// every committed bulk store of this thread has read its shared-memory source
-__device__ __forceinline__ void bulk_wait_read_all() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-}
-// every committed bulk store of this thread is complete
-__device__ __forceinline__ void bulk_wait_all() {
-  asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-}
-
-// Address of the same shared-memory variable in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-  return r;
-}
-template <typename T>
-__device__ __forceinline__ Q4<T> ld_dsmem_q4(uint32_t addr);
-template <>
-__device__ __forceinline__ Q4<float> ld_dsmem_q4<float>(uint32_t addr) {
-  Q4<float> v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(addr)
-               : "memory");
-  return v;
+__device__ __forceinline__ void pdl_launch_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 // ---- tensor memory (tcgen05, sm_100a+) used as per-thread parking space. A CTA holds
@@ -312,35 +263,8 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&r)[16]) {
       : "r"(taddr)
       : "memory");
 }
-// r[0..7] <- 8 consecutive columns of this thread's lane (complete after tmem_wait_ld)
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&r)[8]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]),
-        "=f"(r[7])
-      : "r"(taddr)
-      : "memory");
-}
-__device__ __forceinline__ void tmem_st8(uint32_t taddr, const float (&r)[8]) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr),
-      "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7])
-      : "memory");
-}
-// r[0..1] <- 2 consecutive columns of this thread's lane (complete after tmem_wait_ld)
-__device__ __forceinline__ void tmem_ld2(uint32_t taddr, float (&r)[2]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0, %1}, [%2];"
-               : "=f"(r[0]), "=f"(r[1])
-               : "r"(taddr)
-               : "memory");
-}
 // Waits for this thread's tensor-memory loads; naming the destination registers as
 // operands keeps every use of them after the wait.
-__device__ __forceinline__ void tmem_wait_ld_regs(float (&r)[8]) {
-  asm volatile("tcgen05.wait::ld.sync.aligned;"
-               : "+f"(r[0]), "+f"(r[1]), "+f"(r[2]), "+f"(r[3]), "+f"(r[4]), "+f"(r[5]),
-                 "+f"(r[6]), "+f"(r[7])::"memory");
-}
 __device__ __forceinline__ void tmem_wait_ld_regs(float (&r)[16]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+f"(r[0]), "+f"(r[1]), "+f"(r[2]), "+f"(r[3]), "+f"(r[4]), "+f"(r[5]),
@@ -353,22 +277,6 @@ __device__ __forceinline__ void named_barrier(int id, int count) {
 }
 __device__ __forceinline__ void tmem_wait_st() {
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
-// Cluster barrier without release semantics: orders execution only (no wait for this
-// thread's outstanding global stores); the wait side keeps acquire.
-// split cluster barrier: arrive without release semantics, and the matching wait
-__device__ __forceinline__ void cluster_arrive_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_sync_relaxed() {
-  asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" :::
-                   "memory");
 }
 
 }  // namespace dgb

@@ -29,6 +29,7 @@ struct dirac_ctx {
   void *beta1_im = nullptr, *beta2T_im = nullptr;  // complex stretching: Im(b - 1)
   void *u_n = nullptr, *u_t = nullptr, *u2_t = nullptr;
   void *tw_x_alt = nullptr, *tw_y_alt = nullptr;  // twiddles of the alternative radix
+  void *tw_x_team = nullptr, *tw_y_team = nullptr;  // twiddles of the team pass (complex64)
   void *tw_x = nullptr, *tw_y = nullptr, *mult_x = nullptr, *mult_y = nullptr,
        *dmult_x = nullptr, *dmult_y = nullptr;
   double* staging = nullptr;  // [2][ny][nx] complex128 for host transfers
@@ -53,8 +54,8 @@ struct dirac_ctx {
   void** k_vptr = nullptr;          // device copy of the basis pointers
   double* k_partials = nullptr;     // inner-product partial sums
   double* k_coef = nullptr;         // combination coefficients (device)
-  // complex64 axes of 1024 points: the step tables (x at dt and dt/2, y) in the order of
-  // perm1024, for the 1024-point persistent pass
+  // complex64 axes of 256 points or more: the step tables (x at dt and dt/2, y) in the
+  // order of team_perm, for the team pass
   void *mult_px = nullptr, *mult_py = nullptr, *mult_pxh = nullptr;
   void *mult_xh = nullptr, *u2_n = nullptr;  // symmetric order: x multipliers at dt/2,
                                              // U^2 in the normal layout
@@ -75,5 +76,5 @@ struct dirac_ctx {
 // Library-internal helpers implemented in dirac_api.cu.
 dirac_status dgb_tables_for_dt(dirac_ctx* ctx, double dt);
 size_t dgb_footprint_bytes(int nx, int ny, dirac_precision prec);
-// Launch option (0, 1, 2 = persistent) for a pass of line length L.
+// Launch option (0, 1, 2 = team pass) for a pass of line length L.
 int dgb_pass_opt(const dirac_ctx* ctx, int threads, int L);

@@ -87,14 +87,13 @@ static int pass_opt(const dirac_ctx* ctx, int shape, int L) {
   if (threads == 256) return 0;
   if (threads == 512) return 1;
   if (threads == 1024) return 2;
-  // Default, by measurement on the strained-graphene grids: complex64 the persistent
-  // prefetching pass for lines of 1024 points or more, the smaller shape for 128- and
-  // 256-point lines (0.016 against 0.018 ms per 256^2 step, 0.0166 against 0.0187 per
-  // 128^2), else the larger; complex128 the smaller shape for 1024-point lines (one line
-  // per CTA: 1024 CTAs spread over the SMs to within one line, 0.74 against 0.89 ms per
-  // 1024^2 step) and for lines of 128 points or fewer (0.050 against 0.168 ms per 128^2
-  // step), else the larger.
-  if (ctx->prec == DIRAC_C64) return L >= 1024 ? 2 : (L == 256 || L == 128) ? 0 : 1;
+  // Default, by measurement: complex64 the team pass for lines of 256 points or more (256^2
+  // 0.0109 against 0.0118 ms per step for the radix-8 pass, 1024^2 0.0291 against 0.039), the
+  // smaller shape for 128-point lines (0.0166 against 0.0187 per 128^2), else the larger;
+  // complex128 the smaller shape for 1024-point lines (one line per CTA: 1024 CTAs spread
+  // over the SMs to within one line, 0.74 against 0.89 ms per 1024^2 step) and for lines of
+  // 128 points or fewer (0.050 against 0.168 ms per 128^2 step), else the larger.
+  if (ctx->prec == DIRAC_C64) return L >= 256 ? 2 : L == 128 ? 0 : 1;
   return (L == 1024 || L <= 128) ? 0 : 1;
 }
 
@@ -107,9 +106,6 @@ static dirac_status device_error(dirac_ctx* ctx) {
     return fail(ctx, DIRAC_ECUDA, "debug build: an index check of a line pass failed");
   if (flag) {
     cudaMemset(ctx->d_err, 0, sizeof(int));
-    if (flag == 2)  // the 4096-point pass's staging tile (never expected)
-      return fail(ctx, DIRAC_ECUDA, "a line pass found its shared-memory staging tile "
-                                    "misaligned for tensor stores; the state is not valid");
     return fail(ctx, DIRAC_ETIMEOUT, "a bounded device wait ran out; the state is not valid");
   }
   return DIRAC_OK;
@@ -124,6 +120,7 @@ static LinePassArgs<T> pass_args(dirac_ctx* ctx, int axis) {
   a.sigma = axis;
   a.tw = (const Cx<T>*)(axis == 0 ? ctx->tw_x : ctx->tw_y);
   a.tw_alt = (const Cx<T>*)(axis == 0 ? ctx->tw_x_alt : ctx->tw_y_alt);
+  a.tw_team = (const Cx<T>*)(axis == 0 ? ctx->tw_x_team : ctx->tw_y_team);
   return a;
 }
 
@@ -164,12 +161,14 @@ static dirac_status tables_for_dt(dirac_ctx* ctx, double dt) {
        "x multipliers (dt/2)");
     ctx->launches += 1;
   }
-  // the same tables in the 1024-point persistent pass's order
+  // the same tables in the team pass's order
   const void* perm_src[3] = {ctx->mult_x, ctx->mult_y, ctx->mult_xh};
   void* perm_dst[3] = {ctx->mult_px, ctx->mult_py, ctx->mult_pxh};
   for (int t = 0; t < 3; ++t) {
     if (!perm_dst[t]) continue;
-    CK(launch_perm1024<T>((const Q4<T>*)perm_src[t], (Q4<T>*)perm_dst[t], st), "multiplier order");
+    CK(launch_team_perm<T>(t == 1 ? ctx->ny : ctx->nx, (const Q4<T>*)perm_src[t],
+                           (Q4<T>*)perm_dst[t], st),
+       "multiplier order");
     ctx->launches += 1;
   }
   ctx->dt_cached = dt;
@@ -670,10 +669,14 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
     CK(dalloc(ctx, &ctx->tw_y_alt, ny * sizeof(Cx<T>)), "allocate tables");
   CK(dalloc(ctx, &ctx->mult_x, nx * sizeof(Q4<T>)), "allocate tables");
   CK(dalloc(ctx, &ctx->mult_y, ny * sizeof(Q4<T>)), "allocate tables");
-  if (sizeof(T) == 4 && nx == 1024)  // the 1024-point persistent pass's table order
+  if (sizeof(T) == 4 && team_length(nx)) {  // the team pass's table order and twiddles
     CK(dalloc(ctx, &ctx->mult_px, nx * sizeof(Q4<T>)), "allocate tables");
-  if (sizeof(T) == 4 && ny == 1024)
+    CK(dalloc(ctx, &ctx->tw_x_team, nx * sizeof(Cx<T>)), "allocate tables");
+  }
+  if (sizeof(T) == 4 && team_length(ny)) {
     CK(dalloc(ctx, &ctx->mult_py, ny * sizeof(Q4<T>)), "allocate tables");
+    CK(dalloc(ctx, &ctx->tw_y_team, ny * sizeof(Cx<T>)), "allocate tables");
+  }
   CK(dalloc(ctx, &ctx->dmult_x, nx * sizeof(Q4<T>)), "allocate tables");
   CK(dalloc(ctx, &ctx->dmult_y, ny * sizeof(Q4<T>)), "allocate tables");
   CK(dalloc(ctx, (void**)&ctx->staging, 2 * n * 2 * sizeof(double)), "allocate staging");
@@ -751,6 +754,10 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
     CK(launch_twiddles<T>(nx, line_pass_radix_alt<T>(nx), (Cx<T>*)ctx->tw_x_alt, st), "twiddles");
   if (ctx->tw_y_alt)
     CK(launch_twiddles<T>(ny, line_pass_radix_alt<T>(ny), (Cx<T>*)ctx->tw_y_alt, st), "twiddles");
+  if (ctx->tw_x_team)
+    CK(launch_team_twiddles<T>(nx, (Cx<T>*)ctx->tw_x_team, st), "twiddles");
+  if (ctx->tw_y_team)
+    CK(launch_team_twiddles<T>(ny, (Cx<T>*)ctx->tw_y_team, st), "twiddles");
   CK(launch_deriv_mult<T>(nx, ctx->ax, (Q4<T>*)ctx->dmult_x, st), "derivative table");
   CK(launch_deriv_mult<T>(ny, ctx->ay, (Q4<T>*)ctx->dmult_y, st), "derivative table");
   ctx->launches += 7;
@@ -803,7 +810,7 @@ static dirac_status tune_pass(dirac_ctx* ctx, int axis, int reps, int* best, flo
   *best = 0;
   *best_ms = 1e30f;
   for (int t : options) {
-    if (t == 1024 && !(sizeof(T) == 4 && L >= 256)) continue;  // persistent: complex64 only
+    if (t == 1024 && !(sizeof(T) == 4 && L >= 256)) continue;  // team pass: complex64 only
     if ((t & DIRAC_LAUNCH_ALT_RADIX) && !line_pass_radix_alt<T>(L)) continue;
     const int opt = pass_opt(ctx, t, L);
     cudaError_t e = cudaSuccess;

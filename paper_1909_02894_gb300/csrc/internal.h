@@ -10,18 +10,42 @@
 
 namespace dgb {
 
+// Kernel launch with, if `pdl`, programmatic stream serialization: the kernel may be scheduled
+// while its predecessor in the stream still runs (it calls pdl_wait before it touches memory),
+// and, if cluster > 1, that cluster size.
+template <typename... P, typename... A>
+inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                              cudaStream_t st, bool pdl, int cluster, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[2];
+  unsigned n = 0;
+  if (pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = cluster;
+    attr[n].val.clusterDim.y = 1;
+    attr[n++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Sets the text that dirac_last_error(NULL) returns (errors without a context).
 void set_global_error(const std::string& msg);
 
 // Enqueues one fused line pass (MODE_STEP or MODE_DERIV). opt selects the CTA shape:
-// 0 = about 256 threads per CTA, 1 = 512 threads, 2 = the persistent prefetching
-// variant (complex64 step mode, lines of 256..4096 points; otherwise as 1).
+// 0 = about 256 threads per CTA, 1 = 512 threads, 2 = the radix-16 team pass (complex64
+// step mode, lines of 256..4096 points; otherwise as 1).
 template <typename T>
 cudaError_t launch_line_pass(const LinePassArgs<T>& a, int mode, int opt, cudaStream_t st);
-// Every step of a batch tick of one class in one persistent launch (complex64, square
-// grids, 256..2048-point lines; cudaErrorInvalidValue otherwise).
-template <typename T>
-cudaError_t launch_line_pass_tick(const LinePassArgs<T>& a, cudaStream_t st);
 // Elements per thread (8 or 16) the line pass uses for line length L; the twiddle table
 // of that axis must be built for the same value.
 template <typename T>
@@ -72,8 +96,11 @@ template <typename T>
 cudaError_t launch_twiddles(int n, int e, Cx<T>* tw, cudaStream_t st);
 template <typename T>
 cudaError_t launch_step_mult(int n, double a, double dt, Q4<T>* mult, cudaStream_t st);
+// Team pass (lines of n = 256..4096 points): a multiplier table in its order, its twiddles.
 template <typename T>
-cudaError_t launch_perm1024(const Q4<T>* src, Q4<T>* dst, cudaStream_t st);
+cudaError_t launch_team_perm(int n, const Q4<T>* src, Q4<T>* dst, cudaStream_t st);
+template <typename T>
+cudaError_t launch_team_twiddles(int n, Cx<T>* tw, cudaStream_t st);
 template <typename T>
 cudaError_t launch_deriv_mult(int n, double a, Q4<T>* mult, cudaStream_t st);
 

@@ -1,11 +1,9 @@
 // Launch logic of the fused line pass, instantiated once per precision.
 #pragma once
-#include <cuda.h>
 #include <cuda_runtime.h>
-#include <string.h>
 
 #include "internal.h"
-#include "persist_pass.cuh"
+#include "team_pass.cuh"
 
 namespace dgb {
 
@@ -24,6 +22,14 @@ constexpr int radix_e(int L) {
 template <typename T>
 constexpr int radix_alt(int L) {
   return L < 256 ? 0 : sizeof(T) == 4 ? (L <= 4096 ? 16 : 0) : (L <= 2048 ? 8 : 0);
+}
+
+static int sm_count() {
+  static int cached[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cached[dev]) cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev);
+  return cached[dev];
 }
 
 template <typename T, int L, int LPC, int MODE, int E = radix_e<T>(L)>
@@ -45,21 +51,13 @@ static cudaError_t launch_one(const LinePassArgs<T>& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     configured[dev] = true;
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((a.inst ? a.inst_capacity : 1) * (a.n_lines / LPC), 1, 1);
-  cfg.blockDim = dim3(Gm::THREADS, 1, 1);
-  cfg.dynamicSmemBytes = Gm::SMEM;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  if (Gm::CS > 1) {
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = Gm::CS;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-  }
-  return cudaLaunchKernelEx(&cfg, kern, a);
+  const int grid = (a.inst ? a.inst_capacity : 1) * (a.n_lines / LPC);
+  // Programmatic dependent launch saves 0.0023 ms per pass. Not for complex128 passes of
+  // several waves, which it made slower (1024^2: 0.755 against 0.734 ms per step; 512^2, one
+  // wave: 0.194 against 0.199), nor in a batch's graph, whose kernels start faster without
+  // (13 128^2 instances: 0.0179 with, 0.0158 ms per step without).
+  const bool pdl = !a.inst && (sizeof(T) == 4 || grid <= 2 * sm_count());
+  return launch_pdl(kern, dim3(grid), dim3(Gm::THREADS), Gm::SMEM, st, pdl, Gm::CS, a);
 }
 
 // Two CTA shapes per line length (opt 0 smaller, opt 1 larger; lines of 32 points or
@@ -118,94 +116,61 @@ static cudaError_t dispatch(const LinePassArgs<T>& a, int opt, cudaStream_t st) 
   }
 }
 
-static int sm_count() {
-  static int cached[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!cached[dev]) cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev);
-  return cached[dev];
-}
-
-// Tensor map of a transposed complex64 output out[rows][n_lines] (16-byte points) as a 2D
-// float tensor of 4 n_lines x rows, with boxes of 4 x 256 (one point of 256 rows): a
-// staged 4096-point line is 16 such boxes. The encoder is taken from the driver at the
-// first call.
-static cudaError_t out_tensor_map(CUtensorMap* m, void* out, int n_lines, int rows) {
-  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                              const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                              const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-  static const Encode encode = []() -> Encode {
-    void* fn = nullptr;
-    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault,
-                                         &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      return nullptr;
-    return reinterpret_cast<Encode>(fn);
-  }();
-  if (!encode) return cudaErrorNotSupported;
-  if (n_lines < 1 || rows % 256 != 0 || (reinterpret_cast<uintptr_t>(out) & 15))
+// The radix-16 team pass (complex64 step mode, 256..4096-point lines): as many CTAs as can
+// be resident (128 registers: 512 threads per SM; each CTA takes its share of the tensor
+// memory), at most one per work unit. The CTAs per SM follow from TGeo, as the occupancy
+// query reports one CTA per SM for kernels that allocate tensor memory.
+template <int L, int LPC, bool PAIR, bool BATCH, int SIGMA>
+static cudaError_t launch_team_as(const LinePassArgs<float>& a0, cudaStream_t st) {
+  using G = TGeo<L, LPC, PAIR>;
+  // one U field per pass; b - 1 real
+  if (!a0.err || !a0.tw_team || (!BATCH && !a0.mult_perm) || a0.n_lines % G::LPU != 0 ||
+      (a0.u_load && a0.u_store) || a0.beta_im)
     return cudaErrorInvalidValue;
-  const cuuint64_t dims[2] = {(cuuint64_t)4 * (cuuint64_t)n_lines, (cuuint64_t)rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)n_lines * 16};  // bytes between rows
-  const cuuint32_t box[2] = {4, 256};
-  const cuuint32_t elem_strides[2] = {1, 1};
-  const CUresult r = encode(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, out, dims, strides, box,
-                            elem_strides, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                            CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
-// Persistent prefetching variant (complex64 step mode, 256..4096-point lines): one
-// 1024-thread CTA per SM (clusters of 2 for 4096-point lines), as
-// many as can be resident, at most one per group of 4096 points.
-template <int L>
-static cudaError_t launch_persist(const LinePassArgs<float>& a, cudaStream_t st) {
-  using PG = PGeo<float, L>;
-  // one U field per pass: the U landing zone holds either the load-side or the
-  // store-side matrices (batched launches keep the same rule per instance)
-  if (!a.err || a.n_lines % PG::GL != 0 || (a.u_load && a.u_store) || a.beta_im) return cudaErrorInvalidValue;
-  auto kern = a.inst ? line_pass_persistent<float, L, true> : line_pass_persistent<float, L, false>;
-  static int max_clusters[2][64] = {};
+  LinePassArgs<float> a = a0;
+  a.tw = a0.tw_team;
+  auto kern = line_pass_team<L, LPC, PAIR, BATCH, SIGMA>;
+  static bool configured[64] = {false};
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
   if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(PG::THREADS, 1, 1);
-  cfg.dynamicSmemBytes = PG::SMEM;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = PG::CS;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int& cached = max_clusters[a.inst ? 1 : 0][dev];
-  if (!cached) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG::SMEM);
+  if (!configured[dev]) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
     if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3(PG::CS * 64, 1, 1);
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
-    if (e != cudaSuccess) return e;
-    if (n <= 0) return cudaErrorInvalidConfiguration;
-    cached = n;
+    configured[dev] = true;
   }
-  const int groups = (a.inst ? a.inst_capacity : 1) * (a.n_lines / PG::LPI);
-  int clusters = cached;
-  if (clusters > groups / PG::CS) clusters = groups / PG::CS;
-  cfg.gridDim = dim3(clusters * PG::CS, 1, 1);
-  CUtensorMap tmap;
-  memset(&tmap, 0, sizeof(tmap));
-  if (L == 4096 && !a.inst && !a.store_normal) {  // the tensor stores of the output tiles
-    e = out_tensor_map(&tmap, a.out, a.n_lines, L);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaLaunchKernelEx(&cfg, kern, a, groups, a.err, tmap);
+  const int units = (BATCH ? a.inst_capacity : 1) * (a.n_lines / G::LPU);
+  const int ctas = (units + G::GROUPS - 1) / G::GROUPS, most = G::MINB * sm_count();
+  return launch_pdl(kern, dim3(ctas < most ? ctas : most), dim3(G::THREADS), G::SMEM, st, true, 0,
+                    a, units, a.err);
+}
+
+// How the lines are spread, by the points of a launch (all instances together):
+//  up to 2^18  small CTAs (512 points at once), as many as possible: latency decides;
+//  up to 2^20  CTAs of 2048 points, output staged in segments of 2048 / L lines;
+//  above       pairs of lines per team, whole 32-byte sectors written from registers without
+//              staging (batches from 2^21: their capacity, which sizes the launch, exceeds the
+//              number of running instances by up to 2).
+// Measured per step of two passes (ms), small | staged | pairs: 256^2 0.0109 | 0.0160 | 0.0239,
+// 512 x 256 0.0121 | 0.0158, 512^2 0.0149 | 0.0154 | 0.0240, 1024 x 256 0.0153 | 0.0172 |
+// 0.0257, 512 x 1024 0.0249 | 0.0193, 1024^2 - | 0.0325 | 0.0291, 512 x 2048 - | 0.0361 |
+// 0.0301, 2048^2 - | 0.138 | 0.085.
+template <int L, bool BATCH, int SIGMA>
+static cudaError_t launch_team_sized(const LinePassArgs<float>& a, cudaStream_t st) {
+  constexpr int SMALL = L >= 512 ? 1 : 512 / L, LPC = L >= 2048 ? 1 : 2048 / L;
+  const size_t points = (size_t)(BATCH ? a.inst_capacity : 1) * a.n_lines * L;
+  if (points >= ((size_t)1 << (BATCH ? 21 : 20)))
+    return launch_team_as<L, LPC, true, BATCH, SIGMA>(a, st);
+  if (points <= ((size_t)1 << 18)) return launch_team_as<L, SMALL, false, BATCH, SIGMA>(a, st);
+  return launch_team_as<L, LPC, false, BATCH, SIGMA>(a, st);
+}
+
+template <int L>
+static cudaError_t launch_team(const LinePassArgs<float>& a, cudaStream_t st) {
+  if (a.inst)
+    return a.sigma == 0 ? launch_team_sized<L, true, 0>(a, st) : launch_team_sized<L, true, 1>(a, st);
+  return a.sigma == 0 ? launch_team_sized<L, false, 0>(a, st) : launch_team_sized<L, false, 1>(a, st);
 }
 
 // The alternative radix schedule (radix_alt), opt 3 the smaller and opt 4 the larger of two
@@ -248,70 +213,16 @@ cudaError_t launch_line_pass(const LinePassArgs<T>& a, int mode, int opt, cudaSt
   if constexpr (sizeof(T) == 4) {
     if (opt == 2) {
       switch (a.L) {
-        case 256: return launch_persist<256>(a, st);
-        case 512: return launch_persist<512>(a, st);
-        case 1024: return launch_persist<1024>(a, st);
-        case 2048: return launch_persist<2048>(a, st);
-        case 4096: return launch_persist<4096>(a, st);
+        case 256: return launch_team<256>(a, st);
+        case 512: return launch_team<512>(a, st);
+        case 1024: return launch_team<1024>(a, st);
+        case 2048: return launch_team<2048>(a, st);
+        case 4096: return launch_team<4096>(a, st);
         default: break;
       }
     }
   }
   return dispatch<T, MODE_STEP>(a, opt >= 1 ? 1 : 0, st);
-}
-
-// Batched tick launch (complex64, square grids, 256..2048-point lines): every step of
-// the tick in one persistent launch, one 1024-thread CTA per SM, work items from a
-// queue with per-instance dependencies (see line_pass_persistent). a.inst, a.n_inst and
-// the tick fields describe the whole tick; a.tw serves both passes (equal line lengths).
-template <int L>
-static cudaError_t launch_persist_tick(const LinePassArgs<float>& a, cudaStream_t st) {
-  using PG = PGeo<float, L>;
-  if constexpr (PG::CS != 1) {
-    return cudaErrorInvalidValue;
-  } else {
-    if (!a.err || !a.inst || !a.n_inst || !a.tick_queue || !a.tick_done || a.tick_k < 1 ||
-        a.tick_k > PG::TICK_K_MAX ||
-        a.n_lines != L || a.n_lines % PG::GL != 0 || a.beta_im)
-      return cudaErrorInvalidValue;
-    auto kern = line_pass_persistent<float, L, true, true>;
-    static int max_blocks[64] = {};
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!max_blocks[dev]) {
-      e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG::SMEM);
-      if (e != cudaSuccess) return e;
-      int per_sm = 0;
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, PG::THREADS, PG::SMEM);
-      if (e != cudaSuccess) return e;
-      if (per_sm <= 0) return cudaErrorInvalidConfiguration;
-      max_blocks[dev] = per_sm * sm_count();
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(max_blocks[dev], 1, 1);
-    cfg.blockDim = dim3(PG::THREADS, 1, 1);
-    cfg.dynamicSmemBytes = PG::SMEM;
-    cfg.stream = st;
-    CUtensorMap tmap;
-    memset(&tmap, 0, sizeof(tmap));
-    return cudaLaunchKernelEx(&cfg, kern, a, 0, a.err, tmap);
-  }
-}
-
-template <typename T>
-cudaError_t launch_line_pass_tick(const LinePassArgs<T>& a, cudaStream_t st) {
-  if constexpr (sizeof(T) == 4) {
-    switch (a.L) {
-      case 256: return launch_persist_tick<256>(a, st);
-      case 512: return launch_persist_tick<512>(a, st);
-      case 1024: return launch_persist_tick<1024>(a, st);
-      case 2048: return launch_persist_tick<2048>(a, st);
-      default: break;
-    }
-  }
-  return cudaErrorInvalidValue;
 }
 
 template <typename T>

@@ -57,29 +57,23 @@ struct LinePassArgs {
   int sigma;            // 0: sigma_x (x pass), 1: sigma_y (y pass)
   const Cx<T>* tw;      // per-pass twiddles, see tw_offset (at most L entries)
   const Cx<T>* tw_alt;  // the same for the alternative radix schedule (or nullptr)
+  const Cx<T>* tw_team;  // twiddles of the radix-16 team pass (launch_team_twiddles), or nullptr
   const Q4<T>* mult;    // per k index q: step ((cos - 1) hi, lo, sin hi, lo) / (2L);
                         // derivative (0, 0, xi hi, xi lo) / L
-  const Q4<T>* mult_perm;  // 1024-point lines: the step table with entry q at perm1024(q),
-                           // read by the 1024-point persistent pass; or nullptr
+  const Q4<T>* mult_perm;  // complex64 lines of 256 points or more: the step table with entry
+                           // q at team_perm(L, q), read by the team pass; or nullptr
   const T* beta;        // b - 1 per input point, or nullptr (b = 1)
   const T* beta_im;     // imaginary part of b - 1 (complex stretching), or nullptr
   const Q4<T>* u_load;  // U applied to psi when it is read, or nullptr
   const Q4<T>* u_store; // U applied to psi_new before the store, or nullptr
-  int* err;             // device error flag (persistent variant: bounded-wait timeouts)
+  int* err;             // device error flag (team pass: bounded-wait timeouts)
   const InstPtrs<T>* inst;  // batched launch: per-instance pointers (overrides the above)
   const int* n_inst;        // batched launch: number of active instances (device memory)
   int inst_capacity;        // batched launch: table entries (host side, sizes the grid)
   unsigned test_extra_tx;   // test hook: bytes a bulk copy never delivers (0 normally);
-                            // makes the persistent pass's bounded wait run out
+                            // makes the team pass's bounded wait run out
   int store_normal;         // 0 = out is [L][n_lines] (transposed store), 1 = out is
                             // [n_lines][L] like `in` (out must not alias in)
-  // Batched tick launch (the persistent pass runs every step of a tick in one launch):
-  // inst is then the tick's table [tick_k steps][2 passes][inst_capacity], n_inst the
-  // active count per step; work items are taken from *tick_queue (zero at launch) and
-  // tick_done[i] counts the finished line groups of instance slot i (zero at launch).
-  int tick_k;
-  int* tick_queue;
-  int* tick_done;
 };
 
 // Batched launches: a block (or group) of lines belongs to instance `k`; take that
@@ -426,6 +420,8 @@ __global__ void __launch_bounds__(Geo<T, L, LPC, E>::THREADS,
   constexpr int J = Gm::J;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cx<T>* smem = reinterpret_cast<Cx<T>*>(smem_raw);
+  pdl_wait();
+  pdl_launch_next();
 
   // batched launch: blocks of one instance are consecutive (whole clusters), and blocks
   // past the active instances leave at once (together with their cluster)

@@ -5,7 +5,6 @@ namespace dgb {
 template cudaError_t launch_line_pass<float>(const LinePassArgs<float>&, int, int, cudaStream_t);
 template int line_pass_radix<float>(int);
 template int line_pass_radix_alt<float>(int);
-template cudaError_t launch_line_pass_tick<float>(const LinePassArgs<float>&, cudaStream_t);
 
 // Debug builds: reads and clears this translation unit's index-check flag (0 otherwise).
 int dgb_debug_flag_c64() {

@@ -349,27 +349,52 @@ cudaError_t launch_step_mult(int n, double a, double dt, Q4<T>* mult, cudaStream
   return cudaGetLastError();
 }
 
-constexpr bool perm1024_is_a_permutation() {
-  bool seen[1024] = {};
-  for (int k = 0; k < 1024; ++k) {
-    const int p = perm1024(k);
-    if (p < 0 || p >= 1024 || seen[p]) return false;
+constexpr bool team_perm_is_a_permutation(int L) {
+  bool seen[4096] = {};
+  for (int k = 0; k < L; ++k) {
+    const int p = team_perm(L, k);
+    if (p < 0 || p >= L || seen[p]) return false;
     seen[p] = true;
   }
   return true;
 }
-static_assert(perm1024_is_a_permutation(), "perm1024 must map 0..1023 onto itself");
+static_assert(team_perm_is_a_permutation(256) && team_perm_is_a_permutation(512) &&
+                  team_perm_is_a_permutation(1024) && team_perm_is_a_permutation(2048) &&
+                  team_perm_is_a_permutation(4096),
+              "team_perm must map 0..L-1 onto itself");
 
-// dst[perm1024(q)] = src[q] for the 1024 entries of a 1024-point step table
+// dst[team_perm(n, q)] = src[q] for the n entries of a multiplier table
 template <typename T>
-__global__ void k_perm1024(const Q4<T>* __restrict__ src, Q4<T>* __restrict__ dst) {
+__global__ void k_team_perm(int n, const Q4<T>* __restrict__ src, Q4<T>* __restrict__ dst) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
-  if (q < 1024) dst[perm1024(q)] = src[q];
+  if (q < n) dst[team_perm(n, q)] = src[q];
 }
 
 template <typename T>
-cudaError_t launch_perm1024(const Q4<T>* src, Q4<T>* dst, cudaStream_t st) {
-  k_perm1024<T><<<nblocks(1024), TPB, 0, st>>>(src, dst);
+cudaError_t launch_team_perm(int n, const Q4<T>* src, Q4<T>* dst, cudaStream_t st) {
+  k_team_perm<T><<<nblocks(n), TPB, 0, st>>>(n, src, dst);
+  return cudaGetLastError();
+}
+
+// Twiddles of the team pass for n-point lines, T = n/16, R2 = n/256: entry (k - 1) T + j =
+// exp(-2 pi i k j / n) (k = 1..15, j < T), then at 15 T the entries (k - 1) R2 + u =
+// exp(-2 pi i k u / T) (u < R2). Computed in FP64; at most n entries.
+template <typename T>
+__global__ void k_team_twiddles(int n, Cx<T>* tw) {
+  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  const int t = n / 16, r2 = n / 256;
+  if (m >= 15 * (t + r2)) return;
+  double frac;
+  if (m < 15 * t) frac = (double)((m / t + 1) * (m % t)) / n;
+  else frac = (double)(((m - 15 * t) / r2 + 1) * ((m - 15 * t) % r2)) / t;
+  double s, c;
+  sincospi(-2.0 * frac, &s, &c);
+  tw[m] = {(T)c, (T)s};
+}
+
+template <typename T>
+cudaError_t launch_team_twiddles(int n, Cx<T>* tw, cudaStream_t st) {
+  k_team_twiddles<T><<<nblocks(n), TPB, 0, st>>>(n, tw);
   return cudaGetLastError();
 }
 
@@ -426,7 +451,8 @@ cudaError_t launch_transpose(const Q4<T>* in, Q4<T>* out, int rows, int cols, cu
       cudaStream_t);                                                                         \
   template cudaError_t launch_twiddles<T>(int, int, Cx<T>*, cudaStream_t);                    \
   template cudaError_t launch_step_mult<T>(int, double, double, Q4<T>*, cudaStream_t);        \
-  template cudaError_t launch_perm1024<T>(const Q4<T>*, Q4<T>*, cudaStream_t);                \
+  template cudaError_t launch_team_perm<T>(int, const Q4<T>*, Q4<T>*, cudaStream_t);          \
+  template cudaError_t launch_team_twiddles<T>(int, Cx<T>*, cudaStream_t);                    \
   template cudaError_t launch_deriv_mult<T>(int, double, Q4<T>*, cudaStream_t);               \
   template cudaError_t launch_transpose<T>(const Q4<T>*, Q4<T>*, int, int, cudaStream_t);
 INST(float)
