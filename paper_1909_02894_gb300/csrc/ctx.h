@@ -7,6 +7,9 @@
 
 #include "../../include/dirac.h"
 
+// inner products of one Arnoldi step: 4 per basis vector (at most 100), norms
+constexpr size_t kKrylovHost = 1024;
+
 struct dirac_ctx {
   int nx = 0, ny = 0;
   double ax = 0, ay = 0, mass = 0, c = 1;
@@ -54,9 +57,13 @@ struct dirac_ctx {
   void** k_vptr = nullptr;          // device copy of the basis pointers
   double* k_partials = nullptr;     // inner-product partial sums
   double* k_coef = nullptr;         // combination coefficients (device)
+  double* k_dots = nullptr;         // inner products (device), kKrylovHost values
+  unsigned* k_ticket = nullptr;     // counter of the inner products' last block
+  double* k_host = nullptr;         // pinned: inner products (first half), coefficients (second)
   // complex64 axes of 256 points or more: the step tables (x at dt and dt/2, y) in the
   // order of team_perm, for the team pass
   void *mult_px = nullptr, *mult_py = nullptr, *mult_pxh = nullptr;
+  void *dmult_px = nullptr, *dmult_py = nullptr;  // derivative tables in that order
   void *mult_xh = nullptr, *u2_n = nullptr;  // symmetric order: x multipliers at dt/2,
                                              // U^2 in the normal layout
   int* d_err = nullptr;       // device error flag written by bounded waits

@@ -70,6 +70,8 @@ static cudaError_t dalloc(dirac_ctx* ctx, void** p, size_t bytes) {
 }
 
 static void free_all(dirac_ctx* ctx) {
+  if (ctx->k_host) cudaFreeHost(ctx->k_host);
+  ctx->k_host = nullptr;
   for (void* p : ctx->allocs) cudaFree(p);
   ctx->allocs.clear();
 }
@@ -253,29 +255,89 @@ static dirac_status step_symmetric(dirac_ctx* ctx, long n) {
   return DIRAC_OK;
 }
 
-// out = alpha S(in) + beta prev, acc += gamma out, with S(in) = sum_j b^j sigma_j [[d_j]] in
-// (so dt A = -dt S): x derivative (row pass, rows back in place), transpose, y derivative
-// (transposed store back to rows), pointwise combine. psiT, scratch1, scratch2 are scratch.
+// One application of the unsplit operator, S(v) = sum_j b^j sigma_j [[d_j]] v (so dt A = -dt S):
+//   out = (ar + i ai) S(in) + (gr + i gi) base + beta prev, then U out if u is not null.
+// `in` is in the normal (tr = false) or the transposed layout; out_rows: the result stays in
+// the layout of the second pass' rows, the other one than `in`'s; otherwise it returns to the
+// layout of `in`. base, prev and u are in the layout of the rows; in_t receives `in` in that
+// layout (base may be in_t).
+struct UnsplitOp {
+  const void* in = nullptr;
+  bool tr = false;
+  void* in_t = nullptr;
+  void* out = nullptr;
+  bool out_rows = false;
+  double ar = 0.0, ai = 0.0;
+  const void* base = nullptr;
+  double gr = 0.0, gi = 0.0;
+  const void* prev = nullptr;
+  double beta = 0.0;
+  const void* u = nullptr;
+};
+
+// complex64 grids whose axes both have team-pass lengths run the operator as two team passes,
+// with the result in either layout; the others as two derivative passes, a transpose and a
+// pointwise combine, everything in the normal layout.
+static bool unsplit_team(const dirac_ctx* ctx) {
+  return ctx->prec == DIRAC_C64 && ctx->dmult_px && ctx->dmult_py && !ctx->beta1_im;
+}
+
+// in -> out through two team passes; scratch1 holds the first axis' term.
+static dirac_status unsplit_apply_team(dirac_ctx* ctx, const UnsplitOp& op) {
+  cudaStream_t st = ctx->stream;
+  for (int phase = 1; phase <= 2; ++phase) {
+    UnsplitArgs a{};
+    a.axis = (phase == 1) == op.tr ? 1 : 0;  // phase 1 runs along the rows of `in`
+    a.n_lines = a.axis == 0 ? ctx->ny : ctx->nx;
+    a.beta = (const float*)(a.axis == 0 ? ctx->beta1 : ctx->beta2T);
+    a.tw = (const Cx<float>*)(a.axis == 0 ? ctx->tw_x_team : ctx->tw_y_team);
+    a.mult = (const Q4<float>*)(a.axis == 0 ? ctx->dmult_px : ctx->dmult_py);
+    a.err = ctx->d_err;
+    if (phase == 1) {
+      a.in = (const Q4<float>*)op.in;
+      a.out = (Q4<float>*)ctx->scratch1;
+      a.out_in = (Q4<float>*)op.in_t;
+    } else {
+      a.in = (const Q4<float>*)op.in_t;
+      a.out = (Q4<float>*)op.out;
+      a.s_other = (const Q4<float>*)ctx->scratch1;
+      a.ar = (float)op.ar;
+      a.ai = (float)op.ai;
+      a.base = (const Q4<float>*)op.base;
+      a.gr = (float)op.gr;
+      a.gi = (float)op.gi;
+      a.prev = (const Q4<float>*)op.prev;
+      a.beta_prev = (float)op.beta;
+      a.u_store = (const Q4<float>*)op.u;
+      a.store_normal = op.out_rows ? 1 : 0;
+    }
+    CK(launch_unsplit(a, a.axis == 0 ? ctx->nx : ctx->ny, phase, st), "unsplit operator");
+  }
+  ctx->launches += 2;
+  return DIRAC_OK;
+}
+
+// The general path: normal layout throughout (op.tr, op.in_t, op.out_rows and op.u unused, base
+// and prev in the normal layout). psiT, scratch1 and scratch2 are scratch.
 template <typename T>
-static dirac_status unsplit_apply(dirac_ctx* ctx, const void* in, void* out, double ar,
-                                  double ai, const void* prev, double beta, double gr,
-                                  double gi, void* acc) {
+static dirac_status unsplit_apply(dirac_ctx* ctx, const UnsplitOp& op) {
   cudaStream_t st = ctx->stream;
   LinePassArgs<T> ax = pass_args<T>(ctx, 0), ay = pass_args<T>(ctx, 1);
-  ax.in = (const Q4<T>*)in;
+  ax.in = (const Q4<T>*)op.in;
   ax.out = (Q4<T>*)ctx->scratch1;
   ax.mult = (const Q4<T>*)ctx->dmult_x;
   ax.store_normal = 1;
   CK(launch_line_pass<T>(ax, MODE_DERIV, 0, st), "x derivative");
-  CK(launch_transpose<T>((const Q4<T>*)in, (Q4<T>*)ctx->psiT, ctx->ny, ctx->nx, st), "transpose");
+  CK(launch_transpose<T>((const Q4<T>*)op.in, (Q4<T>*)ctx->psiT, ctx->ny, ctx->nx, st),
+     "transpose");
   ay.in = (const Q4<T>*)ctx->psiT;
   ay.out = (Q4<T>*)ctx->scratch2;
   ay.mult = (const Q4<T>*)ctx->dmult_y;
   CK(launch_line_pass<T>(ay, MODE_DERIV, 0, st), "y derivative");
   CK(launch_unsplit_combine<T>((const Q4<T>*)ctx->scratch1, (const Q4<T>*)ctx->scratch2, ctx->a1,
                                ctx->a2, ctx->sxinv, ctx->syinv, ctx->sxinv_im, ctx->syinv_im,
-                               ctx->nx, ctx->ny, ar, ai,
-                               (const Q4<T>*)prev, beta, gr, gi, (Q4<T>*)out, (Q4<T>*)acc, st),
+                               ctx->nx, ctx->ny, op.ar, op.ai, (const Q4<T>*)op.base, op.gr,
+                               op.gi, (const Q4<T>*)op.prev, op.beta, (Q4<T>*)op.out, st),
      "combine");
   ctx->launches += 4;
   return DIRAC_OK;
@@ -288,8 +350,12 @@ static dirac_status unsplit_apply(dirac_ctx* ctx, const void* in, void* out, dou
   } while (0)
 
 // The polynomial scheme (eq. poly): U, the middle step, U per step, with U^2 between
-// consecutive steps of a call. Four state-sized buffers (the state and pool[0..2]) rotate:
-// the middle step's sum becomes the new state.
+// consecutive steps of a call. The middle step's sum is evaluated from its highest term down,
+// so that no separate sum is kept: Taylor by Horner's rule, t <- psi + (dt/q) A t for q = N..1;
+// Chebyshev by Clenshaw's recurrence, b_k = c_k psi + 2 B b_{k+1} - b_{k+2}, the sum being
+// c_0 psi + B b_1 - b_2, with B = (i dt / R) A = -(i dt / R) S, c_k = (2 - delta_k0) (-i)^k
+// J_k(R) and b_N = c_N psi (folded into the factors of the first two applications). The team
+// passes alternate the layout of the terms; b_{k+2} is then always in the layout of b_k.
 template <typename T>
 static dirac_status step_poly(dirac_ctx* ctx, long n, double dt) {
   cudaStream_t st = ctx->stream;
@@ -326,94 +392,152 @@ static dirac_status step_poly(dirac_ctx* ctx, long n, double dt) {
     if (!(R > 0.0) || !bessel_j_series(R, N, jq.data()))
       return fail(ctx, DIRAC_EINVAL, "no Chebyshev bound for this grid and dt");
   }
+  using cd = std::complex<double>;
+  auto c_of = [&](int k) {  // (2 - delta_k0) (-i)^k J_k
+    static const double pr[4] = {1.0, 0.0, -1.0, 0.0}, pi_[4] = {0.0, -1.0, 0.0, 1.0};
+    return (k == 0 ? 1.0 : 2.0) * jq[k] * cd(pr[k & 3], pi_[k & 3]);
+  };
+  const bool team = unsplit_team(ctx);
   for (long s = 0; s < n; ++s) {
     if (s == 0) CKS(apply_half<T>(ctx, ctx->psi, false));
-    void* bufs[4] = {ctx->psi, ctx->pool[0], ctx->pool[1], ctx->pool[2]};
-    void* acc = bufs[3];
-    if (!cheb) {
-      // acc = sum_q (dt A)^q / q! psi; (dt/q) A t = -(dt/q) S(t)
-      CK(cudaMemcpyAsync(acc, bufs[0], bytes, cudaMemcpyDeviceToDevice, st), "copy");
-      void *cur = bufs[0], *nxt = bufs[1], *spare = bufs[2];
-      for (int q = 1; q <= N; ++q) {
-        CKS(unsplit_apply<T>(ctx, cur, nxt, -dt / q, 0.0, nullptr, 0.0, 1.0, 0.0, acc));
-        cur = nxt;
-        nxt = (cur == bufs[1]) ? spare : bufs[1];
+    const bool last_step = s + 1 == n;
+    // U after the middle step, inside the last application where it can be
+    const bool fuse_u = team && !ctx->has_pot && !ctx->u_identity;
+    const void *cur = ctx->psi, *prev = nullptr;  // b_{k+1}, b_{k+2}
+    for (int i = 1; i <= N; ++i) {  // application i makes term k = N - i
+      const int k = N - i;
+      UnsplitOp op;
+      op.in = cur;
+      op.tr = team && i % 2 == 0;
+      cd al, ga;
+      if (!cheb) {
+        al = -dt / (k + 1);
+        ga = 1.0;
+      } else {
+        al = cd(0.0, -dt / R) * (k == 0 ? 1.0 : 2.0);
+        ga = c_of(k);
+        if (i == 1) al *= c_of(N);
+        if (i == 2) ga -= c_of(N);
+        if (i >= 3) {
+          op.prev = prev;
+          op.beta = -1.0;
+        }
       }
-    } else {
-      // phi_0 = psi, phi_1 = B phi_0, phi_{q+1} = 2 B phi_q - phi_{q-1} with
-      // B = (i dt / R) A = -(i dt / R) S; acc = sum_q (2 - delta_q0) (-i)^q J_q(R) phi_q
-      CK(launch_scale<T>((Q4<T>*)acc, (const Q4<T>*)bufs[0], jq[0], 0.0, np, st), "scale");
-      ctx->launches += 1;
-      static const double pr[4] = {1.0, 0.0, -1.0, 0.0}, pi_[4] = {0.0, -1.0, 0.0, 1.0};
-      void *prev = bufs[0], *cur = bufs[1], *spare = bufs[2];
-      if (N >= 1)
-        CKS(unsplit_apply<T>(ctx, prev, cur, 0.0, -dt / R, nullptr, 0.0, 2.0 * pr[1] * jq[1],
-                             2.0 * pi_[1] * jq[1], acc));
-      for (int q = 2; q <= N; ++q) {
-        CKS(unsplit_apply<T>(ctx, cur, spare, 0.0, -2.0 * dt / R, prev, -1.0,
-                             2.0 * pr[q & 3] * jq[q], 2.0 * pi_[q & 3] * jq[q], acc));
-        void* t = prev;
-        prev = cur;
-        cur = spare;
-        spare = t;
+      op.ar = al.real();
+      op.ai = al.imag();
+      op.gr = ga.real();
+      op.gi = ga.imag();
+      int slot = 0;  // a buffer that holds neither b_{k+1} nor b_{k+2}
+      while (ctx->pool[slot] == cur || ctx->pool[slot] == prev) ++slot;
+      op.out = ctx->pool[slot];
+      if (team) {
+        const bool rows_tr = !op.tr;  // the second pass' rows are in the transposed layout
+        op.in_t = i == 1 ? ctx->psiT : ctx->scratch2;
+        op.base = rows_tr ? ctx->psiT : ctx->psi;
+        op.out_rows = !(i == N && rows_tr);  // the sum ends in the normal layout
+        if (i == N && fuse_u)
+          op.u = rows_tr ? (last_step ? ctx->u_t : ctx->u2_t) : (last_step ? ctx->u_n : ctx->u2_n);
+        CKS(unsplit_apply_team(ctx, op));
+      } else {
+        op.base = ctx->psi;
+        CKS(unsplit_apply<T>(ctx, op));
       }
+      prev = cur;
+      cur = op.out;
+      if (i == 1) prev = nullptr;  // b_N is never stored
     }
-    // the sum is the new state; the other three buffers become the pool
-    int k = 0;
-    for (void* b : bufs)
-      if (b != acc) ctx->pool[k++] = b;
-    ctx->psi = acc;
-    CKS(apply_half<T>(ctx, ctx->psi, s + 1 < n));
+    // the sum is the new state; the old state's buffer joins the pool
+    for (void*& p : ctx->pool)
+      if (p == cur) {
+        p = ctx->psi;
+        break;
+      }
+    ctx->psi = (void*)cur;
+    if (!fuse_u) CKS(apply_half<T>(ctx, ctx->psi, !last_step));
   }
   return DIRAC_OK;
 }
 
 // ---- Scheme I (eq. cn): U, G psi* = G~ psi by restarted GMRES, U (U^2 between steps).
 // G v = v - dt/2 A v = v + dt/2 S(v), G~ v = v - dt/2 S(v) (S as in unsplit_apply).
-constexpr int kKrylovBlocks = 304;
+constexpr int kKrylovBlocks = 608;
 
-// <V_i, w> for i < count, V = the device pointer array starting at slot first.
+// out = v + a S(v), normal layout
 template <typename T>
-static dirac_status krylov_dots(dirac_ctx* ctx, int first, int count, const void* w,
-                                std::vector<std::complex<double>>& out) {
-  cudaStream_t st = ctx->stream;
-  CK(launch_multi_dot<T>((const Q4<T>* const*)(ctx->k_vptr + first), count, (const Q4<T>*)w,
-                         npts(ctx), ctx->k_partials, kKrylovBlocks, st),
-     "inner products");
-  std::vector<double> h(2 * (size_t)kKrylovBlocks * count);
-  CK(cudaMemcpyAsync(h.data(), ctx->k_partials, h.size() * sizeof(double),
-                     cudaMemcpyDeviceToHost, st),
-     "inner products");
-  CK(cudaStreamSynchronize(st), "inner products");
-  out.assign(count, 0.0);
-  for (int i = 0; i < count; ++i) {
-    double re = 0.0, im = 0.0;
-    for (int b = 0; b < kKrylovBlocks; ++b) {
-      re += h[2 * ((size_t)i * kKrylovBlocks + b)];
-      im += h[2 * ((size_t)i * kKrylovBlocks + b) + 1];
-    }
-    out[i] = {re, im};
+static dirac_status cn_apply(dirac_ctx* ctx, const void* v, void* out, double a) {
+  UnsplitOp op;
+  op.in = v;
+  op.out = out;
+  op.ar = a;
+  op.gr = 1.0;
+  op.in_t = ctx->psiT;
+  if (unsplit_team(ctx)) {
+    op.base = ctx->psiT;  // the transposed copy of v
+    return unsplit_apply_team(ctx, op);
   }
-  ctx->launches += 1;
+  op.base = v;
+  return unsplit_apply<T>(ctx, op);
+}
+
+// Copies `count` doubles of the device's dot products to the pinned host buffer and waits.
+static dirac_status krylov_fetch(dirac_ctx* ctx, size_t count) {
+  CK(cudaMemcpyAsync(ctx->k_host, ctx->k_dots, count * sizeof(double), cudaMemcpyDeviceToHost,
+                     ctx->stream),
+     "inner products");
+  CK(cudaStreamSynchronize(ctx->stream), "inner products");
   return DIRAC_OK;
 }
 
-// out += sum_i c_i V_{first + i}
+// out += sum_{i < c.size()} c_i V_i
 template <typename T>
-static dirac_status krylov_combine(dirac_ctx* ctx, void* out, int first,
+static dirac_status krylov_combine(dirac_ctx* ctx, void* out,
                                    const std::vector<std::complex<double>>& c) {
-  std::vector<double> h(2 * c.size());
+  double* h = ctx->k_host + kKrylovHost / 2;  // not read by the device at this point
   for (size_t i = 0; i < c.size(); ++i) {
     h[2 * i] = c[i].real();
     h[2 * i + 1] = c[i].imag();
   }
-  CK(cudaMemcpyAsync(ctx->k_coef, h.data(), h.size() * sizeof(double), cudaMemcpyHostToDevice,
+  CK(cudaMemcpyAsync(ctx->k_coef, h, 2 * c.size() * sizeof(double), cudaMemcpyHostToDevice,
                      ctx->stream),
      "coefficients");
-  CK(launch_multi_axpy<T>((Q4<T>*)out, (const Q4<T>* const*)(ctx->k_vptr + first), ctx->k_coef,
+  CK(launch_multi_axpy<T>((Q4<T>*)out, (const Q4<T>* const*)ctx->k_vptr, ctx->k_coef,
                           (int)c.size(), npts(ctx), ctx->stream),
      "combination");
   ctx->launches += 1;
+  return DIRAC_OK;
+}
+
+// One Arnoldi step after w = G V_j is in kv[j + 1]: classical Gram-Schmidt twice against V_0..V_j
+// and the norm, everything on the device. dots: h (2 m values), second h (2 m), norm^2, 1/norm.
+template <typename T>
+static dirac_status krylov_orthogonalise(dirac_ctx* ctx, int m) {
+  cudaStream_t st = ctx->stream;
+  const size_t np = npts(ctx);
+  const auto V = (const Q4<T>* const*)ctx->k_vptr;
+  Q4<T>* w = (Q4<T>*)ctx->kv[m];
+  double *d0 = ctx->k_dots, *d1 = d0 + 2 * m, *d2 = d1 + 2 * m;
+  CK(launch_gram_schmidt<T>(0, V, m, w, nullptr, np, ctx->k_partials, ctx->k_ticket, d0,
+                            kKrylovBlocks, st),
+     "inner products");
+  if (m <= 4) {
+    // the first combination and the second products in one sweep
+    CK(launch_gram_schmidt<T>(1, V, m, w, d0, np, ctx->k_partials, ctx->k_ticket, d1,
+                              kKrylovBlocks, st),
+       "inner products");
+  } else {
+    CK(launch_gram_schmidt<T>(2, V, m, w, d0, np, ctx->k_partials, ctx->k_ticket, d2,
+                              kKrylovBlocks, st),
+       "combination");
+    CK(launch_gram_schmidt<T>(0, V, m, w, nullptr, np, ctx->k_partials, ctx->k_ticket, d1,
+                              kKrylovBlocks, st),
+       "inner products");
+    ctx->launches += 1;
+  }
+  CK(launch_gram_schmidt<T>(2, V, m, w, d1, np, ctx->k_partials, ctx->k_ticket, d2, kKrylovBlocks,
+                            st),
+     "combination");
+  CK(launch_normalise<T>(w, d2 + 1, np, st), "normalise");
+  ctx->launches += 4;
   return DIRAC_OK;
 }
 
@@ -423,7 +547,7 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
   const size_t np = npts(ctx), bytes = np * sizeof(Q4<T>);
   const int m = ctx->krylov_m;
   const double tol = ctx->krylov_tol > 0.0 ? ctx->krylov_tol : (sizeof(T) == 8 ? 1e-14 : 3e-7);
-  // buffers: basis V_0..V_m, the right-hand side, the pointer table (basis, then rhs)
+  // buffers: basis V_0..V_m, the right-hand side, the pointer table of the basis
   while ((int)ctx->kv.size() < m + 1) {
     void* p = nullptr;
     CK(dalloc(ctx, &p, bytes), "allocate Krylov basis");
@@ -436,60 +560,55 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
     CK(dalloc(ctx, (void**)&ctx->k_partials, 2 * (size_t)kKrylovBlocks * 102 * sizeof(double)),
        "scratch");
   if (!ctx->k_coef) CK(dalloc(ctx, (void**)&ctx->k_coef, 2 * 102 * sizeof(double)), "scratch");
+  if (!ctx->k_dots) CK(dalloc(ctx, (void**)&ctx->k_dots, kKrylovHost * sizeof(double)), "scratch");
   if (!ctx->k_vptr) CK(dalloc(ctx, (void**)&ctx->k_vptr, 102 * sizeof(void*)), "scratch");
-  {
-    std::vector<void*> table(ctx->kv.begin(), ctx->kv.begin() + m + 1);
-    table.push_back(ctx->k_rhs);
-    CK(cudaMemcpy(ctx->k_vptr, table.data(), table.size() * sizeof(void*), cudaMemcpyHostToDevice),
-       "pointer table");
+  if (!ctx->k_host)
+    CK(cudaMallocHost((void**)&ctx->k_host, kKrylovHost * sizeof(double)), "scratch");
+  if (!ctx->k_ticket) {
+    CK(dalloc(ctx, (void**)&ctx->k_ticket, sizeof(unsigned)), "scratch");
+    CK(cudaMemsetAsync(ctx->k_ticket, 0, sizeof(unsigned), st), "scratch");
   }
+  CK(cudaMemcpyAsync(ctx->k_vptr, ctx->kv.data(), (m + 1) * sizeof(void*), cudaMemcpyHostToDevice,
+                     st),
+     "pointer table");
   using cd = std::complex<double>;
-  std::vector<cd> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m), h, h2;
+  std::vector<cd> H((size_t)(m + 1) * m), cs(m), sn(m), g(m + 1), y(m);
   for (long s = 0; s < n; ++s) {
     if (s == 0) CKS(apply_half<T>(ctx, ctx->psi, false));
     void* x = ctx->psi;
-    CKS(unsplit_apply<T>(ctx, x, ctx->k_rhs, -0.5 * dt, 0.0, x, 1.0, 0.0, 0.0, nullptr));
-    CKS(krylov_dots<T>(ctx, m + 1, 1, ctx->k_rhs, h));
-    const double bnorm = sqrt(h[0].real());
+    CKS(cn_apply<T>(ctx, x, ctx->k_rhs, -0.5 * dt));
+    double bnorm = 0.0;
     bool converged = false;
     for (int cycle = 0; cycle <= ctx->krylov_restarts && !converged; ++cycle) {
-      // r = rhs - G x into V_0
+      // r = rhs - G x into V_0; for the initial guess psi, G~ psi - G psi = 2 (rhs - psi)
       void* v0 = ctx->kv[0];
-      CKS(unsplit_apply<T>(ctx, x, v0, 0.5 * dt, 0.0, x, 1.0, 0.0, 0.0, nullptr));
-      CK(launch_axpby<T>((Q4<T>*)v0, 1.0, (const Q4<T>*)ctx->k_rhs, -1.0, (const Q4<T>*)v0, np, st),
+      if (cycle > 0) CKS(cn_apply<T>(ctx, x, v0, 0.5 * dt));
+      CK(launch_residual<T>(cycle > 0 ? 1 : 0, (const Q4<T>*)ctx->k_rhs, (const Q4<T>*)x,
+                            (Q4<T>*)v0, np, ctx->k_partials, ctx->k_ticket, ctx->k_dots,
+                            kKrylovBlocks, st),
          "residual");
-      CKS(krylov_dots<T>(ctx, 0, 1, v0, h));
-      const double beta = sqrt(fmax(h[0].real(), 0.0));
+      CK(launch_normalise<T>((Q4<T>*)v0, ctx->k_dots + 2, np, st), "normalise");
+      ctx->launches += 2;
+      CKS(krylov_fetch(ctx, 2));
+      const double beta = sqrt(fmax(ctx->k_host[0], 0.0));
+      if (cycle == 0) bnorm = sqrt(ctx->k_host[1]);
       if (beta <= tol * bnorm || beta == 0.0) {
         converged = true;
         break;
       }
       if (cycle == ctx->krylov_restarts) break;
-      CK(launch_scale<T>((Q4<T>*)v0, (const Q4<T>*)v0, 1.0 / beta, 0.0, np, st), "normalise");
       std::fill(g.begin(), g.end(), cd(0.0));
       g[0] = beta;
       int kdim = 0;
       for (int j = 0; j < m; ++j) {
-        void* w = ctx->kv[j + 1];
-        CKS(unsplit_apply<T>(ctx, ctx->kv[j], w, 0.5 * dt, 0.0, ctx->kv[j], 1.0, 0.0, 0.0,
-                             nullptr));
-        // classical Gram-Schmidt, twice
-        CKS(krylov_dots<T>(ctx, 0, j + 1, w, h));
-        std::vector<cd> neg(j + 1);
-        for (int i = 0; i <= j; ++i) neg[i] = -h[i];
-        CKS(krylov_combine<T>(ctx, w, 0, neg));
-        CKS(krylov_dots<T>(ctx, 0, j + 1, w, h2));
-        for (int i = 0; i <= j; ++i) {
-          neg[i] = -h2[i];
-          h[i] += h2[i];
-        }
-        CKS(krylov_combine<T>(ctx, w, 0, neg));
-        std::vector<cd> nn;
-        CKS(krylov_dots<T>(ctx, j + 1, 1, w, nn));
-        const double hn = sqrt(fmax(nn[0].real(), 0.0));
-        if (hn > 0.0)
-          CK(launch_scale<T>((Q4<T>*)w, (const Q4<T>*)w, 1.0 / hn, 0.0, np, st), "normalise");
-        for (int i = 0; i <= j; ++i) H[(size_t)i * m + j] = h[i];
+        CKS(cn_apply<T>(ctx, ctx->kv[j], ctx->kv[j + 1], 0.5 * dt));
+        CKS(krylov_orthogonalise<T>(ctx, j + 1));
+        CKS(krylov_fetch(ctx, 4 * (size_t)(j + 1) + 1));
+        const double* d = ctx->k_host;
+        for (int i = 0; i <= j; ++i)
+          H[(size_t)i * m + j] = cd(d[2 * i], d[2 * i + 1]) +
+                                 cd(d[2 * (j + 1) + 2 * i], d[2 * (j + 1) + 2 * i + 1]);
+        const double hn = sqrt(fmax(d[4 * (j + 1)], 0.0));
         H[(size_t)(j + 1) * m + j] = hn;
         for (int i = 0; i < j; ++i) {  // earlier Givens rotations on column j
           const cd a = H[(size_t)i * m + j], b = H[(size_t)(i + 1) * m + j];
@@ -513,8 +632,7 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
         for (int t = i + 1; t < kdim; ++t) acc -= H[(size_t)i * m + t] * y[t];
         y[i] = acc / H[(size_t)i * m + i];
       }
-      CKS(krylov_combine<T>(ctx, x, 0, std::vector<cd>(y.begin(), y.begin() + kdim)));
-      ctx->launches += 3;
+      CKS(krylov_combine<T>(ctx, x, std::vector<cd>(y.begin(), y.begin() + kdim)));
     }
     if (!converged) return fail(ctx, DIRAC_ENOCONV, "Scheme I: GMRES did not converge");
     CKS(apply_half<T>(ctx, ctx->psi, s + 1 < n));
@@ -677,6 +795,10 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
     CK(dalloc(ctx, &ctx->mult_py, ny * sizeof(Q4<T>)), "allocate tables");
     CK(dalloc(ctx, &ctx->tw_y_team, ny * sizeof(Cx<T>)), "allocate tables");
   }
+  if (ctx->tw_x_team)
+    CK(dalloc(ctx, &ctx->dmult_px, nx * sizeof(Q4<T>)), "allocate tables");
+  if (ctx->tw_y_team)
+    CK(dalloc(ctx, &ctx->dmult_py, ny * sizeof(Q4<T>)), "allocate tables");
   CK(dalloc(ctx, &ctx->dmult_x, nx * sizeof(Q4<T>)), "allocate tables");
   CK(dalloc(ctx, &ctx->dmult_y, ny * sizeof(Q4<T>)), "allocate tables");
   CK(dalloc(ctx, (void**)&ctx->staging, 2 * n * 2 * sizeof(double)), "allocate staging");
@@ -760,6 +882,12 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
     CK(launch_team_twiddles<T>(ny, (Cx<T>*)ctx->tw_y_team, st), "twiddles");
   CK(launch_deriv_mult<T>(nx, ctx->ax, (Q4<T>*)ctx->dmult_x, st), "derivative table");
   CK(launch_deriv_mult<T>(ny, ctx->ay, (Q4<T>*)ctx->dmult_y, st), "derivative table");
+  if (ctx->dmult_px)
+    CK(launch_team_perm<T>(nx, (const Q4<T>*)ctx->dmult_x, (Q4<T>*)ctx->dmult_px, st),
+       "multiplier order");
+  if (ctx->dmult_py)
+    CK(launch_team_perm<T>(ny, (const Q4<T>*)ctx->dmult_y, (Q4<T>*)ctx->dmult_py, st),
+       "multiplier order");
   ctx->launches += 7;
   CK(cudaStreamSynchronize(st), "create");
   ctx->dt_cached = 0.0;

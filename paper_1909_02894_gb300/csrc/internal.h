@@ -115,19 +115,22 @@ cudaError_t launch_halfstep_general(const double* a1, const double* a2, const do
 template <typename T>
 cudaError_t launch_apply_ug(Q4<T>* psi, const Q4<T>* ug, size_t n, cudaStream_t st);
 
+// One phase (1 or 2) of the unsplit operator on complex64 rows of L = 256..4096 points.
+cudaError_t launch_unsplit(const UnsplitArgs& a, int L, int phase, cudaStream_t st);
+
 // ---- unsplit polynomial scheme (unsplit.cu)
 // psi <- U psi at every point (normal layout).
 template <typename T>
 cudaError_t launch_apply_u(Q4<T>* psi, const Q4<T>* u, size_t n, cudaStream_t st);
-// out = alpha (b1 sigma_x dx + b2 sigma_y dy) + beta prev (prev may be null); acc +=
-// gamma out (acc may be null); b^j = a^j / S^j from the FP64 fields (complex when the
+// out = alpha (b1 sigma_x dx + b2 sigma_y dy) + gamma base + beta prev (base and prev may
+// be null); b^j = a^j / S^j from the FP64 fields (complex when the
 // imaginary parts of 1/S are given); all normal layout.
 template <typename T>
 cudaError_t launch_unsplit_combine(const Q4<T>* dx, const Q4<T>* dy, const double* a1,
                                    const double* a2, const double* sxinv, const double* syinv,
                                    const double* sxinv_im, const double* syinv_im, int nx,
-                                   int ny, double ar, double ai, const Q4<T>* prev,
-                                   double beta, double gr, double gi, Q4<T>* out, Q4<T>* acc,
+                                   int ny, double ar, double ai, const Q4<T>* base, double gr,
+                                   double gi, const Q4<T>* prev, double beta, Q4<T>* out,
                                    cudaStream_t st);
 // out = c in.
 template <typename T>
@@ -137,20 +140,30 @@ cudaError_t launch_scale(Q4<T>* out, const Q4<T>* in, double cr, double ci, size
 cudaError_t launch_max_b(const double* a1, const double* a2, const double* sxinv,
                          const double* syinv, const double* sxinv_im, const double* syinv_im,
                          int nx, int ny, double* partials, int n_blocks, cudaStream_t st);
-// Krylov building blocks (Scheme I). Partial inner products <V_i, w> (i < count) in
-// FP64: partials[2 (i n_blocks + b)] (re, im) per block b; V is a device array of count
-// pointers.
+// Krylov building blocks (Scheme I); V is a device array of count vector pointers, every
+// launch uses at most n_blocks blocks per chunk of vectors and leaves its sums, added in a fixed
+// order, in device memory (partials: 2 n_blocks count doubles; ticket: a zeroed counter).
+// kind 0: dots[2 i] = <V_i, w> (re, im);
+// kind 1: w -= sum_i coef_i V_i, then dots as for kind 0 (count <= 4);
+// kind 2: w -= sum_i coef_i V_i, then dots[0] = <w, w>, dots[1] = 1 / sqrt(dots[0]) (1 unless
+// dots[0] > 0).
 template <typename T>
-cudaError_t launch_multi_dot(const Q4<T>* const* V, int count, const Q4<T>* w, size_t n,
-                             double* partials, int n_blocks, cudaStream_t st);
+cudaError_t launch_gram_schmidt(int kind, const Q4<T>* const* V, int count, Q4<T>* w,
+                                const double* coef, size_t n, double* partials, unsigned* ticket,
+                                double* dots, int n_blocks, cudaStream_t st);
+// v = 2 (rhs - x) (mode 0) or rhs - v (mode 1); dots[0] = <v, v>, dots[1] = <rhs, rhs> (mode 0),
+// dots[2] = 1 / sqrt(dots[0]) (1 unless dots[0] > 0).
+template <typename T>
+cudaError_t launch_residual(int mode, const Q4<T>* rhs, const Q4<T>* x, Q4<T>* v, size_t n,
+                            double* partials, unsigned* ticket, double* dots, int n_blocks,
+                            cudaStream_t st);
+// v *= inv[0] (device memory).
+template <typename T>
+cudaError_t launch_normalise(Q4<T>* v, const double* inv, size_t n, cudaStream_t st);
 // out += sum_i coef_i V_i with complex FP64 coef (device array of 2 count doubles).
 template <typename T>
 cudaError_t launch_multi_axpy(Q4<T>* out, const Q4<T>* const* V, const double* coef, int count,
                               size_t n, cudaStream_t st);
-// out = a x + b y.
-template <typename T>
-cudaError_t launch_axpby(Q4<T>* out, double a, const Q4<T>* x, double b, const Q4<T>* y,
-                         size_t n, cudaStream_t st);
 // J_0(x) .. J_n(x) into out[0..n] (host, FP64); false for x < 0 or n < 0.
 bool bessel_j_series(double x, int n, double* out);
 

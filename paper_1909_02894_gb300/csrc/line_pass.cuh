@@ -76,6 +76,30 @@ struct LinePassArgs {
                             // [n_lines][L] like `in` (out must not alias in)
 };
 
+// One phase of the unsplit operator (team_unsplit.cuh). All arrays are [n_lines][L] in the
+// layout of the rows, except the transposed outputs ([L][n_lines]).
+struct UnsplitArgs {
+  const Q4<float>* in;
+  Q4<float>* out;       // phase 1: b sigma d in, transposed; phase 2: the result
+  Q4<float>* out_in;    // phase 1: a transposed copy of `in`
+  const float* beta;    // b - 1 of this axis
+  const Cx<float>* tw;  // launch_team_twiddles of this axis
+  const Q4<float>* mult;  // derivative multipliers of this axis, in team_perm order
+  int n_lines;
+  int axis;               // 0: sigma_x, 1: sigma_y
+  // phase 2: out = (ar + i ai) (s_other + this axis' term) + (gr + i gi) base + beta_prev prev,
+  // then U out if u_store; base, prev and u_store may be null
+  const Q4<float>* s_other;
+  float ar, ai;
+  const Q4<float>* base;
+  float gr, gi;
+  const Q4<float>* prev;
+  float beta_prev;
+  const Q4<float>* u_store;
+  int store_normal;  // 1: out is [n_lines][L], 0: transposed
+  int* err;
+};
+
 // Batched launches: a block (or group) of lines belongs to instance `k`; take that
 // instance's pointers.
 template <typename T>

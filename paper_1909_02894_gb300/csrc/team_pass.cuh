@@ -44,27 +44,36 @@ namespace dgb {
 constexpr uint64_t kWaitNs = 1500000000ull;  // 1.5 s: a copy of 64 KB takes microseconds
 constexpr int kErrTimeout = 1;
 
-// LPC teams per CTA. PAIR: groups of GT threads (a team, or the two teams of a warp) work
-// independently on their own units and mbarriers; otherwise the CTA is one group.
-template <int L, int LPC_, bool PAIR>
-struct TGeo {
+// Geometry of one line: T threads, blocks of R2 of them, exchange slots.
+template <int L>
+struct TLine {
   static constexpr int T = L / 16;       // threads of a team
   static constexpr int R2 = L / 256;     // last radix, threads of a block
   static constexpr int NB = 16 / R2;     // last-radix butterflies per thread
-  static constexpr int LPC = LPC_;       // teams of a CTA
-  static constexpr int THREADS = LPC * T;
-  static constexpr int GT = PAIR ? (T > 32 ? T : 32) : THREADS;  // threads of a group
-  static constexpr int GROUPS = THREADS / GT;
-  static constexpr int LG = GT / T;                // lines a group runs at once
-  static constexpr int LPU = LG * (PAIR ? 2 : 1);  // lines of a work unit
   // Slots (8 bytes) between blocks and between the rows of a block: both exchanges touch 16
   // different 8-byte banks per half-warp when BS = R2 mod 16 and RS = R2 + 1.
   static constexpr int BS = R2 == 16 ? 272 : R2 == 8 ? 152 : R2 == 4 ? 84 : R2 == 2 ? 50 : 17;
   static constexpr int RS = R2 + 1;
   static constexpr int COMP = 16 * BS;              // slots of one component of a line
   static constexpr size_t LINE_BYTES = 2 * (size_t)COMP * 8;
+  static_assert(BS % 16 == R2 % 16 && BS >= 16 * RS - (R2 == 1 ? 15 : 0), "exchange layout");
+  static_assert(LINE_BYTES >= (size_t)L * 16, "landing rows fit the exchange buffer");
+};
+
+// LPC teams per CTA. PAIR: groups of GT threads (a team, or the two teams of a warp) work
+// independently on their own units and mbarriers; otherwise the CTA is one group.
+template <int L, int LPC_, bool PAIR>
+struct TGeo : TLine<L> {
+  using TL = TLine<L>;
+  static constexpr int T = TL::T, R2 = TL::R2;
+  static constexpr int LPC = LPC_;       // teams of a CTA
+  static constexpr int THREADS = LPC * T;
+  static constexpr int GT = PAIR ? (T > 32 ? T : 32) : THREADS;  // threads of a group
+  static constexpr int GROUPS = THREADS / GT;
+  static constexpr int LG = GT / T;                // lines a group runs at once
+  static constexpr int LPU = LG * (PAIR ? 2 : 1);  // lines of a work unit
   static constexpr int SPITCH = L + (LPC > 1 ? 8 / LPC : 0);  // staging rows (points)
-  static constexpr size_t XBYTES = LPC * LINE_BYTES;
+  static constexpr size_t XBYTES = LPC * TL::LINE_BYTES;
   static constexpr size_t STAGE = PAIR ? 0 : (size_t)LPC * SPITCH * 16;
   static constexpr size_t OFF_BAR = ((XBYTES > STAGE ? XBYTES : STAGE) + 15) / 16 * 16;
   // per group: an mbarrier and a failure flag; then the tensor-memory address
@@ -75,8 +84,6 @@ struct TGeo {
   static constexpr int MINB = PAIR ? 512 / THREADS : THREADS >= 64 ? 512 / THREADS : 8;
   static constexpr uint32_t PARK = PAIR ? 128 : 64;  // tensor-memory columns per thread
   static constexpr uint32_t TCOLS = PARK * (THREADS > 128 ? THREADS / 128 : 1);
-  static_assert(BS % 16 == R2 % 16 && BS >= 16 * RS - (R2 == 1 ? 15 : 0), "exchange layout");
-  static_assert(LINE_BYTES >= (size_t)L * 16, "landing rows fit the exchange buffer");
   static_assert(THREADS % 32 == 0 && (THREADS <= 128 || THREADS % 128 == 0), "lane quarters");
   static_assert(SMEM <= 227 * 1024 && (SMEM + 1024) * MINB <= 228 * 1024, "resident CTAs");
   static_assert(TCOLS * MINB <= 512, "tensor memory of the resident CTAs");
@@ -127,11 +134,146 @@ __device__ __forceinline__ void team_dft_r2(Cx<float> (&v)[16]) {
   }
 }
 
+// rows of a line brought into L2, one request per 128 bytes
+template <int L, typename V>
+__device__ __forceinline__ void team_prefetch(const V* p, int j) {
+  constexpr int STEP = 128 / sizeof(V);
+  for (int t = j * STEP; t < L; t += L / 16 * STEP)
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(p + t));
+}
+
+// From the loaded points (element m of thread j: point j + T m, both components) through the
+// forward FFT, the multiply and the inverse FFT up to its last DFT-16, which the caller runs
+// after it has released the exchange buffer. xp: the line's exchange buffer, blk: this
+// thread's block in it; tw1, tw2, mt: this thread's twiddles W_L^(j k) (stride T) and
+// W_T^(u k) (stride R2, shared memory) and multipliers (stride T). mid runs once, between the
+// first exchange's writes and its barrier.
+template <int L, int LPC, bool DERIV, typename Mid>
+__device__ __forceinline__ void team_transform(Cx<float> (&vp)[16], Cx<float> (&vm)[16],
+                                               Cx<float>* xp, Cx<float>* blk,
+                                               const Cx<float>* tw1, const Cx<float>* tw2,
+                                               const Q4<float>* mt, int lt, int j, int u, Mid mid) {
+  using G = TLine<L>;
+  constexpr int T = G::T, R2 = G::R2, NB = G::NB, BS = G::BS, RS = G::RS;
+  // exchange slots of the line and from the block's first one (debug index checks)
+  auto xz = [&](int i) { return (int)dbg_at(i, (size_t)2 * G::COMP); };
+  auto bz = [&](int i) { return (int)dbg_at(i, (size_t)2 * G::COMP - (j / R2) * BS); };
+  dft16<float, false, false>(vp);
+  dft16<float, false, false>(vm);
+  team_sync<T, LPC>(lt);  // the landing rows have been read
+  {
+    const Cx<float>* tw = tw1;
+    xp[xz(j)] = vp[0];
+    xp[xz(G::COMP + j)] = vm[0];
+#pragma unroll
+    for (int k = 1; k < 16; ++k) {
+      const Cx<float> w = ldg_cx(tw + (k - 1) * T);
+      xp[xz(k * BS + j)] = cmul(vp[k], w);
+      xp[xz(G::COMP + k * BS + j)] = cmul(vm[k], w);
+    }
+  }
+  mid();
+  team_sync<T, LPC>(lt);
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    vp[r] = blk[bz(u + R2 * r)];
+    vm[r] = blk[bz(G::COMP + u + R2 * r)];
+  }
+  dft16<float, false, false>(vp);
+  dft16<float, false, false>(vm);
+  if constexpr (R2 > 1) {
+    const Cx<float>* tw = tw2;
+    __syncwarp();  // the block's threads have read it
+    blk[bz(u)] = vp[0];
+    blk[bz(G::COMP + u)] = vm[0];
+#pragma unroll
+    for (int k = 1; k < 16; ++k) {
+      const Cx<float> w = tw[(k - 1) * R2];
+      blk[bz(k * RS + u)] = cmul(vp[k], w);
+      blk[bz(G::COMP + k * RS + u)] = cmul(vm[k], w);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+#pragma unroll
+      for (int t = 0; t < R2; ++t) {
+        vp[q * R2 + t] = blk[bz((u + R2 * q) * RS + t)];
+        vm[q * R2 + t] = blk[bz(G::COMP + (u + R2 * q) * RS + t)];
+      }
+    team_dft_r2<R2, false>(vp);
+    team_dft_r2<R2, false>(vm);
+  }
+  // k-space multiply. Step: eigenvalue +1 by (cos - 1) - i sin, -1 by (cos - 1) + i sin;
+  // derivative: both components by i xi
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    const Q4<float> q = ldg_q4(mt + e * T);
+    {
+      const float vr = vp[e].re, vi = vp[e].im;
+      if constexpr (DERIV)
+        vp[e] = {-(q.z * vi + q.w * vi), q.z * vr + q.w * vr};
+      else
+        vp[e] = {q.x * vr + ((q.y * vr + q.w * vi) + q.z * vi),
+                 q.x * vi + ((q.y * vi - q.w * vr) - q.z * vr)};
+    }
+    {
+      const float vr = vm[e].re, vi = vm[e].im;
+      if constexpr (DERIV)
+        vm[e] = {-(q.z * vi + q.w * vi), q.z * vr + q.w * vr};
+      else
+        vm[e] = {q.x * vr + ((q.y * vr - q.w * vi) - q.z * vi),
+                 q.x * vi + ((q.y * vi + q.w * vr) + q.z * vr)};
+    }
+  }
+  if constexpr (R2 > 1) {
+    team_dft_r2<R2, true>(vp);
+    team_dft_r2<R2, true>(vm);
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+#pragma unroll
+      for (int t = 0; t < R2; ++t) {
+        blk[bz((u + R2 * q) * RS + t)] = vp[q * R2 + t];
+        blk[bz(G::COMP + (u + R2 * q) * RS + t)] = vm[q * R2 + t];
+      }
+    __syncwarp();
+    const Cx<float>* tw = tw2;
+    vp[0] = blk[bz(u)];
+    vm[0] = blk[bz(G::COMP + u)];
+#pragma unroll
+    for (int k = 1; k < 16; ++k) {
+      const Cx<float> w = tw[(k - 1) * R2];
+      vp[k] = cmulc(blk[bz(k * RS + u)], w);
+      vm[k] = cmulc(blk[bz(G::COMP + k * RS + u)], w);
+    }
+    __syncwarp();  // the block's threads have read it
+  }
+  dft16<float, true, false>(vp);
+  dft16<float, true, false>(vm);
+#pragma unroll
+  for (int r = 0; r < 16; ++r) {
+    blk[bz(u + R2 * r)] = vp[r];
+    blk[bz(G::COMP + u + R2 * r)] = vm[r];
+  }
+  team_sync<T, LPC>(lt);
+  {
+    const Cx<float>* tw = tw1;
+    asm volatile("" : "+l"(tw));
+    vp[0] = xp[xz(j)];
+    vm[0] = xp[xz(G::COMP + j)];
+#pragma unroll
+    for (int k = 1; k < 16; ++k) {
+      const Cx<float> w = ldg_cx(tw + (k - 1) * T);
+      vp[k] = cmulc(xp[xz(k * BS + j)], w);
+      vm[k] = cmulc(xp[xz(G::COMP + k * BS + j)], w);
+    }
+  }
+}
+
 template <int L, int LPC, bool PAIR, bool BATCH, int SIGMA>
 __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR>::MINB)
     line_pass_team(const LinePassArgs<float> a0, int n_units, int* __restrict__ err) {
   using G = TGeo<L, LPC, PAIR>;
-  constexpr int T = G::T, R2 = G::R2, NB = G::NB, BS = G::BS, RS = G::RS;
+  constexpr int T = G::T, R2 = G::R2, BS = G::BS;
   extern __shared__ __align__(128) unsigned char tsm[];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int lt = tid / T, j = tid - lt * T;
@@ -149,11 +291,9 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
   pdl_wait();
   pdl_launch_next();
   const int upi = a0.n_lines / G::LPU;  // units of an instance
-  // index checks of the debug build (no code otherwise): landing rows, exchange slots of the
-  // line and from the block's first one, staging, points of the global arrays
+  // index checks of the debug build (no code otherwise): landing rows, staging, points of the
+  // global arrays
   auto lz = [&](int i) { return (int)dbg_at(i, (size_t)L); };
-  auto xz = [&](int i) { return (int)dbg_at(i, (size_t)2 * G::COMP); };
-  auto bz = [&](int i) { return (int)dbg_at(i, (size_t)2 * G::COMP - (j / R2) * BS); };
   auto sz = [&](int i) { return (int)dbg_at(i, (size_t)LPC * G::SPITCH); };
   auto gz = [&](size_t i) { return dbg_at(i, (size_t)a0.n_lines * L); };
   if constexpr (BATCH) n_units = *a0.n_inst * upi;
@@ -208,7 +348,6 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
     const int line = ul * G::LPU + (PAIR ? 2 * lg + h : lg);
     const size_t row = (size_t)line * L;
     Cx<float> vp[16], vm[16];
-    const Cx<float>* tw1 = a.tw + j;
     const bool ok = mbar_wait_bounded(bar, par, kWaitNs);
     par ^= 1u;
     if (a.u_load) {  // first pass of a call: U applied to the landed points in place
@@ -237,118 +376,12 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
       }
       tmem_st16(tpark + (uint32_t)((PAIR ? 64 * h : 0) + 16 * g), pk);
     }
-    dft16<float, false, false>(vp);
-    dft16<float, false, false>(vm);
-    team_sync<T, LPC>(lt);  // the landing rows have been read
-    {
-      const Cx<float>* tw = tw1;
-      xp[xz(j)] = vp[0];
-      xp[xz(G::COMP + j)] = vm[0];
-#pragma unroll
-      for (int k = 1; k < 16; ++k) {
-        const Cx<float> w = ldg_cx(tw + (k - 1) * T);
-        xp[xz(k * BS + j)] = cmul(vp[k], w);
-        xp[xz(G::COMP + k * BS + j)] = cmul(vm[k], w);
-      }
-    }
-    // the line's coefficients into L2, a line's transforms ahead of their use (bulk prefetches
-    // queue with the landing copies and were slower)
-    if (a.u_store)
-      for (int t = j * 8; t < L; t += T * 8)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.u_store + row + t));
-    if (a.beta)
-      for (int t = j * 32; t < L; t += T * 32)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(a.beta + row + t));
-    team_sync<T, LPC>(lt);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      vp[r] = blk[bz(u + R2 * r)];
-      vm[r] = blk[bz(G::COMP + u + R2 * r)];
-    }
-    dft16<float, false, false>(vp);
-    dft16<float, false, false>(vm);
-    if constexpr (R2 > 1) {
-      const Cx<float>* tw = tw2s + u;
-      __syncwarp();  // the block's threads have read it
-      blk[bz(u)] = vp[0];
-      blk[bz(G::COMP + u)] = vm[0];
-#pragma unroll
-      for (int k = 1; k < 16; ++k) {
-        const Cx<float> w = tw[(k - 1) * R2];
-        blk[bz(k * RS + u)] = cmul(vp[k], w);
-        blk[bz(G::COMP + k * RS + u)] = cmul(vm[k], w);
-      }
-      __syncwarp();
-#pragma unroll
-      for (int q = 0; q < NB; ++q)
-#pragma unroll
-        for (int t = 0; t < R2; ++t) {
-          vp[q * R2 + t] = blk[bz((u + R2 * q) * RS + t)];
-          vm[q * R2 + t] = blk[bz(G::COMP + (u + R2 * q) * RS + t)];
-        }
-      team_dft_r2<R2, false>(vp);
-      team_dft_r2<R2, false>(vm);
-    }
-    // k-space multiply: eigenvalue +1 by (cos - 1) - i sin, -1 by (cos - 1) + i sin
-    {
-      const Q4<float>* mt = a.mult_perm + j;
-#pragma unroll
-      for (int e = 0; e < 16; ++e) {
-        const Q4<float> q = ldg_q4(mt + e * T);
-        {
-          const float vr = vp[e].re, vi = vp[e].im;
-          vp[e] = {q.x * vr + ((q.y * vr + q.w * vi) + q.z * vi),
-                   q.x * vi + ((q.y * vi - q.w * vr) - q.z * vr)};
-        }
-        {
-          const float vr = vm[e].re, vi = vm[e].im;
-          vm[e] = {q.x * vr + ((q.y * vr - q.w * vi) - q.z * vi),
-                   q.x * vi + ((q.y * vi + q.w * vr) + q.z * vr)};
-        }
-      }
-    }
-    if constexpr (R2 > 1) {
-      team_dft_r2<R2, true>(vp);
-      team_dft_r2<R2, true>(vm);
-#pragma unroll
-      for (int q = 0; q < NB; ++q)
-#pragma unroll
-        for (int t = 0; t < R2; ++t) {
-          blk[bz((u + R2 * q) * RS + t)] = vp[q * R2 + t];
-          blk[bz(G::COMP + (u + R2 * q) * RS + t)] = vm[q * R2 + t];
-        }
-      __syncwarp();
-      const Cx<float>* tw = tw2s + u;
-      vp[0] = blk[bz(u)];
-      vm[0] = blk[bz(G::COMP + u)];
-#pragma unroll
-      for (int k = 1; k < 16; ++k) {
-        const Cx<float> w = tw[(k - 1) * R2];
-        vp[k] = cmulc(blk[bz(k * RS + u)], w);
-        vm[k] = cmulc(blk[bz(G::COMP + k * RS + u)], w);
-      }
-      __syncwarp();  // the block's threads have read it
-    }
-    dft16<float, true, false>(vp);
-    dft16<float, true, false>(vm);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      blk[bz(u + R2 * r)] = vp[r];
-      blk[bz(G::COMP + u + R2 * r)] = vm[r];
-    }
-    team_sync<T, LPC>(lt);
-    {
-      const Cx<float>* tw = tw1;
-      asm volatile("" : "+l"(tw));
-      vp[0] = xp[xz(j)];
-      vm[0] = xp[xz(G::COMP + j)];
-#pragma unroll
-      for (int k = 1; k < 16; ++k) {
-        const Cx<float> w = ldg_cx(tw + (k - 1) * T);
-        vp[k] = cmulc(xp[xz(k * BS + j)], w);
-        vm[k] = cmulc(xp[xz(G::COMP + k * BS + j)], w);
-      }
-    }
+    team_transform<L, LPC, false>(vp, vm, xp, blk, a.tw + j, tw2s + u, a.mult_perm + j, lt, j, u, [&]() {
+      // the line's coefficients into L2, a line's transforms ahead of their use (bulk
+      // prefetches queue with the landing copies and were slower)
+      if (a.u_store) team_prefetch<L>(a.u_store + row, j);
+      if (a.beta) team_prefetch<L>(a.beta + row, j);
+    });
     // the exchange buffer is free: the next rows may land in it
     if (!ok) *bad = 1;
     group_sync();

@@ -38,14 +38,14 @@ __global__ void k_apply_ug(Q4<T>* psi, const Q4<T>* ug, size_t n) {
 }
 
 // S = b1 sigma_x dx + b2 sigma_y dy with sigma_x (u, v) = (v, u), sigma_y (u, v) =
-// (-i v, i u); out = alpha S + beta prev; acc += gamma out.
+// (-i v, i u); out = alpha S + gamma base + beta prev.
 // b^j complex with complex stretching (sxinv_im, syinv_im not null).
 template <typename T>
 __global__ void k_unsplit_combine(const Q4<T>* dx, const Q4<T>* dy, const double* a1,
                                   const double* a2, const double* sxinv, const double* syinv,
                                   const double* sxinv_im, const double* syinv_im, int nx,
-                                  int ny, T ar, T ai, const Q4<T>* prev, T beta, T gr, T gi,
-                                  Q4<T>* out, Q4<T>* acc) {
+                                  int ny, T ar, T ai, const Q4<T>* base, T gr, T gi,
+                                  const Q4<T>* prev, T beta, Q4<T>* out) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= (size_t)nx * ny) return;
   const int j = (int)(k / nx), i = (int)(k - (size_t)j * nx);
@@ -60,6 +60,13 @@ __global__ void k_unsplit_combine(const Q4<T>* dx, const Q4<T>* dy, const double
   const T s2r = (b1 * x.x - b1i * x.y) + (b2 * t2r - b2i * t2i);
   const T s2i = (b1 * x.y + b1i * x.x) + (b2 * t2i + b2i * t2r);
   Q4<T> o = {ar * s1r - ai * s1i, ar * s1i + ai * s1r, ar * s2r - ai * s2i, ar * s2i + ai * s2r};
+  if (base) {
+    const Q4<T> p = base[k];
+    o.x += gr * p.x - gi * p.y;
+    o.y += gr * p.y + gi * p.x;
+    o.z += gr * p.z - gi * p.w;
+    o.w += gr * p.w + gi * p.z;
+  }
   if (prev) {
     const Q4<T> p = prev[k];
     o.x += beta * p.x;
@@ -68,23 +75,6 @@ __global__ void k_unsplit_combine(const Q4<T>* dx, const Q4<T>* dy, const double
     o.w += beta * p.w;
   }
   out[k] = o;
-  if (acc) {
-    Q4<T> s = acc[k];
-    s.x += gr * o.x - gi * o.y;
-    s.y += gr * o.y + gi * o.x;
-    s.z += gr * o.z - gi * o.w;
-    s.w += gr * o.w + gi * o.z;
-    acc[k] = s;
-  }
-}
-
-// out = c in (complex c)
-template <typename T>
-__global__ void k_scale(Q4<T>* out, const Q4<T>* in, T cr, T ci, size_t n) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const Q4<T> v = in[k];
-  out[k] = {cr * v.x - ci * v.y, cr * v.y + ci * v.x, cr * v.z - ci * v.w, cr * v.w + ci * v.z};
 }
 
 // Per-block maxima of |b1| and |b2| (grid-stride), partials[2 b], partials[2 b + 1].
@@ -116,35 +106,222 @@ __global__ void k_max_b(const double* a1, const double* a2, const double* sxinv,
   }
 }
 
-// ---- Krylov building blocks (Scheme I): FP64 accumulation of complex inner products
-// <V_i, w> = sum conj(V_i) w over both components; block (x, i) writes its partial sum
-// of vector i to partials[2 (i gridDim.x + x)], fixed grid so the sum order is fixed.
+// ---- Krylov building blocks (Scheme I): complex inner products <V_i, w> = sum conj(V_i) w
+// over both components, accumulated beyond the state's precision.
+//
+// FP64 states: FP64 fused multiply-adds. FP32 states: the FP64 pipe (two lanes per SM and
+// clock, conversions included) made a product of two vectors cost 14 us at 512^2, four times
+// its memory traffic; instead each product is split exactly into its FP32 rounding and the
+// remainder (an FMA), and both are added to a sum of three FP32 terms by two-sums (Knuth; the
+// scheme of Ogita, Rump and Oishi's DotK with K = 3, threefold FP32 precision), within 8
+// points of a thread and across the 32 lanes of a warp; everything beyond is added in FP64.
+// Error of a product of unit vectors against the exact sum, 4096 to 2^20 points (noise and wave
+// packets, emulated): at most 2.8e-17, the same as FP64 fused multiply-adds per thread (rms
+// 1.3e-19..1.2e-17 and 1.1e-19..1.2e-17).
 template <typename T>
-__global__ void k_multi_dot(const Q4<T>* const* V, const Q4<T>* w, size_t n, double* partials) {
-  __shared__ double sr[TPB], si[TPB];
-  const Q4<T>* v = V[blockIdx.y];
-  double ar = 0.0, ai = 0.0;
-  for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
-       k += (size_t)gridDim.x * blockDim.x) {
-    const Q4<T> a = v[k], b = w[k];
-    ar += (double)a.x * b.x + (double)a.y * b.y + (double)a.z * b.z + (double)a.w * b.w;
-    ai += (double)a.x * b.y - (double)a.y * b.x + (double)a.z * b.w - (double)a.w * b.z;
+struct DotAcc;
+template <>
+struct DotAcc<double> {
+  double d = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { d += a * b; }
+  __device__ __forceinline__ void sub(double a, double b) { d -= a * b; }
+  __device__ __forceinline__ void flush() {}
+  // the warp's sum (valid in lane 0); `flushed` (uniform): flush has been called
+  __device__ __forceinline__ double warp_total(bool) {
+    for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+    return d;
   }
-  sr[threadIdx.x] = ar;
-  si[threadIdx.x] = ai;
-  __syncthreads();
-  for (int s = TPB / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) {
-      sr[threadIdx.x] += sr[threadIdx.x + s];
-      si[threadIdx.x] += si[threadIdx.x + s];
+};
+template <>
+struct DotAcc<float> {
+  double d = 0.0;
+  float s = 0.f, c = 0.f, g = 0.f;
+  // x <- the rounded x + p; returns the rounding error exactly
+  static __device__ __forceinline__ float two_sum(float& x, float p) {
+    const float t = __fadd_rn(x, p), z = __fsub_rn(t, x);
+    const float r = __fadd_rn(__fsub_rn(x, __fsub_rn(t, z)), __fsub_rn(p, z));
+    x = t;
+    return r;
+  }
+  // the sum of hi + lo, lo at the scale of hi's rounding
+  __device__ __forceinline__ void add_pair(float hi, float lo) {
+    const float r1 = two_sum(s, hi), r2 = two_sum(lo, r1), r3 = two_sum(c, lo);
+    g = __fadd_rn(g, __fadd_rn(r2, r3));
+  }
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    add_pair(p, __fmaf_rn(a, b, -p));
+  }
+  __device__ __forceinline__ void sub(float a, float b) { add(-a, b); }
+  __device__ __forceinline__ void flush() {
+    d += (double)s + ((double)c + (double)g);
+    s = c = g = 0.f;
+  }
+  __device__ __forceinline__ double warp_total(bool flushed) {
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ps = __shfl_down_sync(0xffffffffu, s, o);
+      const float pc = __shfl_down_sync(0xffffffffu, c, o);
+      const float pg = __shfl_down_sync(0xffffffffu, g, o);
+      add_pair(ps, pc);
+      g = __fadd_rn(g, pg);
     }
+    if (flushed)
+      for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
+    return (threadIdx.x & 31) == 0 ? d + ((double)s + ((double)c + (double)g)) : 0.0;
+  }
+};
+template <typename T>
+__device__ __forceinline__ void dot_point(DotAcc<T>& re, DotAcc<T>& im, const Q4<T>& a,
+                                          const Q4<T>& b) {
+  re.add(a.x, b.x);
+  re.add(a.y, b.y);
+  re.add(a.z, b.z);
+  re.add(a.w, b.w);
+  im.add(a.x, b.y);
+  im.sub(a.y, b.x);
+  im.add(a.z, b.w);
+  im.sub(a.w, b.z);
+}
+template <typename A, typename T>
+__device__ __forceinline__ void norm_point(DotAcc<A>& re, const Q4<T>& a) {
+  re.add(a.x, a.x);
+  re.add(a.y, a.y);
+  re.add(a.z, a.z);
+  re.add(a.w, a.w);
+}
+
+// Sums `count` values per block (accumulators acc[i] of each thread) into partials[i gridDim.x +
+// block]; the grid's last block to finish adds the blocks' partial sums, in the order of a
+// fixed tree, into result[i], and resets the ticket. total: values over all gridDim.y chunks;
+// first: this chunk's first value. INV: result[total] = 1 / sqrt(result[0]), or 1 unless
+// result[0] > 0.
+template <int N, bool INV, typename A>
+__device__ __forceinline__ void grid_sums(DotAcc<A> (&acc)[N], bool flushed, int count, int first,
+                                          int total, double* partials, unsigned* ticket,
+                                          double* result) {
+  __shared__ double sh[N][TPB / 32];
+  __shared__ bool last;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (i < count) {
+      const double v = acc[i].warp_total(flushed);
+      if (lane == 0) sh[i][wid] = v;
+    }
+  __syncthreads();
+  if ((int)threadIdx.x < count) {
+    double v = 0.0;
+    for (int t = 0; t < TPB / 32; ++t) v += sh[threadIdx.x][t];
+    partials[(size_t)(first + threadIdx.x) * gridDim.x + blockIdx.x] = v;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int i = wid; i < total; i += TPB / 32) {
+    double v = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(partials + (size_t)i * gridDim.x + b);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) result[i] = v;
+  }
+  if constexpr (INV) {
     __syncthreads();
+    if (threadIdx.x == 0) result[total] = result[0] > 0.0 ? 1.0 / sqrt(result[0]) : 1.0;
   }
-  if (threadIdx.x == 0) {
-    const size_t o = 2 * ((size_t)blockIdx.y * gridDim.x + blockIdx.x);
-    partials[o] = sr[0];
-    partials[o + 1] = si[0];
+  if (threadIdx.x == 0) *ticket = 0;
+}
+
+constexpr int kChunk = 4;  // vectors whose products a thread accumulates at once
+
+// KIND 0: dots of the chunk's vectors with w. KIND 1 (one chunk): w -= sum coef_i V_i first.
+// KIND 2 (grid.y = 1): w -= sum coef_i V_i over all `count` vectors, then the norm of w.
+template <typename T, int KIND>
+__global__ void __launch_bounds__(TPB) k_gram_schmidt(const Q4<T>* const* V, int count, Q4<T>* w,
+                                                      const double* coef, size_t n,
+                                                      double* partials, unsigned* ticket,
+                                                      double* dots) {
+  const int first = KIND == 0 ? blockIdx.y * kChunk : 0;
+  const int c = KIND == 2 ? count : min(kChunk, count - first);
+  DotAcc<T> acc[KIND == 2 ? 1 : 2 * kChunk];  // re, im of each product; the norm
+  int since = 0;
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  const bool flushed = n > 8 * stride;
+  for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
+    Q4<T> x = w[k];
+    if constexpr (KIND == 2) {
+      for (int i = 0; i < c; ++i) {
+        const T cr = (T)-coef[2 * i], ci = (T)-coef[2 * i + 1];
+        const Q4<T> v = V[i][k];
+        x.x += cr * v.x - ci * v.y;
+        x.y += cr * v.y + ci * v.x;
+        x.z += cr * v.z - ci * v.w;
+        x.w += cr * v.w + ci * v.z;
+      }
+      w[k] = x;
+      norm_point(acc[0], x);
+    } else {
+      Q4<T> v[kChunk];
+#pragma unroll
+      for (int i = 0; i < kChunk; ++i)
+        if (i < c) v[i] = V[first + i][k];
+      if constexpr (KIND == 1) {
+#pragma unroll
+        for (int i = 0; i < kChunk; ++i)
+          if (i < c) {
+            const T cr = (T)-coef[2 * i], ci = (T)-coef[2 * i + 1];
+            x.x += cr * v[i].x - ci * v[i].y;
+            x.y += cr * v[i].y + ci * v[i].x;
+            x.z += cr * v[i].z - ci * v[i].w;
+            x.w += cr * v[i].w + ci * v[i].z;
+          }
+        w[k] = x;
+      }
+#pragma unroll
+      for (int i = 0; i < kChunk; ++i)
+        if (i < c) dot_point(acc[2 * i], acc[2 * i + 1], v[i], x);
+    }
+    if (flushed && ++since == 8) {
+      since = 0;
+#pragma unroll
+      for (int i = 0; i < (KIND == 2 ? 1 : 2 * kChunk); ++i) acc[i].flush();
+    }
   }
+  if constexpr (KIND == 2)
+    grid_sums<1, true>(acc, flushed, 1, 0, 1, partials, ticket, dots);
+  else
+    grid_sums<2 * kChunk, false>(acc, flushed, 2 * c, 2 * first, 2 * count, partials, ticket, dots);
+}
+
+// FP64 sums in both precisions: these vectors carry the state's own scale, whose squares may
+// leave the FP32 range (the basis vectors above have unit norm).
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_residual(int mode, const Q4<T>* rhs, const Q4<T>* x,
+                                                  Q4<T>* v, size_t n, double* partials,
+                                                  unsigned* ticket, double* dots) {
+  DotAcc<double> acc[2];
+  const size_t stride = (size_t)gridDim.x * blockDim.x;
+  for (size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x; k < n; k += stride) {
+    const Q4<T> b = rhs[k], q = mode == 0 ? x[k] : v[k];
+    const T f = mode == 0 ? T(2) : T(1);
+    const Q4<T> r = {f * (b.x - q.x), f * (b.y - q.y), f * (b.z - q.z), f * (b.w - q.w)};
+    v[k] = r;
+    norm_point(acc[0], r);
+    if (mode == 0) norm_point(acc[1], b);
+  }
+  grid_sums<2, true>(acc, true, 2, 0, 2, partials, ticket, dots);
+}
+
+// v *= inv[0]
+template <typename T>
+__global__ void k_normalise(Q4<T>* v, const double* inv, size_t n) {
+  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= n) return;
+  const T c = (T)inv[0];
+  const Q4<T> p = v[k];
+  v[k] = {c * p.x, c * p.y, c * p.z, c * p.w};
 }
 
 // out += sum_i c_i V_i (c complex, coef[2 i], coef[2 i + 1]; FP64 coefficients)
@@ -165,19 +342,41 @@ __global__ void k_multi_axpy(Q4<T>* out, const Q4<T>* const* V, const double* co
   out[k] = o;
 }
 
-// out = a x + b y (real a, b)
-template <typename T>
-__global__ void k_axpby(Q4<T>* out, T a, const Q4<T>* x, T b, const Q4<T>* y, size_t n) {
-  const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
-  const Q4<T> p = x[k], q = y[k];
-  out[k] = {a * p.x + b * q.x, a * p.y + b * q.y, a * p.z + b * q.z, a * p.w + b * q.w};
+// Blocks of a reduction over n points: four points per thread (the sums across threads cost as
+// much as several points), at most n_max.
+static int sum_blocks(size_t n, int n_max) {
+  const size_t b = (n + 4 * TPB - 1) / (4 * TPB);
+  return (int)(b < (size_t)n_max ? b : (size_t)n_max);
 }
 
 template <typename T>
-cudaError_t launch_multi_dot(const Q4<T>* const* V, int count, const Q4<T>* w, size_t n,
-                             double* partials, int n_blocks, cudaStream_t st) {
-  k_multi_dot<T><<<dim3(n_blocks, count), TPB, 0, st>>>(V, w, n, partials);
+cudaError_t launch_gram_schmidt(int kind, const Q4<T>* const* V, int count, Q4<T>* w,
+                                const double* coef, size_t n, double* partials, unsigned* ticket,
+                                double* dots, int n_blocks, cudaStream_t st) {
+  if (count < 1 || (kind == 1 && count > kChunk)) return cudaErrorInvalidValue;
+  n_blocks = sum_blocks(n, n_blocks);
+  if (kind == 0)
+    k_gram_schmidt<T, 0><<<dim3(n_blocks, (count + kChunk - 1) / kChunk), TPB, 0, st>>>(
+        V, count, w, coef, n, partials, ticket, dots);
+  else if (kind == 1)
+    k_gram_schmidt<T, 1><<<n_blocks, TPB, 0, st>>>(V, count, w, coef, n, partials, ticket, dots);
+  else
+    k_gram_schmidt<T, 2><<<n_blocks, TPB, 0, st>>>(V, count, w, coef, n, partials, ticket, dots);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_residual(int mode, const Q4<T>* rhs, const Q4<T>* x, Q4<T>* v, size_t n,
+                            double* partials, unsigned* ticket, double* dots, int n_blocks,
+                            cudaStream_t st) {
+  n_blocks = sum_blocks(n, n_blocks);
+  k_residual<T><<<n_blocks, TPB, 0, st>>>(mode, rhs, x, v, n, partials, ticket, dots);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t launch_normalise(Q4<T>* v, const double* inv, size_t n, cudaStream_t st) {
+  k_normalise<T><<<blocks_for(n), TPB, 0, st>>>(v, inv, n);
   return cudaGetLastError();
 }
 
@@ -185,13 +384,6 @@ template <typename T>
 cudaError_t launch_multi_axpy(Q4<T>* out, const Q4<T>* const* V, const double* coef, int count,
                               size_t n, cudaStream_t st) {
   k_multi_axpy<T><<<blocks_for(n), TPB, 0, st>>>(out, V, coef, count, n);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_axpby(Q4<T>* out, double a, const Q4<T>* x, double b, const Q4<T>* y,
-                         size_t n, cudaStream_t st) {
-  k_axpby<T><<<blocks_for(n), TPB, 0, st>>>(out, (T)a, x, (T)b, y, n);
   return cudaGetLastError();
 }
 
@@ -211,19 +403,12 @@ template <typename T>
 cudaError_t launch_unsplit_combine(const Q4<T>* dx, const Q4<T>* dy, const double* a1,
                                    const double* a2, const double* sxinv, const double* syinv,
                                    const double* sxinv_im, const double* syinv_im, int nx,
-                                   int ny, double ar, double ai, const Q4<T>* prev,
-                                   double beta, double gr, double gi, Q4<T>* out, Q4<T>* acc,
+                                   int ny, double ar, double ai, const Q4<T>* base, double gr,
+                                   double gi, const Q4<T>* prev, double beta, Q4<T>* out,
                                    cudaStream_t st) {
   k_unsplit_combine<T><<<blocks_for((size_t)nx * ny), TPB, 0, st>>>(
-      dx, dy, a1, a2, sxinv, syinv, sxinv_im, syinv_im, nx, ny, (T)ar, (T)ai, prev, (T)beta,
-      (T)gr, (T)gi, out, acc);
-  return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_scale(Q4<T>* out, const Q4<T>* in, double cr, double ci, size_t n,
-                         cudaStream_t st) {
-  k_scale<T><<<blocks_for(n), TPB, 0, st>>>(out, in, (T)cr, (T)ci, n);
+      dx, dy, a1, a2, sxinv, syinv, sxinv_im, syinv_im, nx, ny, (T)ar, (T)ai, base, (T)gr, (T)gi,
+      prev, (T)beta, out);
   return cudaGetLastError();
 }
 
@@ -273,15 +458,15 @@ bool bessel_j_series(double x, int n, double* out) {
   template cudaError_t launch_unsplit_combine<T>(                                            \
       const Q4<T>*, const Q4<T>*, const double*, const double*, const double*, const double*, \
       const double*, const double*, int, int, double, double, const Q4<T>*, double, double,  \
-      double, Q4<T>*, Q4<T>*, cudaStream_t);                                                 \
-  template cudaError_t launch_scale<T>(Q4<T>*, const Q4<T>*, double, double, size_t,         \
-                                       cudaStream_t);                                        \
-  template cudaError_t launch_multi_dot<T>(const Q4<T>* const*, int, const Q4<T>*, size_t,    \
-                                           double*, int, cudaStream_t);                      \
+      const Q4<T>*, double, Q4<T>*, cudaStream_t);                                           \
+  template cudaError_t launch_gram_schmidt<T>(int, const Q4<T>* const*, int, Q4<T>*,          \
+                                              const double*, size_t, double*, unsigned*,      \
+                                              double*, int, cudaStream_t);                    \
+  template cudaError_t launch_residual<T>(int, const Q4<T>*, const Q4<T>*, Q4<T>*, size_t,    \
+                                          double*, unsigned*, double*, int, cudaStream_t);    \
+  template cudaError_t launch_normalise<T>(Q4<T>*, const double*, size_t, cudaStream_t);      \
   template cudaError_t launch_multi_axpy<T>(Q4<T>*, const Q4<T>* const*, const double*, int,  \
-                                            size_t, cudaStream_t);                           \
-  template cudaError_t launch_axpby<T>(Q4<T>*, double, const Q4<T>*, double, const Q4<T>*,   \
-                                       size_t, cudaStream_t);
+                                            size_t, cudaStream_t);
 INST(float)
 INST(double)
 #undef INST

@@ -1,0 +1,92 @@
+"""The radix-16 team pass and the unsplit operator built on it (complex64, axes of 256..4096
+points) against the oracle, at the edges of their launch rules: small CTAs up to 2^18 points,
+staged output up to 2^20, line pairs above; 16 lines of every length; odd and even polynomial
+degrees (the terms alternate between the two layouts); more than four Krylov vectors.
+
+Tolerance: 1e-5 (rel-L2 and layer maximum), the complex64 tolerance of the other parity tests.
+"""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1909_02894_gb300 as D
+from paper_1909_02894_gb300 import workloads as W
+from parity_util import assert_parity
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-5
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    D.build()
+    oracle.build()
+
+
+def grid(nx, ny, noise=0.01, steps=3):
+    ax, ay = 0.1 * nx, 0.1 * ny
+    X, Y = W.mesh(nx, ny, ax, ay)
+    g11 = 1.0 + 0.2 * np.exp(-((X - 0.1 * ax) ** 2 + Y ** 2) / (0.2 * ax * ay))
+    g22 = 1.0 + 0.1 * np.exp(-(X ** 2 + (Y + 0.1 * ay) ** 2) / (0.3 * ax * ay))
+    psi0 = W.wave_packet(nx, ny, ax, ay, 0.1 * min(ax, ay) + 0.5, (1.0, -0.7))
+    psi0 += noise * W.random_state(nx, ny, nx + 3 * ny)
+    return W.Workload("team", nx, ny, ax, ay, np.ones((ny, nx)), g11, g22, mass=0.4, c=1.0,
+                      pml_width_x=nx // 16, pml_width_y=ny // 16, pml_type=1, sigma0=0.5,
+                      theta=0.0, psi0=psi0, dt=0.03, steps=steps)
+
+
+@pytest.mark.parametrize("scheme", [D.DIRAC_SCHEME_II, D.DIRAC_SCHEME_II_SYMMETRIC],
+                         ids=["printed", "symmetric"])
+@pytest.mark.parametrize("nx,ny", [(256, 16), (512, 16), (512, 512), (1024, 256), (512, 1024),
+                                   (1024, 1024), (256, 4096), (2048, 512)])
+def test_step_matches_oracle_in_every_launch_shape(nx, ny, scheme):
+    w = grid(nx, ny)
+    osch = oracle.SCHEME_II if scheme == D.DIRAC_SCHEME_II else oracle.SCHEME_II_SYMMETRIC
+    ref = oracle.run(oracle.Problem.from_workload(w), w.psi0, w.dt, 3, scheme=osch)
+    with D.Simulation(w, precision=D.DIRAC_C64, scheme=scheme) as s:
+        D.dirac_set_launch(s.ctx, 1024, 1024)
+        s.set_state(w.psi0)
+        s.step(3, w.dt)
+        assert_parity(s.get_state(), ref, w, TOL)
+
+
+@pytest.mark.parametrize("scheme,family", [(D.DIRAC_SCHEME_POLY_TAYLOR, oracle.POLY_TAYLOR),
+                                           (D.DIRAC_SCHEME_POLY_CHEBYSHEV, oracle.POLY_CHEBYSHEV)])
+@pytest.mark.parametrize("nx,ny,degree", [(256, 512, 1), (256, 512, 2), (256, 512, 3),
+                                          (256, 512, 8), (1024, 1024, 3), (1024, 1024, 8)])
+def test_polynomial_schemes_on_the_team_operator(nx, ny, scheme, family, degree):
+    w = grid(nx, ny, noise=0.0)
+    ref = oracle.run_poly(oracle.Problem.from_workload(w), w.psi0, w.dt, 3, family=family,
+                          order=degree)
+    with D.Simulation(w, precision=D.DIRAC_C64, scheme=scheme, poly_degree=degree) as s:
+        s.set_state(w.psi0)
+        s.step(2, w.dt)
+        s.step(1, w.dt)
+        assert_parity(s.get_state(), ref, w, TOL)
+
+
+@pytest.mark.parametrize("prec", [D.DIRAC_C64, D.DIRAC_C128], ids=["c64", "c128"])
+def test_krylov_solver_beyond_four_vectors(prec):
+    """White noise at a larger time step needs more than four basis vectors per solve: the
+    Gram-Schmidt sweeps beyond the fused one, in chunks of four."""
+    w = grid(256, 256, noise=0.5, steps=2)
+    ref, _ = oracle.run_cn(oracle.Problem.from_workload(w), w.psi0, 0.06, 2, tol=1e-14)
+    with D.Simulation(w, precision=prec, scheme=D.DIRAC_SCHEME_CRANK_NICOLSON) as s:
+        D.dirac_set_krylov(s.ctx, 0.0, 30, 100)
+        s.set_state(w.psi0)
+        s.step(2, 0.06)
+        got = s.get_state()
+        assert D.dirac_krylov_iterations(s.ctx) >= 2 * 6
+    assert_parity(got, ref, w, 1e-11 if prec == D.DIRAC_C128 else TOL)
+
+
+def test_krylov_norms_keep_the_state_s_scale():
+    """States whose squared amplitudes leave the FP32 range are solved as accurately."""
+    w = grid(256, 256, noise=0.0)
+    for scale in (1e-24, 1e22):
+        psi0 = w.psi0 * scale
+        ref, _ = oracle.run_cn(oracle.Problem.from_workload(w), psi0, w.dt, 1, tol=1e-14)
+        with D.Simulation(w, precision=D.DIRAC_C64, scheme=D.DIRAC_SCHEME_CRANK_NICOLSON) as s:
+            s.set_state(psi0)
+            s.step(1, w.dt)
+            assert_parity(s.get_state(), ref, w, TOL)
