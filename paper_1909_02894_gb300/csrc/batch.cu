@@ -4,7 +4,8 @@
 // active context by up to K steps through a device table of per-instance pointers
 // [K steps][2 passes][capacity]. Each class launches, for each step, one x-pass and one
 // y-pass over all its active contexts. The classes run on parallel branches of a CUDA graph
-// so that their work overlaps on the device. The graph of a tick is captured once per
+// so that their work overlaps on the device, but for the classes whose every launch fills it
+// (fills_device), which follow each other on one branch. The graph of a tick is captured once per
 // class layout (classes present and their table capacities) and replayed; between
 // ticks only the tables and the active counts (device memory) change, so contexts are
 // admitted and retired without re-capturing. Within a step, contexts are ordered by
@@ -236,6 +237,18 @@ static dirac_status launch_class_step(dirac_batch* b, Class& c, int k, cudaStrea
   return DIRAC_OK;
 }
 
+// A class whose passes launch the team pass in pairs of lines (launch_team_sized) holds every
+// SM for the length of a pass. Two such classes side by side only delay each other and the
+// small ones: 32 contexts of 128^2..1024^2, 0.174 ms per step with every class on its own
+// branch, 0.164 with all on one, 0.149 with the 512^2 and 1024^2 classes on one and the small
+// ones beside it.
+static bool fills_device(const dirac_batch* b, const Class& c) {
+  if (b->prec != DIRAC_C64 || !team_length(c.nx) || !team_length(c.ny)) return false;
+  for (int p = 0; p < 2; ++p)
+    if (c.opt[p] != -1 && c.opt[p] != 2) return false;
+  return (size_t)c.capacity * c.nx * c.ny >= kTeamPairPointsBatch;
+}
+
 // Capture (or reuse) the graph of one tick for the current class layout.
 template <typename T>
 static dirac_status tick_graph(dirac_batch* b, int K) {
@@ -255,15 +268,19 @@ static dirac_status tick_graph(dirac_batch* b, int K) {
   for (auto& kv : b->classes) {
     Class& c = kv.second;
     if (e != cudaSuccess || st != DIRAC_OK) break;
-    e = cudaStreamWaitEvent(c.stream, b->fork, 0);
+    const bool shared = fills_device(b, c);
+    cudaStream_t st_c = shared ? b->stream : c.stream;
+    if (!shared) e = cudaStreamWaitEvent(c.stream, b->fork, 0);
     for (int k = 0; k < K && e == cudaSuccess && st == DIRAC_OK; ++k)
-      st = launch_class_step<T>(b, c, k, c.stream);
+      st = launch_class_step<T>(b, c, k, st_c);
+    if (shared) continue;
     cudaEvent_t j = nullptr;
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&j, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventRecord(j, c.stream);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, j, 0);
     if (j) joins.push_back(j);
   }
+  for (cudaEvent_t j : joins)  // after the shared branch, which must not wait for the others
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, j, 0);
   cudaError_t e2 = cudaStreamEndCapture(b->stream, &g);
   for (cudaEvent_t j : joins) cudaEventDestroy(j);
   if (st != DIRAC_OK) {

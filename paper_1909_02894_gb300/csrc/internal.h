@@ -46,6 +46,8 @@ void set_global_error(const std::string& msg);
 // step mode, lines of 256..4096 points; otherwise as 1).
 template <typename T>
 cudaError_t launch_line_pass(const LinePassArgs<T>& a, int mode, int opt, cudaStream_t st);
+// The team pass runs pairs of lines from this many points per launch (see launch_team_sized).
+constexpr size_t kTeamPairPoints = (size_t)1 << 20, kTeamPairPointsBatch = (size_t)1 << 21;
 // Elements per thread (8 or 16) the line pass uses for line length L; the twiddle table
 // of that axis must be built for the same value.
 template <typename T>

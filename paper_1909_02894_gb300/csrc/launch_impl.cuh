@@ -160,7 +160,7 @@ template <int L, bool BATCH, int SIGMA>
 static cudaError_t launch_team_sized(const LinePassArgs<float>& a, cudaStream_t st) {
   constexpr int SMALL = L >= 512 ? 1 : 512 / L, LPC = L >= 2048 ? 1 : 2048 / L;
   const size_t points = (size_t)(BATCH ? a.inst_capacity : 1) * a.n_lines * L;
-  if (points >= ((size_t)1 << (BATCH ? 21 : 20)))
+  if (points >= (BATCH ? kTeamPairPointsBatch : kTeamPairPoints))
     return launch_team_as<L, LPC, true, BATCH, SIGMA>(a, st);
   if (points <= ((size_t)1 << 18)) return launch_team_as<L, SMALL, false, BATCH, SIGMA>(a, st);
   return launch_team_as<L, LPC, false, BATCH, SIGMA>(a, st);

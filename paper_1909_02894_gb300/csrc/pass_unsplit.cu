@@ -41,7 +41,7 @@ static cudaError_t launch_as(const UnsplitArgs& a, cudaStream_t st) {
 template <int L>
 static cudaError_t launch_sized(const UnsplitArgs& a, int phase, cudaStream_t st) {
   constexpr int LPC = L >= 2048 ? 1 : 2048 / L;
-  if ((size_t)a.n_lines * L >= ((size_t)1 << 20))
+  if ((size_t)a.n_lines * L >= kTeamPairPoints)
     return phase == 1 ? launch_as<L, LPC, true, 1>(a, st) : launch_as<L, LPC, true, 2>(a, st);
   return phase == 1 ? launch_as<L, LPC, false, 1>(a, st) : launch_as<L, LPC, false, 2>(a, st);
 }

@@ -90,3 +90,27 @@ def test_krylov_norms_keep_the_state_s_scale():
             s.set_state(psi0)
             s.step(1, w.dt)
             assert_parity(s.get_state(), ref, w, TOL)
+
+
+@pytest.mark.parametrize("scheme", [D.DIRAC_SCHEME_II, D.DIRAC_SCHEME_II_SYMMETRIC],
+                         ids=["printed", "symmetric"])
+@pytest.mark.parametrize("nx,ny", [(512, 256), (128, 512), (256, 128), (1024, 1024)])
+def test_potentials_inside_the_team_pass(nx, ny, scheme):
+    """The general half step in the last pass's store (axes of team-pass length, both layouts)
+    and by its own kernel (the other axes), over two calls and a change of dt."""
+    w = grid(nx, ny)
+    X, Y = W.mesh(nx, ny, w.ax, w.ay)
+    V = 0.8 * np.exp(-(X ** 2 + Y ** 2) / (0.1 * w.ax * w.ay))
+    Ax, Ay = 0.15 * np.sin(np.pi * Y / w.ay), -0.1 * np.sin(np.pi * X / w.ax)
+    prob = oracle.Problem.from_workload(w)
+    prob.V, prob.Ax, prob.Ay = V, Ax, Ay
+    osch = oracle.SCHEME_II if scheme == D.DIRAC_SCHEME_II else oracle.SCHEME_II_SYMMETRIC
+    ref = oracle.run(prob, w.psi0, w.dt, 3, scheme=osch)
+    ref = oracle.run(prob, ref, 0.5 * w.dt, 2, scheme=osch)
+    with D.Simulation(w, precision=D.DIRAC_C64, scheme=scheme) as s:
+        D.dirac_set_potentials(s.ctx, V, Ax, Ay, shape=(ny, nx))
+        s.set_state(w.psi0)
+        s.step(2, w.dt)
+        s.step(1, w.dt)
+        s.step(2, 0.5 * w.dt)
+        assert_parity(s.get_state(), ref, w, TOL)
