@@ -16,6 +16,20 @@ namespace dgb {
 #if DIRAC_DEBUG
 static __device__ int g_dbg_bounds = 0;
 #endif
+// Reads and clears this translation unit's flag (always 0 in release builds).
+inline static int dgb_take_debug_flag() {
+#if DIRAC_DEBUG
+  int v = 0;
+  if (cudaMemcpyFromSymbol(&v, g_dbg_bounds, sizeof(int)) != cudaSuccess) return 1;
+  if (v) {
+    const int z = 0;
+    cudaMemcpyToSymbol(g_dbg_bounds, &z, sizeof(int));
+  }
+  return v;
+#else
+  return 0;
+#endif
+}
 // true when idx < bound (always, in release builds)
 __device__ __forceinline__ bool dbg_in(size_t idx, size_t bound) {
 #if DIRAC_DEBUG
@@ -141,6 +155,17 @@ __device__ __forceinline__ Q4<T> apply_u(Q4<T> u, Q4<T> p) {
   T d2r = u.x * br + u.w * bi + u.y * ar - u.z * ai;
   T d2i = u.x * bi - u.w * br + u.y * ai + u.z * ar;
   return {ar + d1r, ai + d1i, br + d2r, bi + d2i};
+}
+
+// psi <- U psi for a general complex U stored as its deviation from I: r0 = (d00, u01), r1 =
+// (u10, d11).
+template <typename T>
+__device__ __forceinline__ Q4<T> apply_u_general(Q4<T> r0, Q4<T> r1, Q4<T> p) {
+  const T a = p.x, b = p.y, c = p.z, d = p.w;
+  return {a + (r0.x * a - r0.y * b + r0.z * c - r0.w * d),
+          b + (r0.x * b + r0.y * a + r0.z * d + r0.w * c),
+          c + (r1.x * a - r1.y * b + r1.z * c - r1.w * d),
+          d + (r1.x * b + r1.y * a + r1.z * d + r1.w * c)};
 }
 
 }  // namespace dgb

@@ -147,11 +147,18 @@ static dirac_status tables_for_dt(dirac_ctx* ctx, double dt) {
   if (ctx->has_pot) {
     if (!ctx->ug) CK(dalloc(ctx, &ctx->ug, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
     if (!ctx->ug2) CK(dalloc(ctx, &ctx->ug2, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
+    const bool tr = ctx->scheme == DIRAC_SCHEME_II && sizeof(T) == 4 && team_length(ctx->ny);
+    if (tr && !ctx->ug_t)
+      CK(dalloc(ctx, &ctx->ug_t, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
+    if (tr && !ctx->ug2_t)
+      CK(dalloc(ctx, &ctx->ug2_t, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
     CK(launch_halfstep_general<T>(ctx->a1, ctx->a2, ctx->meff, ctx->omx, ctx->omy,
                                   ctx->pot_use[0] ? ctx->pot_v : nullptr,
                                   ctx->pot_use[1] ? ctx->pot_ax : nullptr,
                                   ctx->pot_use[2] ? ctx->pot_ay : nullptr, ctx->nx, ctx->ny, dt,
-                                  (Q4<T>*)ctx->ug, (Q4<T>*)ctx->ug2, st),
+                                  (Q4<T>*)ctx->ug, (Q4<T>*)ctx->ug2,
+                                  tr ? (Q4<T>*)ctx->ug_t : nullptr,
+                                  tr ? (Q4<T>*)ctx->ug2_t : nullptr, st),
        "half-step matrices with potentials");
     ctx->launches += 1;
   }
@@ -218,7 +225,9 @@ static dirac_status step_symmetric(dirac_ctx* ctx, long n) {
   void* oth = ctx->psiT;
   const int opt_x = pass_opt(ctx, ctx->threads_x, ctx->nx);
   const int opt_y = pass_opt(ctx, ctx->threads_y, ctx->ny);
-  const bool fused = !ctx->has_pot;  // potentials: U applied by its own kernel
+  // potentials: as in step_impl, the later U in the last x pass's row store
+  const bool fused = !ctx->has_pot;
+  const bool fused_pot = !fused && sizeof(T) == 4 && opt_x == 2 && team_length(ctx->nx);
   if (!fused) {
     dirac_status r = apply_half<T>(ctx, cur, false);
     if (r != DIRAC_OK) return r;
@@ -236,11 +245,12 @@ static dirac_status step_symmetric(dirac_ctx* ctx, long n) {
     a3.u_store = (!fused || ctx->u_identity)
                      ? nullptr
                      : (const Q4<T>*)(s + 1 == n ? ctx->u_n : ctx->u2_n);
+    a3.ug_store = fused_pot ? (const Q4<T>*)(s + 1 == n ? ctx->ug : ctx->ug2) : nullptr;
     CK(launch_line_pass<T>(a1, MODE_STEP, opt_x, ctx->stream), "x pass (dt/2)");
     CK(launch_line_pass<T>(ay, MODE_STEP, opt_y, ctx->stream), "y pass");
     CK(launch_line_pass<T>(a3, MODE_STEP, opt_x, ctx->stream), "x pass (dt/2, rows)");
     ctx->launches += 3;
-    if (!fused) {
+    if (!fused && !fused_pot) {
       dirac_status r = apply_half<T>(ctx, oth, s + 1 < n);
       if (r != DIRAC_OK) return r;
     }
@@ -665,7 +675,11 @@ static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
   ay.beta_im = (const T*)ctx->beta2T_im;
   ax.test_extra_tx = ay.test_extra_tx = ctx->test_timeout_next;
   ctx->test_timeout_next = 0;
-  const bool fused = !ctx->has_pot;  // potentials: U applied by its own kernel
+  // potentials: the leading U by its own kernel, the later ones in the y pass's store where
+  // that is a team pass, else by their own kernel too
+  const bool fused = !ctx->has_pot;
+  const int opt_y = pass_opt(ctx, ctx->threads_y, ctx->ny);
+  const bool fused_pot = !fused && sizeof(T) == 4 && opt_y == 2 && team_length(ctx->ny);
   if (!fused) CKS(apply_half<T>(ctx, ctx->psi, false));
   for (long s = 0; s < n; ++s) {
     ax.u_load = (fused && s == 0 && !ctx->u_identity) ? (const Q4<T>*)ctx->u_n : nullptr;
@@ -675,10 +689,10 @@ static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
     ay.u_load = nullptr;
     ay.u_store = (!fused || ctx->u_identity) ? nullptr
                                              : (const Q4<T>*)(s + 1 == n ? ctx->u_t : ctx->u2_t);
-    CK(launch_line_pass<T>(ay, MODE_STEP, pass_opt(ctx, ctx->threads_y, ctx->ny), ctx->stream),
-       "y pass");
+    ay.ug_store = fused_pot ? (const Q4<T>*)(s + 1 == n ? ctx->ug_t : ctx->ug2_t) : nullptr;
+    CK(launch_line_pass<T>(ay, MODE_STEP, opt_y, ctx->stream), "y pass");
     ctx->launches += 2;
-    if (!fused) CKS(apply_half<T>(ctx, ctx->psi, s + 1 < n));
+    if (!fused && !fused_pot) CKS(apply_half<T>(ctx, ctx->psi, s + 1 < n));
   }
   return DIRAC_OK;
 }

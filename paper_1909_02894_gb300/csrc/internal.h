@@ -38,6 +38,14 @@ inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t 
   return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
 }
 
+inline int sm_count() {
+  static int cached[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cached[dev]) cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev);
+  return cached[dev];
+}
+
 // Sets the text that dirac_last_error(NULL) returns (errors without a context).
 void set_global_error(const std::string& msg);
 
@@ -60,7 +68,16 @@ int line_pass_radix_alt(int L);
 // translation units; nonzero when a check failed. Always 0 in release builds.
 int dgb_debug_flag_c64();
 int dgb_debug_flag_c128();
-inline int dgb_debug_bounds() { return dgb_debug_flag_c64() | dgb_debug_flag_c128(); }
+int dgb_debug_flag_team_256();
+int dgb_debug_flag_team_512();
+int dgb_debug_flag_team_1024();
+int dgb_debug_flag_team_2048();
+int dgb_debug_flag_team_4096();
+inline int dgb_debug_bounds() {
+  return dgb_debug_flag_c64() | dgb_debug_flag_c128() | dgb_debug_flag_team_256() |
+         dgb_debug_flag_team_512() | dgb_debug_flag_team_1024() | dgb_debug_flag_team_2048() |
+         dgb_debug_flag_team_4096();
+}
 
 // ---- FP64 precompute (precompute.cu)
 // a1, a2, meff, w and the two log fields (packed as a complex128 spinor (f1, f2)) from the
@@ -107,17 +124,25 @@ template <typename T>
 cudaError_t launch_deriv_mult(int n, double a, Q4<T>* mult, cudaStream_t st);
 
 // Half step with static potentials: general complex U and U^2 per point (normal layout,
-// two Q4 per point holding U - I: (d00, u01), (u10, d11)); V, Ax, Ay may be null (0).
+// two Q4 per point holding U - I: (d00, u01), (u10, d11)) and, where ug_t, ug2_t are not
+// null, the same in the transposed layout; V, Ax, Ay may be null (0).
 template <typename T>
 cudaError_t launch_halfstep_general(const double* a1, const double* a2, const double* meff,
                                     const double* omx, const double* omy, const double* V,
                                     const double* Ax, const double* Ay, int nx, int ny,
-                                    double dt, Q4<T>* ug, Q4<T>* ug2, cudaStream_t st);
+                                    double dt, Q4<T>* ug, Q4<T>* ug2, Q4<T>* ug_t, Q4<T>* ug2_t,
+                                    cudaStream_t st);
 // psi <- U psi for such a general U.
 template <typename T>
 cudaError_t launch_apply_ug(Q4<T>* psi, const Q4<T>* ug, size_t n, cudaStream_t st);
 
-// One phase (1 or 2) of the unsplit operator on complex64 rows of L = 256..4096 points.
+// The team pass for one line length (256..4096; one translation unit each, team_<L>.cu), and
+// one phase (1 or 2) of the unsplit operator.
+template <int L>
+cudaError_t launch_team(const LinePassArgs<float>& a, cudaStream_t st);
+template <int L>
+cudaError_t launch_team_unsplit(const UnsplitArgs& a, int phase, cudaStream_t st);
+// One phase of the unsplit operator on complex64 rows of L = 256..4096 points.
 cudaError_t launch_unsplit(const UnsplitArgs& a, int L, int phase, cudaStream_t st);
 
 // ---- unsplit polynomial scheme (unsplit.cu)

@@ -3,7 +3,6 @@
 #include <cuda_runtime.h>
 
 #include "internal.h"
-#include "team_pass.cuh"
 
 namespace dgb {
 
@@ -22,14 +21,6 @@ constexpr int radix_e(int L) {
 template <typename T>
 constexpr int radix_alt(int L) {
   return L < 256 ? 0 : sizeof(T) == 4 ? (L <= 4096 ? 16 : 0) : (L <= 2048 ? 8 : 0);
-}
-
-static int sm_count() {
-  static int cached[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!cached[dev]) cudaDeviceGetAttribute(&cached[dev], cudaDevAttrMultiProcessorCount, dev);
-  return cached[dev];
 }
 
 template <typename T, int L, int LPC, int MODE, int E = radix_e<T>(L)>
@@ -114,63 +105,6 @@ static cudaError_t dispatch(const LinePassArgs<T>& a, int opt, cudaStream_t st) 
     case 2048: return launch_one<T, 2048, 1, MODE>(a, st);
     default: return cudaErrorInvalidValue;
   }
-}
-
-// The radix-16 team pass (complex64 step mode, 256..4096-point lines): as many CTAs as can
-// be resident (128 registers: 512 threads per SM; each CTA takes its share of the tensor
-// memory), at most one per work unit. The CTAs per SM follow from TGeo, as the occupancy
-// query reports one CTA per SM for kernels that allocate tensor memory.
-template <int L, int LPC, bool PAIR, bool BATCH, int SIGMA>
-static cudaError_t launch_team_as(const LinePassArgs<float>& a0, cudaStream_t st) {
-  using G = TGeo<L, LPC, PAIR>;
-  // one U field per pass; b - 1 real
-  if (!a0.err || !a0.tw_team || (!BATCH && !a0.mult_perm) || a0.n_lines % G::LPU != 0 ||
-      (a0.u_load && a0.u_store) || a0.beta_im)
-    return cudaErrorInvalidValue;
-  LinePassArgs<float> a = a0;
-  a.tw = a0.tw_team;
-  auto kern = line_pass_team<L, LPC, PAIR, BATCH, SIGMA>;
-  static bool configured[64] = {false};
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-  if (!configured[dev]) {
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)G::SMEM);
-    if (e != cudaSuccess) return e;
-    configured[dev] = true;
-  }
-  const int units = (BATCH ? a.inst_capacity : 1) * (a.n_lines / G::LPU);
-  const int ctas = (units + G::GROUPS - 1) / G::GROUPS, most = G::MINB * sm_count();
-  return launch_pdl(kern, dim3(ctas < most ? ctas : most), dim3(G::THREADS), G::SMEM, st, true, 0,
-                    a, units, a.err);
-}
-
-// How the lines are spread, by the points of a launch (all instances together):
-//  up to 2^18  small CTAs (512 points at once), as many as possible: latency decides;
-//  up to 2^20  CTAs of 2048 points, output staged in segments of 2048 / L lines;
-//  above       pairs of lines per team, whole 32-byte sectors written from registers without
-//              staging (batches from 2^21: their capacity, which sizes the launch, exceeds the
-//              number of running instances by up to 2).
-// Measured per step of two passes (ms), small | staged | pairs: 256^2 0.0109 | 0.0160 | 0.0239,
-// 512 x 256 0.0121 | 0.0158, 512^2 0.0149 | 0.0154 | 0.0240, 1024 x 256 0.0153 | 0.0172 |
-// 0.0257, 512 x 1024 0.0249 | 0.0193, 1024^2 - | 0.0325 | 0.0291, 512 x 2048 - | 0.0361 |
-// 0.0301, 2048^2 - | 0.138 | 0.085.
-template <int L, bool BATCH, int SIGMA>
-static cudaError_t launch_team_sized(const LinePassArgs<float>& a, cudaStream_t st) {
-  constexpr int SMALL = L >= 512 ? 1 : 512 / L, LPC = L >= 2048 ? 1 : 2048 / L;
-  const size_t points = (size_t)(BATCH ? a.inst_capacity : 1) * a.n_lines * L;
-  if (points >= (BATCH ? kTeamPairPointsBatch : kTeamPairPoints))
-    return launch_team_as<L, LPC, true, BATCH, SIGMA>(a, st);
-  if (points <= ((size_t)1 << 18)) return launch_team_as<L, SMALL, false, BATCH, SIGMA>(a, st);
-  return launch_team_as<L, LPC, false, BATCH, SIGMA>(a, st);
-}
-
-template <int L>
-static cudaError_t launch_team(const LinePassArgs<float>& a, cudaStream_t st) {
-  if (a.inst)
-    return a.sigma == 0 ? launch_team_sized<L, true, 0>(a, st) : launch_team_sized<L, true, 1>(a, st);
-  return a.sigma == 0 ? launch_team_sized<L, false, 0>(a, st) : launch_team_sized<L, false, 1>(a, st);
 }
 
 // The alternative radix schedule (radix_alt), opt 3 the smaller and opt 4 the larger of two

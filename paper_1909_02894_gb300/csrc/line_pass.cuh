@@ -66,6 +66,8 @@ struct LinePassArgs {
   const T* beta_im;     // imaginary part of b - 1 (complex stretching), or nullptr
   const Q4<T>* u_load;  // U applied to psi when it is read, or nullptr
   const Q4<T>* u_store; // U applied to psi_new before the store, or nullptr
+  const Q4<T>* ug_store;  // team pass: a general complex U (two entries per point, see
+                          // apply_u_general) applied before the store, or nullptr
   int* err;             // device error flag (team pass: bounded-wait timeouts)
   const InstPtrs<T>* inst;  // batched launch: per-instance pointers (overrides the above)
   const int* n_inst;        // batched launch: number of active instances (device memory)

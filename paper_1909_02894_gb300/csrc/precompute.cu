@@ -242,10 +242,11 @@ __device__ inline void pauli_exp_general(Z v1, Z v2, Z v3, double phi, Z* d) {
 template <typename T>
 __global__ void k_halfstep_general(const double* a1, const double* a2, const double* meff,
                                    const double* omx, const double* omy, const double* V,
-                                   const double* Ax, const double* Ay, size_t n, double dt,
-                                   Q4<T>* ug, Q4<T>* ug2) {
+                                   const double* Ax, const double* Ay, int nx, int ny,
+                                   double dt, Q4<T>* ug, Q4<T>* ug2, Q4<T>* ug_t, Q4<T>* ug2_t) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= n) return;
+  if (k >= (size_t)nx * ny) return;
+  const size_t row = k / nx, t = (k - row * nx) * ny + row;  // the point's transposed index
   // exponent -i dt/2 [meff sigma_z + F], F = -i sum_j a^j Omega_j sigma_j
   //   - sum_j a^j A_j sigma_j + V I
   const Z v1 = {-0.5 * dt * a1[k] * omx[k], Ax ? 0.5 * dt * a1[k] * Ax[k] : 0.0};
@@ -256,19 +257,27 @@ __global__ void k_halfstep_general(const double* a1, const double* a2, const dou
   pauli_exp_general(v1, v2, v3, phi, d);
   ug[2 * k] = {(T)d[0].r, (T)d[0].i, (T)d[1].r, (T)d[1].i};
   ug[2 * k + 1] = {(T)d[2].r, (T)d[2].i, (T)d[3].r, (T)d[3].i};
+  if (ug_t) {
+    ug_t[2 * t] = ug[2 * k];
+    ug_t[2 * t + 1] = ug[2 * k + 1];
+  }
   pauli_exp_general(zscale(v1, 2.0), zscale(v2, 2.0), zscale(v3, 2.0), 2.0 * phi, d);
   ug2[2 * k] = {(T)d[0].r, (T)d[0].i, (T)d[1].r, (T)d[1].i};
   ug2[2 * k + 1] = {(T)d[2].r, (T)d[2].i, (T)d[3].r, (T)d[3].i};
+  if (ug2_t) {
+    ug2_t[2 * t] = ug2[2 * k];
+    ug2_t[2 * t + 1] = ug2[2 * k + 1];
+  }
 }
 
 template <typename T>
 cudaError_t launch_halfstep_general(const double* a1, const double* a2, const double* meff,
                                     const double* omx, const double* omy, const double* V,
                                     const double* Ax, const double* Ay, int nx, int ny,
-                                    double dt, Q4<T>* ug, Q4<T>* ug2, cudaStream_t st) {
-  const size_t n = (size_t)nx * ny;
-  k_halfstep_general<T><<<nblocks(n), TPB, 0, st>>>(a1, a2, meff, omx, omy, V, Ax, Ay, n, dt,
-                                                    ug, ug2);
+                                    double dt, Q4<T>* ug, Q4<T>* ug2, Q4<T>* ug_t, Q4<T>* ug2_t,
+                                    cudaStream_t st) {
+  k_halfstep_general<T><<<nblocks((size_t)nx * ny), TPB, 0, st>>>(
+      a1, a2, meff, omx, omy, V, Ax, Ay, nx, ny, dt, ug, ug2, ug_t, ug2_t);
   return cudaGetLastError();
 }
 
@@ -448,7 +457,7 @@ cudaError_t launch_transpose(const Q4<T>* in, Q4<T>* out, int rows, int cols, cu
   template cudaError_t launch_halfstep_general<T>(                                            \
       const double*, const double*, const double*, const double*, const double*,             \
       const double*, const double*, const double*, int, int, double, Q4<T>*, Q4<T>*,         \
-      cudaStream_t);                                                                         \
+      Q4<T>*, Q4<T>*, cudaStream_t);                                                         \
   template cudaError_t launch_twiddles<T>(int, int, Cx<T>*, cudaStream_t);                    \
   template cudaError_t launch_step_mult<T>(int, double, double, Q4<T>*, cudaStream_t);        \
   template cudaError_t launch_team_perm<T>(int, const Q4<T>*, Q4<T>*, cudaStream_t);          \

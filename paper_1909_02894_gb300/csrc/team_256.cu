@@ -1,0 +1,8 @@
+// Radix-16 team passes over 256-point lines.
+#include "team_launch.cuh"
+
+namespace dgb {
+template cudaError_t launch_team<256>(const LinePassArgs<float>&, cudaStream_t);
+template cudaError_t launch_team_unsplit<256>(const UnsplitArgs&, int, cudaStream_t);
+int dgb_debug_flag_team_256() { return dgb_take_debug_flag(); }
+}  // namespace dgb

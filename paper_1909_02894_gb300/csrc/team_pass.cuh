@@ -110,6 +110,14 @@ __device__ __forceinline__ float ld_stream(const float* p) {
   asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
   return v;
 }
+// A pointer of a batched instance, loaded where it is used (a volatile load is not kept in
+// registers across the transforms, which have none to spare).
+template <typename P>
+__device__ __forceinline__ P* ld_ptr(P* const* p) {
+  unsigned long long v;
+  asm volatile("ld.global.nc.u64 %0, [%1];" : "=l"(v) : "l"(p));
+  return reinterpret_cast<P*>(v);
+}
 // 32 bytes (two adjacent points) in one store, without a place in L1
 __device__ __forceinline__ void st_points2(Q4<float>* dst, const float* a, const float* b) {
   asm volatile("st.global.L1::no_allocate.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(a[0]),
@@ -269,11 +277,23 @@ __device__ __forceinline__ void team_transform(Cx<float> (&vp)[16], Cx<float> (&
   }
 }
 
-template <int L, int LPC, bool PAIR, bool BATCH, int SIGMA>
+// What a step pass does with its results. Kinds and sigma are template parameters since the
+// kernel's speed depends on its code size (the branches of one general kernel, taken or not,
+// cost 4..6 % in instruction-cache misses at 1024^2 and 4096^2).
+enum TeamOut {
+  TEAM_PLAIN = 0,  // transposed store, no U (x passes; sigma_x: U on load if u_load is set)
+  TEAM_U = 1,      // transposed store after U (y passes; batches: if the instance has one)
+  TEAM_UG = 2,     // transposed store after a general U (static potentials)
+  TEAM_ROWS = 3    // rows back in the input's layout, after U or a general U if set
+};
+
+template <int L, int LPC, bool PAIR, bool BATCH, int SIGMA, int OUT>
 __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR>::MINB)
     line_pass_team(const LinePassArgs<float> a0, int n_units, int* __restrict__ err) {
   using G = TGeo<L, LPC, PAIR>;
   constexpr int T = G::T, R2 = G::R2, BS = G::BS;
+  constexpr bool U_OUT = OUT == TEAM_U || OUT == TEAM_ROWS;
+  constexpr bool UG_OUT = OUT == TEAM_UG || OUT == TEAM_ROWS;
   extern __shared__ __align__(128) unsigned char tsm[];
   const int tid = threadIdx.x, warp = tid >> 5;
   const int lt = tid / T, j = tid - lt * T;
@@ -339,21 +359,21 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
   uint32_t par = 0;
   int h = 0;
   while (unit < n_units) {
-    LinePassArgs<float> a = a0;
-    int ul = unit;
-    if constexpr (BATCH) {
-      bind_instance(a, unit / upi);
-      ul = unit % upi;
-    }
+    const InstPtrs<float>* ip = BATCH ? a0.inst + unit / upi : nullptr;  // the unit's instance
+    const int ul = BATCH ? unit % upi : unit;
     const int line = ul * G::LPU + (PAIR ? 2 * lg + h : lg);
     const size_t row = (size_t)line * L;
     Cx<float> vp[16], vm[16];
     const bool ok = mbar_wait_bounded(bar, par, kWaitNs);
     par ^= 1u;
-    if (a.u_load) {  // first pass of a call: U applied to the landed points in place
+    if constexpr (SIGMA == 0 && OUT == TEAM_PLAIN) {
+      const Q4<float>* u_load = BATCH ? ld_ptr(&ip->u_load) : a0.u_load;
+      if (u_load) {  // first pass of a call: U applied to the landed points in place
 #pragma unroll 4
-      for (int m = 0; m < 16; ++m)
-        land[lz(j + T * m)] = apply_u(ld_stream_q4(a.u_load + gz(row + j + T * m)), land[lz(j + T * m)]);
+        for (int m = 0; m < 16; ++m)
+          land[lz(j + T * m)] =
+              apply_u(ld_stream_q4(u_load + gz(row + j + T * m)), land[lz(j + T * m)]);
+      }
     }
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
@@ -376,11 +396,19 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
       }
       tmem_st16(tpark + (uint32_t)((PAIR ? 64 * h : 0) + 16 * g), pk);
     }
-    team_transform<L, LPC, false>(vp, vm, xp, blk, a.tw + j, tw2s + u, a.mult_perm + j, lt, j, u, [&]() {
+    const Q4<float>* mult = BATCH ? ld_ptr(&ip->mult_perm) : a0.mult_perm;
+    team_transform<L, LPC, false>(vp, vm, xp, blk, a0.tw + j, tw2s + u, mult + j, lt, j, u, [&]() {
       // the line's coefficients into L2, a line's transforms ahead of their use (bulk
       // prefetches queue with the landing copies and were slower)
-      if (a.u_store) team_prefetch<L>(a.u_store + row, j);
-      if (a.beta) team_prefetch<L>(a.beta + row, j);
+      team_prefetch<L>((BATCH ? ld_ptr(&ip->beta) : a0.beta) + row, j);
+      if constexpr (U_OUT) {
+        const Q4<float>* us = BATCH ? ld_ptr(&ip->u_store) : a0.u_store;
+        if (us) team_prefetch<L>(us + row, j);
+      }
+      if (UG_OUT && a0.ug_store) {
+        team_prefetch<L>(a0.ug_store + 2 * row, j);
+        team_prefetch<L>(a0.ug_store + 2 * row + L, j);
+      }
     });
     // the exchange buffer is free: the next rows may land in it
     if (!ok) *bad = 1;
@@ -400,35 +428,27 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
     dft16<float, true, false>(vm);
     tmem_wait_st();
     // ---- epilogue: psi + D + (b - 1) D, U; coefficients in batches of four points
-    float bn[4];
-    Q4<float> un[4];
-    auto coeffs = [&](int g) {
-      const size_t g0 = row + j + T * 4 * g;
-#pragma unroll
-      for (int mm = 0; mm < 4; ++mm) bn[mm] = 0.f;
-      if (a.beta) {
-#pragma unroll
-        for (int mm = 0; mm < 4; ++mm) bn[mm] = ld_stream(a.beta + gz(g0 + T * mm));
-      }
-      if (a.u_store) {
-#pragma unroll
-        for (int mm = 0; mm < 4; ++mm) un[mm] = ld_stream_q4(a.u_store + gz(g0 + T * mm));
-      }
-    };
+    const float* beta = BATCH ? ld_ptr(&ip->beta) : a0.beta;
+    const Q4<float>* u_store = !U_OUT ? nullptr : BATCH ? ld_ptr(&ip->u_store) : a0.u_store;
+    Q4<float>* out = BATCH ? ld_ptr(&ip->out) : a0.out;
+    const bool has_u = U_OUT && ((!BATCH && OUT == TEAM_U) || u_store != nullptr);
     // transposed store of the pair: row j + T m of the output (the opaque step keeps the
     // compiler from holding sixteen row offsets across the loop)
-    size_t dstep = (size_t)T * a.n_lines;
+    size_t dstep = (size_t)T * a0.n_lines;
     asm volatile("" : "+l"(dstep));
-    Q4<float>* dst = a.out + (size_t)j * a.n_lines + (line - 1);
+    Q4<float>* dst = out + (size_t)j * a0.n_lines + (line - 1);
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-      coeffs(g);
+      const size_t g0 = row + j + T * 4 * g;
       float pk[16], bc[4];
       Q4<float> uc[4];
 #pragma unroll
-      for (int mm = 0; mm < 4; ++mm) {
-        bc[mm] = bn[mm];
-        uc[mm] = un[mm];
+      for (int mm = 0; mm < 4; ++mm) bc[mm] = ld_stream(beta + gz(g0 + T * mm));
+      if constexpr (U_OUT) {
+        if (has_u) {
+#pragma unroll
+          for (int mm = 0; mm < 4; ++mm) uc[mm] = ld_stream_q4(u_store + gz(g0 + T * mm));
+        }
       }
       tmem_ld16(tpark + (uint32_t)((PAIR ? 64 * h : 0) + 16 * g), pk);
       tmem_wait_ld_regs(pk);
@@ -450,43 +470,56 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
         pk[4 * mm + 2] = o2.re;
         pk[4 * mm + 3] = o2.im;
       }
-      if (a.u_store) {
+      if constexpr (U_OUT) {
+        if (has_u) {
 #pragma unroll
-        for (int mm = 0; mm < 4; ++mm) {
-          const Q4<float> o =
-              apply_u(uc[mm], Q4<float>{pk[4 * mm], pk[4 * mm + 1], pk[4 * mm + 2], pk[4 * mm + 3]});
-          pk[4 * mm] = o.x;
-          pk[4 * mm + 1] = o.y;
-          pk[4 * mm + 2] = o.z;
-          pk[4 * mm + 3] = o.w;
+          for (int mm = 0; mm < 4; ++mm) {
+            const Q4<float> o =
+                apply_u(uc[mm], Q4<float>{pk[4 * mm], pk[4 * mm + 1], pk[4 * mm + 2], pk[4 * mm + 3]});
+            pk[4 * mm] = o.x;
+            pk[4 * mm + 1] = o.y;
+            pk[4 * mm + 2] = o.z;
+            pk[4 * mm + 3] = o.w;
+          }
         }
       }
-      if (a.store_normal) {
+      if constexpr (UG_OUT) {
+        if (OUT == TEAM_UG || a0.ug_store) {  // static potentials
+#pragma unroll
+          for (int mm = 0; mm < 4; ++mm) {
+            const Q4<float>* ug = a0.ug_store + 2 * gz(g0 + T * mm);
+            const Q4<float> o = apply_u_general(
+                ld_stream_q4(ug), ld_stream_q4(ug + 1),
+                Q4<float>{pk[4 * mm], pk[4 * mm + 1], pk[4 * mm + 2], pk[4 * mm + 3]});
+            pk[4 * mm] = o.x;
+            pk[4 * mm + 1] = o.y;
+            pk[4 * mm + 2] = o.z;
+            pk[4 * mm + 3] = o.w;
+          }
+        }
+      }
+      if constexpr (OUT == TEAM_ROWS) {
 #pragma unroll
         for (int mm = 0; mm < 4; ++mm)
-          a.out[gz(row + j + T * (4 * g + mm))] = {pk[4 * mm], pk[4 * mm + 1], pk[4 * mm + 2],
-                                               pk[4 * mm + 3]};
+          out[gz(g0 + T * mm)] = {pk[4 * mm], pk[4 * mm + 1], pk[4 * mm + 2], pk[4 * mm + 3]};
       } else if constexpr (!PAIR) {
 #pragma unroll
         for (int mm = 0; mm < 4; ++mm)
           reinterpret_cast<Q4<float>*>(tsm)[sz(lt * G::SPITCH + j + T * (4 * g + mm))] = {
               pk[4 * mm], pk[4 * mm + 1], pk[4 * mm + 2], pk[4 * mm + 3]};
       }
-      if constexpr (PAIR) {
-        if (!a.store_normal) {
-          if (h == 0) {
-            tmem_st16(tpark + (uint32_t)(16 * g), pk);
-          } else {
-            float pa[16];
-            tmem_ld16(tpark + (uint32_t)(16 * g), pa);
-            tmem_wait_ld_regs(pa);
+      if constexpr (PAIR && OUT != TEAM_ROWS) {
+        if (h == 0) {
+          tmem_st16(tpark + (uint32_t)(16 * g), pk);
+        } else {
+          float pa[16];
+          tmem_ld16(tpark + (uint32_t)(16 * g), pa);
+          tmem_wait_ld_regs(pa);
 #pragma unroll
-            for (int mm = 0; mm < 4; ++mm)
-            {
-              if (dbg_in((size_t)(dst - a.out) + 1, (size_t)a0.n_lines * L))
-                st_points2(dst, pa + 4 * mm, pk + 4 * mm);
-              dst += dstep;
-            }
+          for (int mm = 0; mm < 4; ++mm) {
+            if (dbg_in((size_t)(dst - out) + 1, (size_t)a0.n_lines * L))
+              st_points2(dst, pa + 4 * mm, pk + 4 * mm);
+            dst += dstep;
           }
         }
       }
@@ -500,15 +533,15 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
       }
     } else {
       __syncthreads();
-      if (!a.store_normal) {
+      if constexpr (OUT != TEAM_ROWS) {
         const Q4<float>* st = reinterpret_cast<const Q4<float>*>(tsm);
         const int g = tid % LPC, i0 = tid / LPC;
-        Q4<float>* dst = a.out + (size_t)i0 * a.n_lines + (ul * G::LPU + g);
+        Q4<float>* dst = out + (size_t)i0 * a0.n_lines + (ul * G::LPU + g);
         constexpr int RPI = G::THREADS / LPC;
 #pragma unroll
         for (int q = 0; q < 16; ++q)
-          if (dbg_in((size_t)(i0 + q * RPI) * a.n_lines + ul * G::LPU + g, (size_t)a0.n_lines * L))
-            dst[(size_t)(q * RPI) * a.n_lines] = st[sz(g * G::SPITCH + i0 + q * RPI)];
+          if (dbg_in((size_t)(i0 + q * RPI) * a0.n_lines + ul * G::LPU + g, (size_t)a0.n_lines * L))
+            dst[(size_t)(q * RPI) * a0.n_lines] = st[sz(g * G::SPITCH + i0 + q * RPI)];
         __syncthreads();
       }
       unit = next;

@@ -28,13 +28,7 @@ template <typename T>
 __global__ void k_apply_ug(Q4<T>* psi, const Q4<T>* ug, size_t n) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
-  const Q4<T> p = psi[k], r0 = ug[2 * k], r1 = ug[2 * k + 1];
-  // row 0: d00 psi1 + u01 psi2; row 1: u10 psi1 + d11 psi2 (complex), added to psi
-  const T a = p.x, b = p.y, c = p.z, d = p.w;
-  psi[k] = {a + (r0.x * a - r0.y * b + r0.z * c - r0.w * d),
-            b + (r0.x * b + r0.y * a + r0.z * d + r0.w * c),
-            c + (r1.x * a - r1.y * b + r1.z * c - r1.w * d),
-            d + (r1.x * b + r1.y * a + r1.z * d + r1.w * c)};
+  psi[k] = apply_u_general(ug[2 * k], ug[2 * k + 1], psi[k]);
 }
 
 // S = b1 sigma_x dx + b2 sigma_y dy with sigma_x (u, v) = (v, u), sigma_y (u, v) =
@@ -417,6 +411,18 @@ cudaError_t launch_max_b(const double* a1, const double* a2, const double* sxinv
                          int nx, int ny, double* partials, int n_blocks, cudaStream_t st) {
   k_max_b<<<n_blocks, TPB, 0, st>>>(a1, a2, sxinv, syinv, sxinv_im, syinv_im, nx, ny, partials);
   return cudaGetLastError();
+}
+
+cudaError_t launch_unsplit(const UnsplitArgs& a, int L, int phase, cudaStream_t st) {
+  if (phase != 1 && phase != 2) return cudaErrorInvalidValue;
+  switch (L) {
+    case 256: return launch_team_unsplit<256>(a, phase, st);
+    case 512: return launch_team_unsplit<512>(a, phase, st);
+    case 1024: return launch_team_unsplit<1024>(a, phase, st);
+    case 2048: return launch_team_unsplit<2048>(a, phase, st);
+    case 4096: return launch_team_unsplit<4096>(a, phase, st);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 // Bessel functions J_0(x) .. J_n(x), x >= 0, by downward recurrence from an order well
