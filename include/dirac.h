@@ -207,13 +207,15 @@ long dirac_krylov_iterations(const dirac_ctx *ctx);
  * shared memory while the current ones are finished); 0 = the default (complex64: the team
  * pass for lines of 256 points or more, the smaller shape for 128-point lines, else the
  * larger; complex128: the smaller shape for 1024-point lines and lines of 128 points or
- * fewer, else the larger). 64- and 128-point lines take
- * 2 or 16 lines per CTA; lines of 32 points or fewer and 4096-point lines have one shape
- * only. 256 or 512 plus
+ * fewer, else the larger; 512-point lines the smaller when there are fewer than 512). The
+ * smaller shape of lines of 128 points or fewer gives each thread 2 (up to 512 lines) or 4
+ * points, the larger takes 16 lines per CTA; 4096-point lines have one shape besides the team
+ * pass. 256 or 512 plus
  * DIRAC_LAUNCH_ALT_RADIX selects the other radix schedule of the FFT passes, where the line
  * length has one: complex64 lines of 256..4096 points in radix-16 instead of radix-8
- * passes, complex128 lines of 256..2048 points in radix-8 instead of radix-16 passes, each
- * with its own lines-per-CTA pair (about 256 | 512 threads); elsewhere the flag is ignored.
+ * passes, complex128 lines of 512..2048 points in radix-8 instead of radix-16 passes (256
+ * points: radix 16 instead of 8), each with its own lines-per-CTA pair (about 256 | 512
+ * threads); elsewhere the flag is ignored.
  * Used by the autotuner. DIRAC_EINVAL for other values. */
 #define DIRAC_LAUNCH_ALT_RADIX 0x10000
 dirac_status dirac_set_launch(dirac_ctx *ctx, int threads_x_pass, int threads_y_pass);
@@ -253,7 +255,9 @@ size_t dirac_footprint_bytes(const dirac_grid *grid, dirac_precision precision);
  * CUDA graph captured once per class layout and replayed. (The environment variable
  * DIRAC_BATCH_TICK of earlier versions, one slower launch per tick with the same results, has
  * no effect.) Each context computes
- * exactly what dirac_step(ctx, n_steps, dt) computes (Sec. 5.2 Scheme II); a submitted
+ * exactly what dirac_step(ctx, n_steps, dt) computes (Sec. 5.2 Scheme II; bit for bit with the
+ * class's CTA shapes, see dirac_batch_launch_shape, which differ from a lone context's default
+ * only for lines of 128 points or fewer and some complex128 lengths); a submitted
  * context belongs to the batch until it is released and must not be stepped, read or
  * destroyed meanwhile. Contexts must have the batch's precision. */
 

@@ -45,6 +45,8 @@ struct Class {
   void* tw_y = nullptr;
   void* tw_x_alt = nullptr;  // the same for the alternative radix schedule (if any)
   void* tw_y_alt = nullptr;
+  void* tw_x_small = nullptr;  // twiddles of the small shape (lines of 128 points or fewer)
+  void* tw_y_small = nullptr;
   void* tw_x_team = nullptr;  // twiddles of the team pass (complex64)
   void* tw_y_team = nullptr;
   int opt[2] = {-1, -1};  // CTA shape of the x / y pass chosen by the autotuner (-1: default)
@@ -116,6 +118,8 @@ static void free_class(Class& c) {
   if (c.tw_y) cudaFree(c.tw_y);
   if (c.tw_x_alt) cudaFree(c.tw_x_alt);
   if (c.tw_y_alt) cudaFree(c.tw_y_alt);
+  if (c.tw_x_small) cudaFree(c.tw_x_small);
+  if (c.tw_y_small) cudaFree(c.tw_y_small);
   if (c.tw_x_team) cudaFree(c.tw_x_team);
   if (c.tw_y_team) cudaFree(c.tw_y_team);
   c = Class();
@@ -222,6 +226,7 @@ static dirac_status launch_class_step(dirac_batch* b, Class& c, int k, cudaStrea
     a.sigma = pass;
     a.tw = (const Cx<T>*)(pass == 0 ? c.tw_x : c.tw_y);
     a.tw_alt = (const Cx<T>*)(pass == 0 ? c.tw_x_alt : c.tw_y_alt);
+    a.tw_small = (const Cx<T>*)(pass == 0 ? c.tw_x_small : c.tw_y_small);
     a.tw_team = (const Cx<T>*)(pass == 0 ? c.tw_x_team : c.tw_y_team);
     a.err = b->d_err;
     a.inst = (const InstPtrs<T>*)c.d_tab + ((size_t)k * 2 + pass) * c.capacity;
@@ -356,12 +361,11 @@ static dirac_status run_tick(dirac_batch* b, int K) {
 }
 
 // Shapes worth timing for a pass over lines of L points (the launcher maps the others onto
-// these): complex64 256..4096 points also the team pass; lines of 32 points or
-// fewer and 4096-point lines have one non-persistent shape.
+// these): complex64 256..4096 points also the team pass; 4096-point lines have one shape else.
 template <typename T>
 static std::vector<int> shape_candidates(int L) {
   std::vector<int> o;
-  if (L >= 64 && L < 4096) o.push_back(0);
+  if (L < 4096) o.push_back(0);
   o.push_back(1);
   if (sizeof(T) == 4 && L >= 256) o.push_back(2);
   if (line_pass_radix_alt<T>(L)) {  // the other radix schedule (3 smaller, 4 larger CTA)
@@ -423,6 +427,7 @@ static dirac_status autotune_class(dirac_batch* b, Class& c, int reps, bool* cha
     a.sigma = pass;
     a.tw = (const Cx<T>*)(pass == 0 ? c.tw_x : c.tw_y);
     a.tw_alt = (const Cx<T>*)(pass == 0 ? c.tw_x_alt : c.tw_y_alt);
+    a.tw_small = (const Cx<T>*)(pass == 0 ? c.tw_x_small : c.tw_y_small);
     a.tw_team = (const Cx<T>*)(pass == 0 ? c.tw_x_team : c.tw_y_team);
     a.err = b->d_err;
     a.inst = d_tab + (size_t)pass * n;
@@ -560,6 +565,17 @@ dirac_status dirac_batch_submit(dirac_batch* b, dirac_ctx* inst, long n_steps, d
     } else {
       if (ax) BCK(launch_twiddles<double>(c.nx, ax, (Cx<double>*)c.tw_x_alt, b->stream), "twiddles");
       if (ay) BCK(launch_twiddles<double>(c.ny, ay, (Cx<double>*)c.tw_y_alt, b->stream), "twiddles");
+    }
+    const int sx = line_pass_radix_small<float>(c.nx, c.ny);  // the same in both precisions
+    const int sy = line_pass_radix_small<float>(c.ny, c.nx);
+    if (sx) BCK(cudaMalloc(&c.tw_x_small, c.nx * cx), "class twiddles");
+    if (sy) BCK(cudaMalloc(&c.tw_y_small, c.ny * cx), "class twiddles");
+    if (b->prec == DIRAC_C64) {
+      if (sx) BCK(launch_twiddles<float>(c.nx, sx, (Cx<float>*)c.tw_x_small, b->stream), "twiddles");
+      if (sy) BCK(launch_twiddles<float>(c.ny, sy, (Cx<float>*)c.tw_y_small, b->stream), "twiddles");
+    } else {
+      if (sx) BCK(launch_twiddles<double>(c.nx, sx, (Cx<double>*)c.tw_x_small, b->stream), "twiddles");
+      if (sy) BCK(launch_twiddles<double>(c.ny, sy, (Cx<double>*)c.tw_y_small, b->stream), "twiddles");
     }
     if (b->prec == DIRAC_C64 && team_length(c.nx)) {
       BCK(cudaMalloc(&c.tw_x_team, c.nx * cx), "class twiddles");

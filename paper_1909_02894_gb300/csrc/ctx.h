@@ -32,6 +32,7 @@ struct dirac_ctx {
   void *beta1_im = nullptr, *beta2T_im = nullptr;  // complex stretching: Im(b - 1)
   void *u_n = nullptr, *u_t = nullptr, *u2_t = nullptr;
   void *tw_x_alt = nullptr, *tw_y_alt = nullptr;  // twiddles of the alternative radix
+  void *tw_x_small = nullptr, *tw_y_small = nullptr;  // of the small shape (<= 128 points)
   void *tw_x_team = nullptr, *tw_y_team = nullptr;  // twiddles of the team pass (complex64)
   void *tw_x = nullptr, *tw_y = nullptr, *mult_x = nullptr, *mult_y = nullptr,
        *dmult_x = nullptr, *dmult_y = nullptr;
@@ -84,5 +85,3 @@ struct dirac_ctx {
 // Library-internal helpers implemented in dirac_api.cu.
 dirac_status dgb_tables_for_dt(dirac_ctx* ctx, double dt);
 size_t dgb_footprint_bytes(int nx, int ny, dirac_precision prec);
-// Launch option (0, 1, 2 = team pass) for a pass of line length L.
-int dgb_pass_opt(const dirac_ctx* ctx, int threads, int L);

@@ -10,6 +10,7 @@
 #include <cstring>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "../../include/dirac.h"
@@ -78,7 +79,7 @@ static void free_all(dirac_ctx* ctx) {
 
 // ------------------------------------------------------------------ precision dispatch
 // launch option for a pass from the dirac_set_launch preference (0 = default)
-static int pass_opt(const dirac_ctx* ctx, int shape, int L) {
+static int pass_opt(const dirac_ctx* ctx, int shape, int L, int n_lines) {
   if (shape & DIRAC_LAUNCH_ALT_RADIX) {  // validated by dirac_set_launch
     const int threads = shape & ~DIRAC_LAUNCH_ALT_RADIX;
     if (ctx->prec == DIRAC_C64 ? line_pass_radix_alt<float>(L) : line_pass_radix_alt<double>(L))
@@ -90,13 +91,13 @@ static int pass_opt(const dirac_ctx* ctx, int shape, int L) {
   if (threads == 512) return 1;
   if (threads == 1024) return 2;
   // Default, by measurement: complex64 the team pass for lines of 256 points or more (256^2
-  // 0.0109 against 0.0118 ms per step for the radix-8 pass, 1024^2 0.0291 against 0.039), the
-  // smaller shape for 128-point lines (0.0166 against 0.0187 per 128^2), else the larger;
-  // complex128 the smaller shape for 1024-point lines (one line per CTA: 1024 CTAs spread
-  // over the SMs to within one line, 0.74 against 0.89 ms per 1024^2 step) and for lines of
-  // 128 points or fewer (0.050 against 0.168 ms per 128^2 step), else the larger.
-  if (ctx->prec == DIRAC_C64) return L >= 256 ? 2 : L == 128 ? 0 : 1;
-  return (L == 1024 || L <= 128) ? 0 : 1;
+  // 0.0109 against 0.0118 ms per step for the radix-8 pass, 1024^2 0.0282 against 0.039); the
+  // smaller shape for lines of 128 points or fewer and, in complex128, for 1024-point lines (one
+  // line per CTA: 1024 CTAs spread over the SMs to within one line, 0.74 against 0.89 ms per
+  // 1024^2 step) and fewer than 512 lines of 512 points (512 x 256: 0.104 against 0.165 ms per
+  // step); else the larger.
+  if (ctx->prec == DIRAC_C64) return L >= 256 ? 2 : 0;
+  return (L == 1024 || L <= 128 || (L == 512 && n_lines < 512)) ? 0 : 1;
 }
 
 // Reads and clears the device error flag (after the stream has been synchronised).
@@ -122,6 +123,7 @@ static LinePassArgs<T> pass_args(dirac_ctx* ctx, int axis) {
   a.sigma = axis;
   a.tw = (const Cx<T>*)(axis == 0 ? ctx->tw_x : ctx->tw_y);
   a.tw_alt = (const Cx<T>*)(axis == 0 ? ctx->tw_x_alt : ctx->tw_y_alt);
+  a.tw_small = (const Cx<T>*)(axis == 0 ? ctx->tw_x_small : ctx->tw_y_small);
   a.tw_team = (const Cx<T>*)(axis == 0 ? ctx->tw_x_team : ctx->tw_y_team);
   return a;
 }
@@ -223,8 +225,8 @@ static dirac_status step_symmetric(dirac_ctx* ctx, long n) {
   ctx->test_timeout_next = 0;
   void* cur = ctx->psi;
   void* oth = ctx->psiT;
-  const int opt_x = pass_opt(ctx, ctx->threads_x, ctx->nx);
-  const int opt_y = pass_opt(ctx, ctx->threads_y, ctx->ny);
+  const int opt_x = pass_opt(ctx, ctx->threads_x, ctx->nx, ctx->ny);
+  const int opt_y = pass_opt(ctx, ctx->threads_y, ctx->ny, ctx->nx);
   // potentials: as in step_impl, the later U in the last x pass's row store
   const bool fused = !ctx->has_pot;
   const bool fused_pot = !fused && sizeof(T) == 4 && opt_x == 2 && team_length(ctx->nx);
@@ -678,13 +680,13 @@ static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
   // potentials: the leading U by its own kernel, the later ones in the y pass's store where
   // that is a team pass, else by their own kernel too
   const bool fused = !ctx->has_pot;
-  const int opt_y = pass_opt(ctx, ctx->threads_y, ctx->ny);
+  const int opt_y = pass_opt(ctx, ctx->threads_y, ctx->ny, ctx->nx);
   const bool fused_pot = !fused && sizeof(T) == 4 && opt_y == 2 && team_length(ctx->ny);
   if (!fused) CKS(apply_half<T>(ctx, ctx->psi, false));
   for (long s = 0; s < n; ++s) {
     ax.u_load = (fused && s == 0 && !ctx->u_identity) ? (const Q4<T>*)ctx->u_n : nullptr;
     ax.u_store = nullptr;
-    CK(launch_line_pass<T>(ax, MODE_STEP, pass_opt(ctx, ctx->threads_x, ctx->nx), ctx->stream),
+    CK(launch_line_pass<T>(ax, MODE_STEP, pass_opt(ctx, ctx->threads_x, ctx->nx, ctx->ny), ctx->stream),
        "x pass");
     ay.u_load = nullptr;
     ay.u_store = (!fused || ctx->u_identity) ? nullptr
@@ -771,14 +773,8 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
   // FP64 fields
   double** f64[] = {&ctx->a1, &ctx->a2, &ctx->meff, &ctx->w, &ctx->omx, &ctx->omy};
   for (double** p : f64) CK(dalloc(ctx, (void**)p, n * sizeof(double)), "allocate fields");
-  CK(dalloc(ctx, (void**)&ctx->sxinv, nx * sizeof(double)), "allocate layer");
-  CK(dalloc(ctx, (void**)&ctx->syinv, ny * sizeof(double)), "allocate layer");
   const bool complex_layer =
       ctx->abs.theta != 0.0 && (ctx->abs.width_x > 0 || ctx->abs.width_y > 0);
-  if (complex_layer) {
-    CK(dalloc(ctx, (void**)&ctx->sxinv_im, nx * sizeof(double)), "allocate layer");
-    CK(dalloc(ctx, (void**)&ctx->syinv_im, ny * sizeof(double)), "allocate layer");
-  }
   // state, coefficient fields, tables
   CK(dalloc(ctx, &ctx->psi, n * sizeof(Q4<T>)), "allocate state");
   CK(dalloc(ctx, &ctx->psiT, n * sizeof(Q4<T>)), "allocate state");
@@ -793,32 +789,48 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
     CK(dalloc(ctx, &ctx->u_t, n * sizeof(Q4<T>)), "allocate half-step");
     CK(dalloc(ctx, &ctx->u2_t, n * sizeof(Q4<T>)), "allocate half-step");
   }
-  CK(dalloc(ctx, &ctx->tw_x, nx * sizeof(Cx<T>)), "allocate tables");
-  CK(dalloc(ctx, &ctx->tw_y, ny * sizeof(Cx<T>)), "allocate tables");
-  if (line_pass_radix_alt<T>(nx))
-    CK(dalloc(ctx, &ctx->tw_x_alt, nx * sizeof(Cx<T>)), "allocate tables");
-  if (line_pass_radix_alt<T>(ny))
-    CK(dalloc(ctx, &ctx->tw_y_alt, ny * sizeof(Cx<T>)), "allocate tables");
-  CK(dalloc(ctx, &ctx->mult_x, nx * sizeof(Q4<T>)), "allocate tables");
-  CK(dalloc(ctx, &ctx->mult_y, ny * sizeof(Q4<T>)), "allocate tables");
-  if (sizeof(T) == 4 && team_length(nx)) {  // the team pass's table order and twiddles
-    CK(dalloc(ctx, &ctx->mult_px, nx * sizeof(Q4<T>)), "allocate tables");
-    CK(dalloc(ctx, &ctx->tw_x_team, nx * sizeof(Cx<T>)), "allocate tables");
+  // the per-axis tables and small buffers share one allocation (each cudaMalloc costs as much as
+  // several of the kernels that fill them)
+  std::vector<std::pair<void**, size_t>> small;
+  auto table = [&](void* p, size_t bytes) { small.push_back({(void**)p, bytes}); };
+  table(&ctx->sxinv, nx * sizeof(double));
+  table(&ctx->syinv, ny * sizeof(double));
+  if (complex_layer) {
+    table(&ctx->sxinv_im, nx * sizeof(double));
+    table(&ctx->syinv_im, ny * sizeof(double));
+  }
+  table(&ctx->tw_x, nx * sizeof(Cx<T>));
+  table(&ctx->tw_y, ny * sizeof(Cx<T>));
+  if (line_pass_radix_alt<T>(nx)) table(&ctx->tw_x_alt, nx * sizeof(Cx<T>));
+  if (line_pass_radix_alt<T>(ny)) table(&ctx->tw_y_alt, ny * sizeof(Cx<T>));
+  if (line_pass_radix_small<T>(nx, ny)) table(&ctx->tw_x_small, nx * sizeof(Cx<T>));
+  if (line_pass_radix_small<T>(ny, nx)) table(&ctx->tw_y_small, ny * sizeof(Cx<T>));
+  table(&ctx->mult_x, nx * sizeof(Q4<T>));
+  table(&ctx->mult_y, ny * sizeof(Q4<T>));
+  table(&ctx->dmult_x, nx * sizeof(Q4<T>));
+  table(&ctx->dmult_y, ny * sizeof(Q4<T>));
+  if (sizeof(T) == 4 && team_length(nx)) {  // the team pass's table orders and twiddles
+    table(&ctx->mult_px, nx * sizeof(Q4<T>));
+    table(&ctx->dmult_px, nx * sizeof(Q4<T>));
+    table(&ctx->tw_x_team, nx * sizeof(Cx<T>));
   }
   if (sizeof(T) == 4 && team_length(ny)) {
-    CK(dalloc(ctx, &ctx->mult_py, ny * sizeof(Q4<T>)), "allocate tables");
-    CK(dalloc(ctx, &ctx->tw_y_team, ny * sizeof(Cx<T>)), "allocate tables");
+    table(&ctx->mult_py, ny * sizeof(Q4<T>));
+    table(&ctx->dmult_py, ny * sizeof(Q4<T>));
+    table(&ctx->tw_y_team, ny * sizeof(Cx<T>));
   }
-  if (ctx->tw_x_team)
-    CK(dalloc(ctx, &ctx->dmult_px, nx * sizeof(Q4<T>)), "allocate tables");
-  if (ctx->tw_y_team)
-    CK(dalloc(ctx, &ctx->dmult_py, ny * sizeof(Q4<T>)), "allocate tables");
-  CK(dalloc(ctx, &ctx->dmult_x, nx * sizeof(Q4<T>)), "allocate tables");
-  CK(dalloc(ctx, &ctx->dmult_y, ny * sizeof(Q4<T>)), "allocate tables");
+  table(&ctx->partials, 4 * sizeof(double) * observables_blocks(n));
+  table(&ctx->result, 4 * sizeof(double));
+  table(&ctx->d_err, sizeof(int));
+  size_t total = 0;
+  for (auto& t : small) total += (t.second + 255) / 256 * 256;
+  unsigned char* arena = nullptr;
+  CK(dalloc(ctx, (void**)&arena, total), "allocate tables");
+  for (auto& t : small) {
+    *t.first = arena;
+    arena += (t.second + 255) / 256 * 256;
+  }
   CK(dalloc(ctx, (void**)&ctx->staging, 2 * n * 2 * sizeof(double)), "allocate staging");
-  CK(dalloc(ctx, (void**)&ctx->partials, 4 * sizeof(double) * observables_blocks(n)), "allocate");
-  CK(dalloc(ctx, (void**)&ctx->result, 4 * sizeof(double)), "allocate");
-  CK(dalloc(ctx, (void**)&ctx->d_err, sizeof(int)), "allocate");
   CK(cudaMemsetAsync(ctx->d_err, 0, sizeof(int), st), "clear error flag");
 
   // metric upload: the staging buffer holds the three fields during creation
@@ -850,17 +862,20 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
     CK(cudaMallocAsync(&ty, ny * sizeof(Cx<double>), st), "allocate");
     CK(cudaMallocAsync(&mx, nx * sizeof(Q4<double>), st), "allocate");
     CK(cudaMallocAsync(&my, ny * sizeof(Q4<double>), st), "allocate");
-    CK(launch_twiddles<double>(nx, line_pass_radix<double>(nx), (Cx<double>*)tx, st), "twiddles");
-    CK(launch_twiddles<double>(ny, line_pass_radix<double>(ny), (Cx<double>*)ty, st), "twiddles");
+    const int sx = line_pass_radix_small<double>(nx, ny), sy = line_pass_radix_small<double>(ny, nx);
+    CK(launch_twiddles<double>(nx, sx ? sx : line_pass_radix<double>(nx), (Cx<double>*)tx, st),
+       "twiddles");
+    CK(launch_twiddles<double>(ny, sy ? sy : line_pass_radix<double>(ny), (Cx<double>*)ty, st),
+       "twiddles");
     CK(launch_deriv_mult<double>(nx, ctx->ax, (Q4<double>*)mx, st), "derivative table");
     CK(launch_deriv_mult<double>(ny, ctx->ay, (Q4<double>*)my, st), "derivative table");
     LinePassArgs<double> d{};
-    d.L = nx; d.n_lines = ny; d.sigma = 0; d.tw = (const Cx<double>*)tx;
+    d.L = nx; d.n_lines = ny; d.sigma = 0; d.tw = d.tw_small = (const Cx<double>*)tx;
     d.mult = (const Q4<double>*)mx; d.in = (const Q4<double>*)logs; d.out = (Q4<double>*)dxT;
     CK(launch_line_pass<double>(d, MODE_DERIV, 0, st), "x derivative of log fields");
     CK(launch_transpose<double>((const Q4<double>*)logs, (Q4<double>*)logsT, ny, nx, st),
        "transpose");
-    d.L = ny; d.n_lines = nx; d.sigma = 1; d.tw = (const Cx<double>*)ty;
+    d.L = ny; d.n_lines = nx; d.sigma = 1; d.tw = d.tw_small = (const Cx<double>*)ty;
     d.mult = (const Q4<double>*)my; d.in = (const Q4<double>*)logsT; d.out = (Q4<double>*)dy;
     CK(launch_line_pass<double>(d, MODE_DERIV, 0, st), "y derivative of log fields");
     const double fac = ctx->conn == DIRAC_CONN_PAPER_2D ? 0.25 : 0.5;
@@ -890,6 +905,12 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
     CK(launch_twiddles<T>(nx, line_pass_radix_alt<T>(nx), (Cx<T>*)ctx->tw_x_alt, st), "twiddles");
   if (ctx->tw_y_alt)
     CK(launch_twiddles<T>(ny, line_pass_radix_alt<T>(ny), (Cx<T>*)ctx->tw_y_alt, st), "twiddles");
+  if (ctx->tw_x_small)
+    CK(launch_twiddles<T>(nx, line_pass_radix_small<T>(nx, ny), (Cx<T>*)ctx->tw_x_small, st),
+       "twiddles");
+  if (ctx->tw_y_small)
+    CK(launch_twiddles<T>(ny, line_pass_radix_small<T>(ny, nx), (Cx<T>*)ctx->tw_y_small, st),
+       "twiddles");
   if (ctx->tw_x_team)
     CK(launch_team_twiddles<T>(nx, (Cx<T>*)ctx->tw_x_team, st), "twiddles");
   if (ctx->tw_y_team)
@@ -912,8 +933,6 @@ static dirac_status create_impl(dirac_ctx* ctx, const double* g_host[3]) {
 dirac_status dgb_tables_for_dt(dirac_ctx* ctx, double dt) {
   return ctx->prec == DIRAC_C64 ? tables_for_dt<float>(ctx, dt) : tables_for_dt<double>(ctx, dt);
 }
-
-int dgb_pass_opt(const dirac_ctx* ctx, int threads, int L) { return pass_opt(ctx, threads, L); }
 
 // Device bytes a context of this size holds at most (creation, state, half-step
 // matrices, staging for host transfers, observables scratch and density).
@@ -954,7 +973,7 @@ static dirac_status tune_pass(dirac_ctx* ctx, int axis, int reps, int* best, flo
   for (int t : options) {
     if (t == 1024 && !(sizeof(T) == 4 && L >= 256)) continue;  // team pass: complex64 only
     if ((t & DIRAC_LAUNCH_ALT_RADIX) && !line_pass_radix_alt<T>(L)) continue;
-    const int opt = pass_opt(ctx, t, L);
+    const int opt = pass_opt(ctx, t, L, a.n_lines);
     cudaError_t e = cudaSuccess;
     for (int w = 0; w < 2 && e == cudaSuccess; ++w) e = launch_line_pass<T>(a, MODE_STEP, opt, ctx->stream);
     if (e == cudaSuccess) e = cudaEventRecord(e0, ctx->stream);

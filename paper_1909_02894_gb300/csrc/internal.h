@@ -64,6 +64,10 @@ int line_pass_radix(int L);
 // launch options 3 and 4 run it, with a twiddle table of that radix in tw_alt.
 template <typename T>
 int line_pass_radix_alt(int L);
+// Elements per thread of launch option 0 and of the derivative mode for lines of 128 points
+// or fewer (0: longer lines), with a twiddle table of that radix in tw_small.
+template <typename T>
+int line_pass_radix_small(int L, int n_lines);
 // Debug builds (-DDIRAC_DEBUG=1): read and clear the index-check flags of the line-pass
 // translation units; nonzero when a check failed. Always 0 in release builds.
 int dgb_debug_flag_c64();

@@ -8,19 +8,26 @@ namespace dgb {
 
 // Elements per thread: FP32 lines of 256 points or more use E = 8 (radix-8 passes; the
 // FFT state of a thread fits the 64-register budget of 1024 threads per SM without
-// spilling), and so do 64- and 128-point lines in both precisions (twice the threads per
-// line: a small grid's pass is bound by the latency of each warp's dependent chain, and
-// halving the chain measured 0.086 -> 0.050 ms per 128^2 complex128 step); the other
-// lengths use E = 16.
+// spilling), and so do 64- and 128-point lines in both precisions and FP64 lines of 256
+// points; the other lengths use E = 16.
 template <typename T>
 constexpr int radix_e(int L) {
-  return ((sizeof(T) == 4 && L >= 256) || L == 64 || L == 128) ? 8 : 16;
+  return ((sizeof(T) == 4 && L >= 256) || L == 64 || L == 128 || L == 256) ? 8 : 16;
 }
+// Elements per thread of the small shape of lines of 128 points or fewer: few, so that a small
+// grid's lines spread over many warps. Its pass is bound by the length of each warp's chain
+// and, in FP64, by the one warp instruction per 64 cycles that a quarter of an SM takes
+// (measured; four warps on different quarters reach the SM's rate of one per 19). Measured per
+// step (ms), E = 8 | 4 | 2: complex128 128^2 0.0463 | 0.0276 | 0.0201, 64^2 (0.045) | 0.0237 |
+// 0.0165; complex64 128^2 0.0122 | 0.0091 | 0.0085, 64^2 0.0099 | 0.0086 | 0.0074. Many lines
+// fill the GPU anyway, and fewer passes win: complex64 128 x 1024 E = 4 0.0136, E = 2 0.0155.
+constexpr int radix_small(int L, int n_lines) { return L > 128 ? 0 : n_lines <= 512 ? 2 : 4; }
 // The other radix schedule the autotuner may choose (0: none): FP32 lines of 256..4096
-// points in radix-16 passes, FP64 lines of 256..2048 points in radix-8 passes.
+// points in radix-16 passes, FP64 lines of 256 points in radix-16, of 512..2048 points in
+// radix-8 passes.
 template <typename T>
 constexpr int radix_alt(int L) {
-  return L < 256 ? 0 : sizeof(T) == 4 ? (L <= 4096 ? 16 : 0) : (L <= 2048 ? 8 : 0);
+  return L < 256 ? 0 : sizeof(T) == 4 ? (L <= 4096 ? 16 : 0) : L == 256 ? 16 : L <= 2048 ? 8 : 0;
 }
 
 template <typename T, int L, int LPC, int MODE, int E = radix_e<T>(L)>
@@ -51,42 +58,51 @@ static cudaError_t launch_one(const LinePassArgs<T>& a, cudaStream_t st) {
   return launch_pdl(kern, dim3(grid), dim3(Gm::THREADS), Gm::SMEM, st, pdl, Gm::CS, a);
 }
 
-// Two CTA shapes per line length (opt 0 smaller, opt 1 larger; lines of 32 points or
-// fewer and 4096-point lines have one). Lines per CTA, by precision:
+// Two CTA shapes per line length (opt 0 smaller, opt 1 larger; 4096-point lines have one).
+// Lines per CTA, by precision:
 //   FP32 (E = 8 from 256 points): 256: 4|8, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1
 //     (256|512 threads, 512|1024 at 2048, 1024 at 4096)
-//   FP64 (E = 16 from 256 points): 256: 1|2, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1 (32..512 threads).
+//   FP64 (E = 16 from 512 points): 256: 1|2, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1 (64..512 threads).
 //     The FP64 pass is bound by the FP64 units and its CTAs hold 128-162 registers per
 //     thread, so few CTAs fit an SM: small CTAs keep all 152 SMs evenly loaded. Measured on
-//     the strained-graphene grids (ms per step, opt 0 | opt 1): 256^2 0.096 | 0.096,
-//     512^2 0.203 | 0.199, 1024^2 0.741 | 0.886, 2048^2 3.61 | 3.20; the shapes used before
-//     (256: 8|16, 512: 4|8, 1024: 2|4) took 0.180 | 0.350, 0.199 | 0.387, 0.885 | 0.832.
-//   both: 64 and 128 points (E = 8) 2|16 lines per CTA, 16 and 32 points 16. Measured
-//     (ms per step, opt 0 | opt 1): complex128 64^2 0.045 | 0.078, 128^2 0.050 | 0.168;
-//     complex64 64^2 0.0156 | 0.0146, 128^2 0.0166 | 0.0187.
+//     the strained-graphene grids (ms per step, opt 0 | opt 1): 512^2 0.203 | 0.199, 1024^2
+//     0.741 | 0.886, 2048^2 3.61 | 3.20.
+//   both, 128 points or fewer: as few lines as fill a warp or two with radix_small elements per
+//     thread (16 points 4 | 2, 32 points 2 | 1 for E = 4 | 2, 64 and 128 points 1) | 16 lines.
+//     A full GPU prefers the larger shape (100 complex64 128^2 instances: 0.074 ms per step
+//     against 0.091 with E = 4), which is the batches' default.
+template <typename T, int MODE, int E>
+static cudaError_t dispatch_small(const LinePassArgs<T>& a, cudaStream_t st) {
+  switch (a.L) {
+    case 16: return launch_one<T, 16, E, MODE, E>(a, st);
+    case 32: return launch_one<T, 32, E / 2, MODE, E>(a, st);
+    case 64: return launch_one<T, 64, 1, MODE, E>(a, st);
+    case 128: return launch_one<T, 128, 1, MODE, E>(a, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
 template <typename T, int MODE>
 static cudaError_t dispatch(const LinePassArgs<T>& a, int opt, cudaStream_t st) {
   constexpr bool F = sizeof(T) == 4;
   const bool big = (MODE == MODE_STEP) && opt != 0;
+  if (!big && a.L <= 128) {
+    if (!a.tw_small) return cudaErrorInvalidValue;
+    LinePassArgs<T> b = a;
+    b.tw = a.tw_small;
+    return radix_small(a.L, a.n_lines) == 2 ? dispatch_small<T, MODE, 2>(b, st)
+                                            : dispatch_small<T, MODE, 4>(b, st);
+  }
   if constexpr (MODE == MODE_STEP) {
-    // 64- and 128-point lines: 2 lines per CTA as the smaller shape (one or two warps; a
-    // small grid then spreads over 8x as many CTAs), 16 as the larger
-    if (!big) {
-      switch (a.L) {
-        case 64: return launch_one<T, 64, 2, MODE>(a, st);
-        case 128: return launch_one<T, 128, 2, MODE>(a, st);
-        default: break;
-      }
+    switch (a.L) {
+      case 16: return launch_one<T, 16, 16, MODE>(a, st);
+      case 32: return launch_one<T, 32, 16, MODE>(a, st);
+      case 64: return launch_one<T, 64, 16, MODE>(a, st);
+      case 128: return launch_one<T, 128, 16, MODE>(a, st);
+      default: break;
     }
   }
-  switch (a.L) {
-    case 16: return launch_one<T, 16, 16, MODE>(a, st);
-    case 32: return launch_one<T, 32, 16, MODE>(a, st);
-    case 64: return launch_one<T, 64, 16, MODE>(a, st);
-    case 128: return launch_one<T, 128, 16, MODE>(a, st);
-    case 4096: return launch_one<T, 4096, 1, MODE>(a, st);
-    default: break;
-  }
+  if (a.L == 4096) return launch_one<T, 4096, 1, MODE>(a, st);
   if constexpr (MODE == MODE_STEP) {
     if (big) {
       switch (a.L) {
@@ -108,8 +124,8 @@ static cudaError_t dispatch(const LinePassArgs<T>& a, int opt, cudaStream_t st) 
 }
 
 // The alternative radix schedule (radix_alt), opt 3 the smaller and opt 4 the larger of two
-// CTA shapes (about 256 and 512 threads; 4096-point FP32 lines and 2048-point FP64 lines
-// have one, 512 threads). Its twiddle table (a.tw_alt) has the layout of that radix.
+// CTA shapes (about 256 and 512 threads; 1 and 2 lines for FP64 lines of 256 points;
+// 4096-point FP32 lines and 2048-point FP64 lines have one, 512 threads). Its twiddle table (a.tw_alt) has the layout of that radix.
 template <typename T>
 static cudaError_t dispatch_alt(const LinePassArgs<T>& a0, int opt, cudaStream_t st) {
   if (!a0.tw_alt) return cudaErrorInvalidValue;
@@ -126,9 +142,9 @@ static cudaError_t dispatch_alt(const LinePassArgs<T>& a0, int opt, cudaStream_t
       case 4096: return launch_one<T, 4096, 1, M, 16>(a, st);
       default: return cudaErrorInvalidValue;
     }
-  } else {  // radix 8: 2 L / 8 threads per line
+  } else {  // radix 8: 2 L / 8 threads per line (256 points: radix 16)
     switch (a.L) {
-      case 256: return big ? launch_one<T, 256, 8, M, 8>(a, st) : launch_one<T, 256, 4, M, 8>(a, st);
+      case 256: return big ? launch_one<T, 256, 2, M, 16>(a, st) : launch_one<T, 256, 1, M, 16>(a, st);
       case 512: return big ? launch_one<T, 512, 4, M, 8>(a, st) : launch_one<T, 512, 2, M, 8>(a, st);
       case 1024: return big ? launch_one<T, 1024, 2, M, 8>(a, st) : launch_one<T, 1024, 1, M, 8>(a, st);
       case 2048: return launch_one<T, 2048, 1, M, 8>(a, st);
@@ -163,5 +179,7 @@ template <typename T>
 int line_pass_radix(int L) { return radix_e<T>(L); }
 template <typename T>
 int line_pass_radix_alt(int L) { return radix_alt<T>(L); }
+template <typename T>
+int line_pass_radix_small(int L, int n_lines) { return radix_small(L, n_lines); }
 
 }  // namespace dgb

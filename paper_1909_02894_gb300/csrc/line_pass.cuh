@@ -17,7 +17,7 @@
 // as a deviation from identity keeps FP32 rounding proportional to |exp(..) - 1|.
 // Derivative mode (Sec. 5 eq. trick): out_c = F^-1[ i xi / L  F psi_c ] per component.
 //
-// FFT: radix-E Stockham autosort (E = 8 or 16 elements per thread). Thread (j, c) of a
+// FFT: radix-E Stockham autosort (E = 2, 4, 8 or 16 elements per thread). Thread (j, c) of a
 // line holds elements j + m L/E (m < E) of component c; that index set is the input of
 // the first pass and the output of the last one for any radix sequence, so the global
 // load, the k-space multiply and the epilogue happen in registers and only the passes in
@@ -57,6 +57,7 @@ struct LinePassArgs {
   int sigma;            // 0: sigma_x (x pass), 1: sigma_y (y pass)
   const Cx<T>* tw;      // per-pass twiddles, see tw_offset (at most L entries)
   const Cx<T>* tw_alt;  // the same for the alternative radix schedule (or nullptr)
+  const Cx<T>* tw_small;  // lines of 128 points or fewer: the same for the small shape's radix
   const Cx<T>* tw_team;  // twiddles of the radix-16 team pass (launch_team_twiddles), or nullptr
   const Q4<T>* mult;    // per k index q: step ((cos - 1) hi, lo, sin hi, lo) / (2L);
                         // derivative (0, 0, xi hi, xi lo) / L
@@ -300,9 +301,9 @@ struct Geo {
   static constexpr size_t SMEM = FFT_BYTES > STAGE_BYTES ? FFT_BYTES : STAGE_BYTES;
   static constexpr int NIT = (L / CS) * GL / THREADS;  // transposed-store items per thread
   static_assert((L & (L - 1)) == 0 && L >= 16, "L must be a power of two >= 16");
-  static_assert(E == 8 || E == 16, "E must be 8 or 16");
+  static_assert(E == 2 || E == 4 || E == 8 || E == 16, "E must be 2, 4, 8 or 16");
   static_assert(THREADS <= 1024, "at most 1024 threads per CTA");
-  static_assert((L / CS) * GL == NIT * THREADS && NIT % 2 == 0, "store items must divide");
+  static_assert((L / CS) * GL == NIT * THREADS && (NIT == 1 || NIT % 2 == 0), "store items must divide");
 };
 
 template <int E>
@@ -418,7 +419,7 @@ __device__ __forceinline__ void fft_passes(Cx<T> (&v)[E], Cx<T>* buf, int j, con
 // registers; FP64 CTAs take up to 128 registers (the FP64 path is ALU bound).
 template <typename T, int THREADS, int E>
 struct MinBlocks {
-  static constexpr int want = sizeof(T) == 4 ? (E == 8 ? 1024 : 512) / THREADS : 1;
+  static constexpr int want = sizeof(T) == 4 ? (E <= 8 ? 1024 : 512) / THREADS : 1;
   static constexpr int value = want < 1 ? 1 : want;
 };
 
@@ -583,11 +584,11 @@ __global__ void __launch_bounds__(Geo<T, L, LPC, E>::THREADS,
   }
   const int line0 = (blk / CS) * GL;
   const int i0 = rank * ROWS;
-  constexpr int HALF = Gm::NIT / 2;
+  constexpr int ROUNDS = Gm::NIT > 1 ? 2 : 1, HALF = Gm::NIT / ROUNDS;
   // (a normal-layout store happened in the epilogue)
   if (!a.store_normal) {
 #pragma unroll
-  for (int h = 0; h < 2; ++h) {
+  for (int h = 0; h < ROUNDS; ++h) {
     Q4<T> val[HALF];
 #pragma unroll
     for (int q = 0; q < HALF; ++q) {

@@ -114,3 +114,24 @@ def test_potentials_inside_the_team_pass(nx, ny, scheme):
         s.step(1, w.dt)
         s.step(2, 0.5 * w.dt)
         assert_parity(s.get_state(), ref, w, TOL)
+
+
+@pytest.mark.parametrize("prec", [D.DIRAC_C64, D.DIRAC_C128], ids=["c64", "c128"])
+@pytest.mark.parametrize("nx,ny", [(16, 1024), (32, 1024), (64, 1024), (128, 1024), (128, 512),
+                                   (64, 16), (32, 32)])
+def test_short_lines_with_two_and_four_points_per_thread(nx, ny, prec):
+    """The small shape of lines of 128 points or fewer around its rule (512 lines), in the step
+    and in the derivative mode (the energy's derivatives), against the oracle."""
+    w = grid(nx, ny, noise=0.0)
+    prob = oracle.Problem.from_workload(w)
+    ref = oracle.run(prob, w.psi0, w.dt, 3)
+    with D.Simulation(w, precision=prec) as s:
+        D.dirac_set_launch(s.ctx, 256, 256)
+        s.set_state(w.psi0)
+        s.step(3, w.dt)
+        got, obs = s.get_state(), s.observables()
+    assert_parity(got, ref, w, 1e-11 if prec == D.DIRAC_C128 else TOL)
+    want = oracle.observables(prob, got)
+    tol = 1e-12 if prec == D.DIRAC_C128 else 1e-6
+    for k in ("norm", "norm_gamma", "energy"):
+        assert abs(obs[k] - want[k]) <= tol * max(1.0, abs(want[k])), k
