@@ -231,14 +231,160 @@ __device__ __forceinline__ void dft16(Cx<T> (&x)[16], const Cx<T>* __restrict__ 
   for (int i = 0; i < 16; ++i) x[i] = y[i];
 }
 
+// ---- FP64 butterflies in fused multiply-adds. The FP64 pass is bound by the number of FP64
+// instructions (the pipe is 85 % busy), so every twiddle w = c (1 + i tau) is applied in two
+// steps that fuse: u = x (1 + i tau) costs two FMAs, and the factor c goes into the additions
+// that follow (Linzer and Feig's scheme). A DFT-4 with three twiddles takes 22 instructions
+// instead of 28, with four 28 instead of 32; DFT-16 144 instead of 160 (its inner twiddles are
+// constants), 186 instead of 220 with its 15 outer ones. Where |c| < 2^-60 the table holds
+// 2^-60: u is then at most 2^60 |x|, and what is lost is below the rounding of x w. Rounding
+// errors are those of the usual product (each is relative to |x|).
+__device__ __forceinline__ Cx<double> fma_c(double s, Cx<double> a, Cx<double> b) {  // s a + b
+  return {fma(s, a.re, b.re), fma(s, a.im, b.im)};
+}
+template <bool INV>
+__device__ __forceinline__ Cx<double> twist(Cx<double> x, double tau) {  // x (1 +- i tau)
+  if (INV) tau = -tau;
+  return {fma(-tau, x.im, x.re), fma(tau, x.re, x.im)};
+}
+// y0, y2 = A +- c1 s; y1, y3 = B -+ i c1 d (forward)
+template <bool INV>
+__device__ __forceinline__ void tw4_out(Cx<double> A, Cx<double> B, Cx<double> s, Cx<double> d,
+                                        double c1, Cx<double>& y0, Cx<double>& y1, Cx<double>& y2,
+                                        Cx<double>& y3) {
+  const double cd = INV ? -c1 : c1;
+  y0 = fma_c(c1, s, A);
+  y2 = fma_c(-c1, s, A);
+  y1 = {fma(cd, d.im, B.re), fma(-cd, d.re, B.im)};
+  y3 = {fma(-cd, d.im, B.re), fma(cd, d.re, B.im)};
+}
+// DFT-4 of x0, w1 x1, w2 x2, w3 x3 (tau_j, c2, c1, r = c3 / c1)
+template <bool INV>
+__device__ __forceinline__ void tw4_plain(Cx<double>& x0, Cx<double>& x1, Cx<double>& x2,
+                                          Cx<double>& x3, double t1, double t2, double t3,
+                                          double c2, double c1, double r) {
+  const Cx<double> u1 = twist<INV>(x1, t1), u2 = twist<INV>(x2, t2), u3 = twist<INV>(x3, t3);
+  const Cx<double> A = fma_c(c2, u2, x0), B = fma_c(-c2, u2, x0);
+  const Cx<double> s = fma_c(r, u3, u1), d = fma_c(-r, u3, u1);
+  tw4_out<INV>(A, B, s, d, c1, x0, x1, x2, x3);
+}
+// DFT-4 of w0 x0 .. w3 x3 (r2 = c2 / c0, r3 = c3 / c1)
+template <bool INV>
+__device__ __forceinline__ void tw4_all(Cx<double>& x0, Cx<double>& x1, Cx<double>& x2,
+                                        Cx<double>& x3, double t0, double t1, double t2,
+                                        double t3, double r2, double r3, double c0, double c1) {
+  const Cx<double> u0 = twist<INV>(x0, t0), u1 = twist<INV>(x1, t1);
+  const Cx<double> u2 = twist<INV>(x2, t2), u3 = twist<INV>(x3, t3);
+  Cx<double> A = fma_c(r2, u2, u0), B = fma_c(-r2, u2, u0);
+  A = {c0 * A.re, c0 * A.im};
+  B = {c0 * B.re, c0 * B.im};
+  const Cx<double> s = fma_c(r3, u3, u1), d = fma_c(-r3, u3, u1);
+  tw4_out<INV>(A, B, s, d, c1, x0, x1, x2, x3);
+}
+// the inner twiddles of DFT-16 and DFT-8: cos and tan of pi / 8, sqrt(1/2)
+constexpr double kC1 = 0.92387953251128675613, kC3 = 0.38268343236508977173;
+constexpr double kT1 = 0.41421356237309504880, kT3 = 2.41421356237309504880;
+constexpr double kC2 = 0.70710678118654752440;
+
+// the second half of DFT-16 = 4 x 4 after the DFT-4s over n1: W16^(n2 k1), DFT-4s, order
+template <bool INV>
+__device__ __forceinline__ void dft16_outer(Cx<double> (&x)[16]) {
+  dft4<double, INV>(x[0], x[1], x[2], x[3]);
+  tw4_plain<INV>(x[4], x[5], x[6], x[7], -kT1, -1.0, -kT3, kC2, kC1, kT1);
+  {
+    // W^2 = sqrt(1/2) (1 - i), W^4 = -i, W^6 = -sqrt(1/2) (1 + i) (forward)
+    const Cx<double> x2 = INV ? mul_i(x[10]) : mul_mi(x[10]);
+    const Cx<double> A = cadd(x[8], x2), B = csub(x[8], x2);
+    const Cx<double> u1 = INV ? Cx<double>{x[9].re - x[9].im, x[9].im + x[9].re}
+                              : Cx<double>{x[9].re + x[9].im, x[9].im - x[9].re};
+    const Cx<double> u3 = INV ? Cx<double>{x[11].re + x[11].im, x[11].im - x[11].re}
+                              : Cx<double>{x[11].re - x[11].im, x[11].im + x[11].re};
+    tw4_out<INV>(A, B, csub(u1, u3), cadd(u1, u3), kC2, x[8], x[9], x[10], x[11]);
+  }
+  tw4_plain<INV>(x[12], x[13], x[14], x[15], -kT3, 1.0, -kT1, -kC2, kC3, -kT3);
+  Cx<double> y[16];
+#pragma unroll
+  for (int k1 = 0; k1 < 4; ++k1)
+#pragma unroll
+    for (int k2 = 0; k2 < 4; ++k2) y[k1 + 4 * k2] = x[4 * k1 + k2];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) x[i] = y[i];
+}
+// the second half of DFT-8 after the DFT-4s of the even and the odd elements
+template <bool INV>
+__device__ __forceinline__ void dft8_outer(Cx<double> (&x)[8], Cx<double> e0, Cx<double> e1,
+                                           Cx<double> e2, Cx<double> e3, Cx<double> o0,
+                                           Cx<double> o1, Cx<double> o2, Cx<double> o3) {
+  const Cx<double> u1 = INV ? Cx<double>{o1.re - o1.im, o1.im + o1.re}
+                            : Cx<double>{o1.re + o1.im, o1.im - o1.re};
+  const Cx<double> u3 = INV ? Cx<double>{o3.re + o3.im, o3.im - o3.re}
+                            : Cx<double>{o3.re - o3.im, o3.im + o3.re};
+  const Cx<double> p2 = INV ? mul_i(o2) : mul_mi(o2);
+  x[0] = cadd(e0, o0);
+  x[4] = csub(e0, o0);
+  x[1] = fma_c(kC2, u1, e1);
+  x[5] = fma_c(-kC2, u1, e1);
+  x[2] = cadd(e2, p2);
+  x[6] = csub(e2, p2);
+  x[3] = fma_c(-kC2, u3, e3);
+  x[7] = fma_c(kC2, u3, e3);
+}
+// R-point butterfly with the pass's twiddles (tw: this k's first slot, step between slots):
+// the slots hold the pairs that the twiddle kernel's tan_pair gives.
+template <int R, bool INV>
+__device__ __forceinline__ void tw_dft(Cx<double> (&x)[R], const Cx<double>* __restrict__ tw,
+                                       int step) {
+  auto slot = [&](int i) { return ldg_cx(tw + i * step); };
+  auto plain = [&](int i, Cx<double>& a, Cx<double>& b, Cx<double>& c, Cx<double>& d) {
+    const Cx<double> p = slot(i), q = slot(i + 1), r = slot(i + 2);
+    tw4_plain<INV>(a, b, c, d, p.re, p.im, q.re, q.im, r.re, r.im);
+  };
+  auto all = [&](int i, Cx<double>& a, Cx<double>& b, Cx<double>& c, Cx<double>& d) {
+    const Cx<double> p = slot(i), q = slot(i + 1), r = slot(i + 2), s = slot(i + 3);
+    tw4_all<INV>(a, b, c, d, p.re, p.im, q.re, q.im, r.re, r.im, s.re, s.im);
+  };
+  if constexpr (R == 2) {
+    const Cx<double> p = slot(0), u = twist<INV>(x[1], p.re), a = x[0];
+    x[0] = fma_c(p.im, u, a);
+    x[1] = fma_c(-p.im, u, a);
+  } else if constexpr (R == 4) {
+    plain(0, x[0], x[1], x[2], x[3]);
+  } else if constexpr (R == 8) {
+    Cx<double> e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
+    Cx<double> o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
+    plain(0, e0, e1, e2, e3);
+    all(3, o0, o1, o2, o3);
+    dft8_outer<INV>(x, e0, e1, e2, e3, o0, o1, o2, o3);
+  } else {
+    plain(0, x[0], x[4], x[8], x[12]);
+    asm volatile("" ::: "memory");
+#pragma unroll
+    for (int n2 = 1; n2 < 4; ++n2) {
+      all(4 * n2 - 1, x[n2], x[n2 + 4], x[n2 + 8], x[n2 + 12]);
+      asm volatile("" ::: "memory");
+    }
+    dft16_outer<INV>(x);
+  }
+}
+
 template <typename T, int R, bool INV>
 __device__ __forceinline__ void dftR(Cx<T> (&x)[R]) {
   if constexpr (R == 2) {
     dft2<T, INV>(x[0], x[1]);
   } else if constexpr (R == 4) {
     dft4<T, INV>(x[0], x[1], x[2], x[3]);
+  } else if constexpr (R == 8 && sizeof(T) == 8) {
+    Cx<T> e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
+    Cx<T> o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
+    dft4<T, INV>(e0, e1, e2, e3);
+    dft4<T, INV>(o0, o1, o2, o3);
+    dft8_outer<INV>(x, e0, e1, e2, e3, o0, o1, o2, o3);
   } else if constexpr (R == 8) {
     dft8<T, INV>(x);
+  } else if constexpr (sizeof(T) == 8) {
+#pragma unroll
+    for (int n2 = 0; n2 < 4; ++n2) dft4<T, INV>(x[n2], x[n2 + 4], x[n2 + 8], x[n2 + 12]);
+    dft16_outer<INV>(x);
   } else {
     dft16<T, INV, false>(x);
   }
@@ -249,7 +395,8 @@ __host__ __device__ constexpr int ilog2c(int v) { return v <= 1 ? 0 : 1 + ilog2c
 
 // Twiddle table layout: the passes after the first (span NS = E, E^2, ...) each own a
 // block [(t - 1) NS + k] = exp(-2 pi i t k / (NS R)), t = 1..R-1, k < NS, so that the
-// lanes of a warp (consecutive k) read consecutive entries. Every pass but the last has
+// lanes of a warp (consecutive k) read consecutive entries (FP64: the same number of slots per
+// k, holding the tangents, cosines and their ratios that tw_dft uses). Every pass but the last has
 // radix E; the block of span NS starts after the (E - 1) NS' entries of each earlier span.
 __host__ __device__ constexpr int tw_offset(int NS, int E) {
   return NS <= E ? 0 : tw_offset(NS / E, E) + (E - 1) * (NS / E);
@@ -321,7 +468,10 @@ __device__ __forceinline__ void pass_compute(Cx<T> (&v)[E], int j, const Cx<T>* 
     Cx<T> x[R];
 #pragma unroll
     for (int t = 0; t < R; ++t) x[t] = v[u + t * NB];
-    if constexpr (NS > 1 && R == 16) {
+    if constexpr (NS > 1 && sizeof(T) == 8) {
+      const int k = (j + u * J) & (NS - 1);
+      tw_dft<R, INV>(x, tw + tw_offset(NS, E) + k, NS);
+    } else if constexpr (NS > 1 && R == 16) {
       const int k = (j + u * J) & (NS - 1);
       dft16<T, INV, true>(x, tw + tw_offset(NS, E) + k, NS);
     } else {

@@ -303,6 +303,29 @@ __device__ inline void split(double v, T* hi, T* lo) {
 // thread: for every pass after the first, span NS (E, E^2, ...) and radix R (E, or the
 // remaining radix for the last pass), entries [(t - 1) NS + k] = exp(-2 pi i t k/(NS R)).
 // Computed in FP64.
+// Slot i (0..r-2) of the FP64 butterflies' twiddles w_t = exp(-2 pi i t phase) = c_t (1 + i
+// tau_t), see tw_dft: groups of a DFT-4 with x0 untwiddled, factors t1..t3: (tau1, tau2), (tau3,
+// c2), (c1, c3/c1); with four factors: (tau0, tau1), (tau2, tau3), (c2/c0, c3/c1), (c0, c1).
+__device__ inline double2 tan_pair(int r, int i, double phase) {
+  auto c = [&](int t) {
+    const double v = cospi(2.0 * t * phase), least = 8.673617379884035e-19;  // 2^-60
+    return fabs(v) < least ? copysign(least, v) : v;
+  };
+  auto tau = [&](int t) { return -sinpi(2.0 * t * phase) / c(t); };
+  if (r == 2) return make_double2(tau(1), c(1));
+  // stride between the factors of a group, first group's t1
+  const int d = r / 4;
+  if (i < 3)
+    return i == 0   ? make_double2(tau(d), tau(2 * d))
+           : i == 1 ? make_double2(tau(3 * d), c(2 * d))
+                    : make_double2(c(d), c(3 * d) / c(d));
+  const int g = (i - 3) / 4 + 1, s = (i - 3) % 4;  // group g: factors g, g + d, g + 2 d, g + 3 d
+  return s == 0   ? make_double2(tau(g), tau(g + d))
+         : s == 1 ? make_double2(tau(g + 2 * d), tau(g + 3 * d))
+         : s == 2 ? make_double2(c(g + 2 * d) / c(g), c(g + 3 * d) / c(g + d))
+                  : make_double2(c(g), c(g + d));
+}
+
 template <typename T>
 __global__ void k_twiddles(int n, int e, Cx<T>* tw) {
   const int m = blockIdx.x * blockDim.x + threadIdx.x;
@@ -317,6 +340,11 @@ __global__ void k_twiddles(int n, int e, Cx<T>* tw) {
     const int cnt = (r - 1) * ns;
     if (m < off + cnt) {
       const int t = (m - off) / ns + 1, k = (m - off) % ns;
+      if constexpr (sizeof(T) == 8) {
+        const double2 p = tan_pair(r, t - 1, (double)k / ((double)ns * r));
+        tw[m] = {(T)p.x, (T)p.y};
+        return;
+      }
       double s, c;
       sincospi(2.0 * (double)t * k / ((double)ns * r), &s, &c);
       tw[m] = {(T)c, (T)(-s)};
