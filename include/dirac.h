@@ -207,7 +207,9 @@ long dirac_krylov_iterations(const dirac_ctx *ctx);
  * shared memory while the current ones are finished); 0 = the default (complex64: the team
  * pass for lines of 256 points or more, the smaller shape for 128-point lines, else the
  * larger; complex128: the smaller shape for 1024-point lines and lines of 128 points or
- * fewer, else the larger; 512-point lines the smaller when there are fewer than 512). The
+ * fewer, else the larger; 512-point lines the smaller when there are fewer than 512; complex64
+ * grids whose axes both have 64 or 128 points run whole Scheme II steps, all of a call, in one
+ * launch). The
  * smaller shape of lines of 128 points or fewer gives each thread 2 (up to 512 lines) or 4
  * points, the larger takes 16 lines per CTA; 4096-point lines have one shape besides the team
  * pass. 256 or 512 plus
@@ -223,7 +225,9 @@ dirac_status dirac_set_launch(dirac_ctx *ctx, int threads_x_pass, int threads_y_
 /* Autotuner: times every CTA shape and radix schedule of the x and the y pass (the
  * dirac_set_launch values; reps launches each, CUDA
  * events on the context's stream, output to scratch memory so the state is unchanged),
- * applies the fastest with dirac_set_launch and returns it in *threads_x, *threads_y.
+ * applies the fastest with dirac_set_launch and returns it in *threads_x, *threads_y (0, 0 for
+ * complex64 Scheme II grids of 64- and 128-point axes, whose default runs whole steps in one
+ * launch).
  * The state must be set; synchronises the stream. */
 dirac_status dirac_autotune(dirac_ctx *ctx, int reps, int *threads_x, int *threads_y);
 

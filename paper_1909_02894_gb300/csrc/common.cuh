@@ -63,14 +63,19 @@ template <typename T>
 __device__ __forceinline__ Cx<T> cadd(Cx<T> a, Cx<T> b) { return {a.re + b.re, a.im + b.im}; }
 template <typename T>
 __device__ __forceinline__ Cx<T> csub(Cx<T> a, Cx<T> b) { return {a.re - b.re, a.im - b.im}; }
+// a b + c in one rounding. Products are written with it where the compiler could contract
+// them in two ways, so that every kernel rounds alike (whole-step launches give the bits of
+// separate passes).
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
 template <typename T>
 __device__ __forceinline__ Cx<T> cmul(Cx<T> a, Cx<T> b) {
-  return {a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re};
+  return {fma_t(a.re, b.re, -(a.im * b.im)), fma_t(a.re, b.im, a.im * b.re)};
 }
 // a * conj(b)
 template <typename T>
 __device__ __forceinline__ Cx<T> cmulc(Cx<T> a, Cx<T> b) {
-  return {a.re * b.re + a.im * b.im, a.im * b.re - a.re * b.im};
+  return {fma_t(a.re, b.re, a.im * b.im), fma_t(a.im, b.re, -(a.re * b.im))};
 }
 // ---- packed FP32 pairs (sm_100 and later): the (re, im) of a complex64 value in one
 // 64-bit register pair, two FP32 operations per instruction, each rounded exactly like its

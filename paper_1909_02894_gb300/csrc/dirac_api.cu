@@ -92,11 +92,16 @@ static int pass_opt(const dirac_ctx* ctx, int shape, int L, int n_lines) {
   if (threads == 1024) return 2;
   // Default, by measurement: complex64 the team pass for lines of 256 points or more (256^2
   // 0.0109 against 0.0118 ms per step for the radix-8 pass, 1024^2 0.0282 against 0.039); the
-  // smaller shape for lines of 128 points or fewer and, in complex128, for 1024-point lines (one
-  // line per CTA: 1024 CTAs spread over the SMs to within one line, 0.74 against 0.89 ms per
-  // 1024^2 step) and fewer than 512 lines of 512 points (512 x 256: 0.104 against 0.165 ms per
-  // step); else the larger.
-  if (ctx->prec == DIRAC_C64) return L >= 256 ? 2 : 0;
+  // smaller shape for lines of 128 points or fewer, but for complex64 lines of 32 points or more
+  // only up to 2^17 points (128 x 1024 0.0137 against 0.0139 ms per step, 128 x 2048 0.0201
+  // against 0.0155, 64 x 1024 0.0121 against 0.0117, 32 x 4096 0.0218 against 0.0200), and, in
+  // complex128, for 1024-point lines (one line per CTA: 1024 CTAs spread over the SMs to within
+  // one line, 0.74 against 0.89 ms per 1024^2 step) and fewer than 512 lines of 512 points (512
+  // x 256: 0.104 against 0.165 ms per step); else the larger.
+  if (ctx->prec == DIRAC_C64) {
+    if (L >= 256) return 2;
+    return L >= 32 && (size_t)L * n_lines >= kWideShortLines ? 1 : 0;
+  }
   return (L == 1024 || L <= 128 || (L == 512 && n_lines < 512)) ? 0 : 1;
 }
 
@@ -652,6 +657,43 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
   return DIRAC_OK;
 }
 
+// Contexts whose Scheme II steps run whole inside one launch (small_steps.cu): default launch
+// shapes, no static potentials.
+static bool whole_steps(const dirac_ctx* ctx, bool any_shape = false) {
+  return ctx->prec == DIRAC_C64 && ctx->scheme == DIRAC_SCHEME_II && !ctx->has_pot &&
+         !ctx->beta1_im && (any_shape || (!ctx->threads_x && !ctx->threads_y)) &&
+         small_steps_grid(ctx->nx, ctx->ny);
+}
+
+// n steps in launches of at most kSmallSteps (a few milliseconds each); *done = false if the
+// device cannot hold the cluster (the steps then run as separate passes).
+constexpr long kSmallSteps = 1024;
+static dirac_status step_small(dirac_ctx* ctx, long n, bool* done) {
+  SmallStepArgs a{};
+  a.psi = (Q4<float>*)ctx->psi;
+  a.beta1 = (const float*)ctx->beta1;
+  a.beta2 = (const float*)ctx->beta2T;
+  a.u_n = ctx->u_identity ? nullptr : (const Q4<float>*)ctx->u_n;
+  a.u_t = ctx->u_identity ? nullptr : (const Q4<float>*)ctx->u_t;
+  a.u2_t = ctx->u_identity ? nullptr : (const Q4<float>*)ctx->u2_t;
+  a.mult_x = (const Q4<float>*)ctx->mult_x;
+  a.mult_y = (const Q4<float>*)ctx->mult_y;
+  a.tw_x = (const Cx<float>*)ctx->tw_x;
+  a.tw_y = (const Cx<float>*)ctx->tw_y;
+  *done = false;
+  for (long s = 0; s < n; s += kSmallSteps) {
+    const long k = n - s < kSmallSteps ? n - s : kSmallSteps;
+    const cudaError_t e = launch_small_steps(a, ctx->nx, ctx->ny, (int)k, s == 0, s + k == n,
+                                             ctx->stream);
+    if (e == cudaErrorNotSupported && s == 0) return DIRAC_OK;
+    CK(e, "steps");
+    ctx->launches += 1;
+  }
+  ctx->test_timeout_next = 0;
+  *done = true;
+  return DIRAC_OK;
+}
+
 template <typename T>
 static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
   if (dt != ctx->dt_cached) {
@@ -662,6 +704,11 @@ static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
   if (ctx->scheme == DIRAC_SCHEME_POLY_TAYLOR || ctx->scheme == DIRAC_SCHEME_POLY_CHEBYSHEV)
     return step_poly<T>(ctx, n, dt);
   if (ctx->scheme == DIRAC_SCHEME_CRANK_NICOLSON) return step_cn<T>(ctx, n, dt);
+  if (sizeof(T) == 4 && whole_steps(ctx)) {
+    bool done = false;
+    CKS(step_small(ctx, n, &done));
+    if (done) return DIRAC_OK;
+  }
   LinePassArgs<T> ax = pass_args<T>(ctx, 0), ay = pass_args<T>(ctx, 1);
   ax.in = (const Q4<T>*)ctx->psi;
   ax.out = (Q4<T>*)ctx->psiT;
@@ -946,7 +993,7 @@ size_t dgb_footprint_bytes(int nx, int ny, dirac_precision prec) {
                      + 4 * sizeof(double) // staging (complex128 spinor)
                      + 2 * q4             // observables scratch
                      + sizeof(double);    // density
-  size_t per_line = (size_t)(nx + ny) * (sizeof(double) + 3 * q4);
+  size_t per_line = (size_t)(nx + ny) * (sizeof(double) + 6 * q4);
   return n * per_point + per_line + 4 * sizeof(double) * 2048 + 4096;
 }
 
@@ -1008,6 +1055,10 @@ static dirac_status autotune_impl(dirac_ctx* ctx, int reps, int* tx, int* ty) {
   if (ctx->dt_cached == 0.0) {
     dirac_status s = tables_for_dt<T>(ctx, 0.01);
     if (s != DIRAC_OK) return s;
+  }
+  if (whole_steps(ctx, true)) {  // the default: whole steps in one launch, faster than any passes
+    *tx = *ty = ctx->threads_x = ctx->threads_y = 0;
+    return DIRAC_OK;
   }
   float mx, my;
   dirac_status s = tune_pass<T>(ctx, 0, reps, tx, &mx);

@@ -64,6 +64,9 @@ int line_pass_radix(int L);
 // launch options 3 and 4 run it, with a twiddle table of that radix in tw_alt.
 template <typename T>
 int line_pass_radix_alt(int L);
+// Short complex64 lines (32 to 128 points): from this many points the larger shape is the
+// faster one (see pass_opt in dirac_api.cu).
+constexpr size_t kWideShortLines = (size_t)1 << 17;
 // Elements per thread of launch option 0 and of the derivative mode for lines of 128 points
 // or fewer (0: longer lines), with a twiddle table of that radix in tw_small.
 template <typename T>
@@ -72,6 +75,7 @@ int line_pass_radix_small(int L, int n_lines);
 // translation units; nonzero when a check failed. Always 0 in release builds.
 int dgb_debug_flag_c64();
 int dgb_debug_flag_c128();
+int dgb_debug_flag_small();
 int dgb_debug_flag_team_256();
 int dgb_debug_flag_team_512();
 int dgb_debug_flag_team_1024();
@@ -80,7 +84,7 @@ int dgb_debug_flag_team_4096();
 inline int dgb_debug_bounds() {
   return dgb_debug_flag_c64() | dgb_debug_flag_c128() | dgb_debug_flag_team_256() |
          dgb_debug_flag_team_512() | dgb_debug_flag_team_1024() | dgb_debug_flag_team_2048() |
-         dgb_debug_flag_team_4096();
+         dgb_debug_flag_team_4096() | dgb_debug_flag_small();
 }
 
 // ---- FP64 precompute (precompute.cu)
@@ -148,6 +152,26 @@ template <int L>
 cudaError_t launch_team_unsplit(const UnsplitArgs& a, int phase, cudaStream_t st);
 // One phase of the unsplit operator on complex64 rows of L = 256..4096 points.
 cudaError_t launch_unsplit(const UnsplitArgs& a, int L, int phase, cudaStream_t st);
+
+// ---- small grids (small_steps.cu): n Scheme II steps of a complex64 grid in one launch, where
+// both axes have 64 or 128 points (small_steps_grid). lead / trail: U before the first / after
+// the last step (U^2 otherwise and between). cudaErrorNotSupported if no cluster of the needed
+// size fits the device.
+struct SmallStepArgs {
+  Q4<float>* psi;       // [ny][nx], updated in place
+  const float* beta1;   // b^1 - 1 [ny][nx]
+  const float* beta2;   // b^2 - 1 [nx][ny]
+  const Q4<float>* u_n;   // U [ny][nx], U and U^2 [nx][ny]; all null when U = I
+  const Q4<float>* u_t;
+  const Q4<float>* u2_t;
+  const Q4<float>* mult_x;
+  const Q4<float>* mult_y;
+  const Cx<float>* tw_x;  // launch_twiddles with 8 elements per thread
+  const Cx<float>* tw_y;
+};
+bool small_steps_grid(int nx, int ny);
+cudaError_t launch_small_steps(const SmallStepArgs& a, int nx, int ny, int n, bool lead,
+                               bool trail, cudaStream_t st);
 
 // ---- unsplit polynomial scheme (unsplit.cu)
 // psi <- U psi at every point (normal layout).

@@ -86,21 +86,22 @@ template <typename T, int MODE>
 static cudaError_t dispatch(const LinePassArgs<T>& a, int opt, cudaStream_t st) {
   constexpr bool F = sizeof(T) == 4;
   const bool big = (MODE == MODE_STEP) && opt != 0;
-  if (!big && a.L <= 128) {
+  // the derivative mode has no option: the larger shape for many short complex64 lines
+  const bool wide = MODE == MODE_STEP ? big
+                                      : F && a.L >= 32 && (size_t)a.L * a.n_lines >= kWideShortLines;
+  if (!wide && a.L <= 128) {
     if (!a.tw_small) return cudaErrorInvalidValue;
     LinePassArgs<T> b = a;
     b.tw = a.tw_small;
     return radix_small(a.L, a.n_lines) == 2 ? dispatch_small<T, MODE, 2>(b, st)
                                             : dispatch_small<T, MODE, 4>(b, st);
   }
-  if constexpr (MODE == MODE_STEP) {
-    switch (a.L) {
-      case 16: return launch_one<T, 16, 16, MODE>(a, st);
-      case 32: return launch_one<T, 32, 16, MODE>(a, st);
-      case 64: return launch_one<T, 64, 16, MODE>(a, st);
-      case 128: return launch_one<T, 128, 16, MODE>(a, st);
-      default: break;
-    }
+  switch (a.L) {
+    case 16: return launch_one<T, 16, 16, MODE>(a, st);
+    case 32: return launch_one<T, 32, 16, MODE>(a, st);
+    case 64: return launch_one<T, 64, 16, MODE>(a, st);
+    case 128: return launch_one<T, 128, 16, MODE>(a, st);
+    default: break;
   }
   if (a.L == 4096) return launch_one<T, 4096, 1, MODE>(a, st);
   if constexpr (MODE == MODE_STEP) {

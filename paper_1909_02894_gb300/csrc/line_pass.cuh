@@ -579,8 +579,8 @@ template <typename T>
 __device__ __forceinline__ Cx<T> apply_u_row(const Q4<T>& u, Cx<T> own, Cx<T> oth, int c) {
   const T s3 = c ? -u.w : u.w, s2 = c ? u.z : -u.z;
   // own + (c0-1) own + i s3 own + (c1 + i s2) oth
-  const T re = u.x * own.re - s3 * own.im + u.y * oth.re - s2 * oth.im;
-  const T im = u.x * own.im + s3 * own.re + u.y * oth.im + s2 * oth.re;
+  const T re = fma_t(-s2, oth.im, fma_t(u.y, oth.re, fma_t(-s3, own.im, u.x * own.re)));
+  const T im = fma_t(s2, oth.re, fma_t(u.y, oth.im, fma_t(s3, own.re, u.x * own.im)));
   return {own.re + re, own.im + im};
 }
 
@@ -661,8 +661,8 @@ __global__ void __launch_bounds__(Geo<T, L, LPC, E>::THREADS,
       // eigenvalue +1 (c = 0): exp(-i th) - 1 = (cos - 1) - i sin; -1 (c = 1): + i sin
       const T sh = -sg * q.z, sl = -sg * q.w;
       if constexpr (sizeof(T) == 4) {
-        v[m] = {q.x * vr + ((q.y * vr - sl * vi) - sh * vi),
-                q.x * vi + ((q.y * vi + sl * vr) + sh * vr)};
+        v[m] = {fma_t(q.x, vr, fma_t(-sh, vi, fma_t(-sl, vi, q.y * vr))),
+                fma_t(q.x, vi, fma_t(sh, vr, fma_t(sl, vr, q.y * vi)))};
       } else {
         v[m] = {q.x * vr - sh * vi, q.x * vi + sh * vr};
       }

@@ -309,7 +309,6 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
   const bool leader = tid == grp * G::GT;
 
   pdl_wait();
-  pdl_launch_next();
   const int upi = a0.n_lines / G::LPU;  // units of an instance
   // index checks of the debug build (no code otherwise): landing rows, staging, points of the
   // global arrays
@@ -351,6 +350,9 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
+  // only now: the next kernel's CTAs take tensor memory when they start and keep it while they
+  // wait for this kernel, so every CTA of this one must hold its own first
+  pdl_launch_next();
   const uint32_t tbase = *tslot;
   const uint32_t tpark =
       tbase + ((32u * (uint32_t)(warp & 3)) << 16) + G::PARK * (uint32_t)(warp >> 2);

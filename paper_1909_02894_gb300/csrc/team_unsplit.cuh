@@ -61,13 +61,15 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
   }
   if (PAIR && warp == 0) tmem_alloc(tslot, G::TCOLS);
   pdl_wait();
-  pdl_launch_next();
   int unit = blockIdx.x + gridDim.x * grp;
   if (leader && unit < n_units) issue(unit, 0);
   for (int t = tid; t < 15 * R2; t += G::THREADS) tw2s[t] = ldg_cx(a.tw + 15 * T + t);
   tmem_fence_before_sync();
   __syncthreads();
   tmem_fence_after_sync();
+  // only now: the next kernel's CTAs take tensor memory when they start and keep it while they
+  // wait for this kernel, so every CTA of this one must hold its own first
+  pdl_launch_next();
   const uint32_t tbase = PAIR ? *tslot : 0;
   const uint32_t tpark =
       tbase + ((32u * (uint32_t)(warp & 3)) << 16) + G::PARK * (uint32_t)(warp >> 2);

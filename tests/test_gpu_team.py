@@ -135,3 +135,33 @@ def test_short_lines_with_two_and_four_points_per_thread(nx, ny, prec):
     tol = 1e-12 if prec == D.DIRAC_C128 else 1e-6
     for k in ("norm", "norm_gamma", "energy"):
         assert abs(obs[k] - want[k]) <= tol * max(1.0, abs(want[k])), k
+
+
+@pytest.mark.parametrize("mass,conn", [(0.4, D.DIRAC_CONN_COVARIANT), (0.0, D.DIRAC_CONN_NONE)],
+                         ids=["curved", "no-half-step"])
+@pytest.mark.parametrize("nx,ny", [(64, 64), (64, 128), (128, 64), (128, 128)])
+def test_whole_steps_in_one_launch(nx, ny, mass, conn):
+    """Default complex64 steps of grids of 64- and 128-point axes (one launch for all steps of a
+    call) equal, bit for bit, the two passes per step of the larger shape, over several calls,
+    a change of dt and more steps than one launch takes, and match the oracle."""
+    w = grid(nx, ny)
+    w.mass = mass
+
+    def run(shape):
+        with D.Simulation(w, precision=D.DIRAC_C64, conn=conn) as s:
+            D.dirac_set_launch(s.ctx, shape, shape)
+            s.set_state(w.psi0)
+            n0 = D.dirac_launch_count(s.ctx)
+            for n, dt in ((1, w.dt), (2, w.dt), (5, 0.5 * w.dt), (1100, 0.5 * w.dt)):
+                s.step(n, dt)
+                if n == 5:
+                    mid = s.get_state()
+            return mid, s.get_state(), D.dirac_launch_count(s.ctx) - n0
+
+    mid, end, launches = run(0)
+    mid2, end2, launches2 = run(512)
+    assert np.array_equal(mid, mid2) and np.array_equal(end, end2)
+    assert launches < 40 < 2 * 1108 <= launches2
+    prob = oracle.Problem.from_workload(w, conn=conn)
+    ref = oracle.run(prob, w.psi0, w.dt, 3)
+    assert_parity(mid, oracle.run(prob, ref, 0.5 * w.dt, 5), w, TOL)
