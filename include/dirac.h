@@ -215,9 +215,9 @@ long dirac_krylov_iterations(const dirac_ctx *ctx);
  * pass. 256 or 512 plus
  * DIRAC_LAUNCH_ALT_RADIX selects the other radix schedule of the FFT passes, where the line
  * length has one: complex64 lines of 256..4096 points in radix-16 instead of radix-8
- * passes, complex128 lines of 512..2048 points in radix-8 instead of radix-16 passes (256
- * points: radix 16 instead of 8), each with its own lines-per-CTA pair (about 256 | 512
- * threads); elsewhere the flag is ignored.
+ * passes, complex128 lines of 256..1024 points in radix-16 instead of radix-8 passes (2048
+ * points: radix 8 instead of 16), each with its own lines-per-CTA pair; elsewhere the flag is
+ * ignored.
  * Used by the autotuner. DIRAC_EINVAL for other values. */
 #define DIRAC_LAUNCH_ALT_RADIX 0x10000
 dirac_status dirac_set_launch(dirac_ctx *ctx, int threads_x_pass, int threads_y_pass);

@@ -747,7 +747,6 @@ static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
 }
 
 // Spectral derivatives of the state: dx (normal layout) into scratch1, dy into scratch2.
-// Uses psiT as the transposed intermediate.
 template <typename T>
 static dirac_status state_derivatives(dirac_ctx* ctx) {
   cudaStream_t st = ctx->stream;
@@ -760,14 +759,13 @@ static dirac_status state_derivatives(dirac_ctx* ctx) {
   ay.out = (Q4<T>*)ctx->scratch2;
   ay.mult = (const Q4<T>*)ctx->dmult_y;
   CK(launch_line_pass<T>(ay, MODE_DERIV, 0, st), "y derivative");
-  // x derivative: psi -> psiT (transposed), then back to the normal layout in scratch1.
+  // x derivative: rows in the normal layout into scratch1.
   ax.in = (const Q4<T>*)ctx->psi;
-  ax.out = (Q4<T>*)ctx->psiT;
+  ax.out = (Q4<T>*)ctx->scratch1;
   ax.mult = (const Q4<T>*)ctx->dmult_x;
+  ax.store_normal = 1;
   CK(launch_line_pass<T>(ax, MODE_DERIV, 0, st), "x derivative");
-  CK(launch_transpose<T>((const Q4<T>*)ctx->psiT, (Q4<T>*)ctx->scratch1, ctx->nx, ctx->ny, st),
-     "transpose");
-  ctx->launches += 4;
+  ctx->launches += 3;
   return DIRAC_OK;
 }
 

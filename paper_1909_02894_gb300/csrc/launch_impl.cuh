@@ -8,11 +8,12 @@ namespace dgb {
 
 // Elements per thread: FP32 lines of 256 points or more use E = 8 (radix-8 passes; the
 // FFT state of a thread fits the 64-register budget of 1024 threads per SM without
-// spilling), and so do 64- and 128-point lines in both precisions and FP64 lines of 256
-// points; the other lengths use E = 16.
+// spilling), and so do 64- and 128-point lines in both precisions and FP64 lines of 256..1024
+// points (with the fused butterflies 1024^2 0.636 against 0.647 ms per step for E = 16, 512^2
+// 0.171 against 0.173, 2048^2 3.01 against 2.82); the other lengths use E = 16.
 template <typename T>
 constexpr int radix_e(int L) {
-  return ((sizeof(T) == 4 && L >= 256) || L == 64 || L == 128 || L == 256) ? 8 : 16;
+  return (sizeof(T) == 4 ? L >= 64 : L >= 64 && L <= 1024) ? 8 : 16;
 }
 // Elements per thread of the small shape of lines of 128 points or fewer: few, so that a small
 // grid's lines spread over many warps. Its pass is bound by the length of each warp's chain
@@ -23,11 +24,11 @@ constexpr int radix_e(int L) {
 // fill the GPU anyway, and fewer passes win: complex64 128 x 1024 E = 4 0.0136, E = 2 0.0155.
 constexpr int radix_small(int L, int n_lines) { return L > 128 ? 0 : n_lines <= 512 ? 2 : 4; }
 // The other radix schedule the autotuner may choose (0: none): FP32 lines of 256..4096
-// points in radix-16 passes, FP64 lines of 256 points in radix-16, of 512..2048 points in
+// points in radix-16 passes, FP64 lines of 256..1024 points in radix-16, of 2048 points in
 // radix-8 passes.
 template <typename T>
 constexpr int radix_alt(int L) {
-  return L < 256 ? 0 : sizeof(T) == 4 ? (L <= 4096 ? 16 : 0) : L == 256 ? 16 : L <= 2048 ? 8 : 0;
+  return L < 256 ? 0 : sizeof(T) == 4 ? (L <= 4096 ? 16 : 0) : L <= 1024 ? 16 : L <= 2048 ? 8 : 0;
 }
 
 template <typename T, int L, int LPC, int MODE, int E = radix_e<T>(L)>
@@ -62,7 +63,7 @@ static cudaError_t launch_one(const LinePassArgs<T>& a, cudaStream_t st) {
 // Lines per CTA, by precision:
 //   FP32 (E = 8 from 256 points): 256: 4|8, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1
 //     (256|512 threads, 512|1024 at 2048, 1024 at 4096)
-//   FP64 (E = 16 from 512 points): 256: 1|2, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1 (64..512 threads).
+//   FP64 (E = 16 from 2048 points): 256: 1|2, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1 (64..512 threads).
 //     The FP64 pass is bound by the FP64 units and its CTAs hold 128-162 registers per
 //     thread, so few CTAs fit an SM: small CTAs keep all 152 SMs evenly loaded. Measured on
 //     the strained-graphene grids (ms per step, opt 0 | opt 1): 512^2 0.203 | 0.199, 1024^2
@@ -143,11 +144,11 @@ static cudaError_t dispatch_alt(const LinePassArgs<T>& a0, int opt, cudaStream_t
       case 4096: return launch_one<T, 4096, 1, M, 16>(a, st);
       default: return cudaErrorInvalidValue;
     }
-  } else {  // radix 8: 2 L / 8 threads per line (256 points: radix 16)
+  } else {  // radix 16 up to 1024 points, radix 8 at 2048
     switch (a.L) {
       case 256: return big ? launch_one<T, 256, 2, M, 16>(a, st) : launch_one<T, 256, 1, M, 16>(a, st);
-      case 512: return big ? launch_one<T, 512, 4, M, 8>(a, st) : launch_one<T, 512, 2, M, 8>(a, st);
-      case 1024: return big ? launch_one<T, 1024, 2, M, 8>(a, st) : launch_one<T, 1024, 1, M, 8>(a, st);
+      case 512: return big ? launch_one<T, 512, 4, M, 16>(a, st) : launch_one<T, 512, 2, M, 16>(a, st);
+      case 1024: return big ? launch_one<T, 1024, 2, M, 16>(a, st) : launch_one<T, 1024, 1, M, 16>(a, st);
       case 2048: return launch_one<T, 2048, 1, M, 8>(a, st);
       default: return cudaErrorInvalidValue;
     }
