@@ -94,7 +94,8 @@ def fft_flops_per_point_step(nx, ny):
     return 20.0 * (np.log2(nx) + np.log2(ny)) + 76.0
 
 
-KERNEL_SOURCES = ("line_pass.cuh", "team_pass.cuh", "launch_impl.cuh", "common.cuh")
+KERNEL_SOURCES = ("line_pass.cuh", "team_pass.cuh", "team_launch.cuh", "launch_impl.cuh",
+                  "common.cuh")
 
 
 def kernel_hash():
