@@ -496,11 +496,8 @@ static dirac_status cn_apply(dirac_ctx* ctx, const void* v, void* out, double a)
   return unsplit_apply<T>(ctx, op);
 }
 
-// Copies `count` doubles of the device's dot products to the pinned host buffer and waits.
-static dirac_status krylov_fetch(dirac_ctx* ctx, size_t count) {
-  CK(cudaMemcpyAsync(ctx->k_host, ctx->k_dots, count * sizeof(double), cudaMemcpyDeviceToHost,
-                     ctx->stream),
-     "inner products");
+// Waits until the dot products, which the normalisation writes, are in the pinned host buffer.
+static dirac_status krylov_fetch(dirac_ctx* ctx) {
   CK(cudaStreamSynchronize(ctx->stream), "inner products");
   return DIRAC_OK;
 }
@@ -553,7 +550,7 @@ static dirac_status krylov_orthogonalise(dirac_ctx* ctx, int m) {
   CK(launch_gram_schmidt<T>(2, V, m, w, d1, np, ctx->k_partials, ctx->k_ticket, d2, kKrylovBlocks,
                             st),
      "combination");
-  CK(launch_normalise<T>(w, d2 + 1, np, st), "normalise");
+  CK(launch_normalise<T>(w, d0, 4 * m + 1, ctx->k_host, np, st), "normalise");
   ctx->launches += 4;
   return DIRAC_OK;
 }
@@ -604,9 +601,9 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
                             (Q4<T>*)v0, np, ctx->k_partials, ctx->k_ticket, ctx->k_dots,
                             kKrylovBlocks, st),
          "residual");
-      CK(launch_normalise<T>((Q4<T>*)v0, ctx->k_dots + 2, np, st), "normalise");
+      CK(launch_normalise<T>((Q4<T>*)v0, ctx->k_dots, 2, ctx->k_host, np, st), "normalise");
       ctx->launches += 2;
-      CKS(krylov_fetch(ctx, 2));
+      CKS(krylov_fetch(ctx));
       const double beta = sqrt(fmax(ctx->k_host[0], 0.0));
       if (cycle == 0) bnorm = sqrt(ctx->k_host[1]);
       if (beta <= tol * bnorm || beta == 0.0) {
@@ -620,7 +617,7 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
       for (int j = 0; j < m; ++j) {
         CKS(cn_apply<T>(ctx, ctx->kv[j], ctx->kv[j + 1], 0.5 * dt));
         CKS(krylov_orthogonalise<T>(ctx, j + 1));
-        CKS(krylov_fetch(ctx, 4 * (size_t)(j + 1) + 1));
+        CKS(krylov_fetch(ctx));
         const double* d = ctx->k_host;
         for (int i = 0; i <= j; ++i)
           H[(size_t)i * m + j] = cd(d[2 * i], d[2 * i + 1]) +

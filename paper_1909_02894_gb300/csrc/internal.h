@@ -214,7 +214,8 @@ cudaError_t launch_residual(int mode, const Q4<T>* rhs, const Q4<T>* x, Q4<T>* v
                             cudaStream_t st);
 // v *= inv[0] (device memory).
 template <typename T>
-cudaError_t launch_normalise(Q4<T>* v, const double* inv, size_t n, cudaStream_t st);
+cudaError_t launch_normalise(Q4<T>* v, const double* dots, int at, double* host, size_t n,
+                             cudaStream_t st);
 // out += sum_i coef_i V_i with complex FP64 coef (device array of 2 count doubles).
 template <typename T>
 cudaError_t launch_multi_axpy(Q4<T>* out, const Q4<T>* const* V, const double* coef, int count,
