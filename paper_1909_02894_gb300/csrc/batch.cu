@@ -77,7 +77,7 @@ struct dirac_batch {
   std::vector<std::pair<std::pair<int, int>, int>> graph_key;  // (class, capacity) list
   int graph_k = 0;
   long graph_kernels = 0;  // kernel nodes in the captured tick
-  cudaEvent_t fork = nullptr, tick_done = nullptr, admit = nullptr;
+  cudaEvent_t fork = nullptr, tick_done = nullptr;
   std::vector<cudaEvent_t> tick_events;  // per tick, recycled
   unsigned long long ticks = 0, ticks_done_seen = 0;
   int* d_err = nullptr;
@@ -484,7 +484,6 @@ dirac_status dirac_batch_create(size_t hbm_budget_bytes, dirac_precision precisi
     b->own_stream = (e == cudaSuccess);
   }
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-  if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->admit, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->tick_done, cudaEventDisableTiming);
   if (e == cudaSuccess) e = cudaEventRecord(b->tick_done, b->stream);
   if (e == cudaSuccess) e = cudaMalloc((void**)&b->d_err, sizeof(int));
@@ -516,16 +515,12 @@ dirac_status dirac_batch_submit(dirac_batch* b, dirac_ctx* inst, long n_steps, d
   const size_t need = dgb_footprint_bytes(inst->nx, inst->ny, inst->prec);
   if (b->used + need > b->budget)
     return bfail(b, DIRAC_ENOMEM, "device-memory budget of the batch exhausted");
+  // the context's work so far must be ordered before the batch's
+  BCK(cudaStreamSynchronize(inst->stream), "submit");
   if (dt != inst->dt_cached) {
     dirac_status st = dgb_tables_for_dt(inst, dt);
     if (st != DIRAC_OK) return bfail(b, st, inst->err);
-  }
-  // the context's work so far comes before the batch's: on the device, as waiting for it here
-  // left the GPU idle between the uploads of contexts submitted one after another (32 contexts,
-  // 32 steps: 5.36 -> 5.08 ms with set_state and get_state)
-  if (inst->stream != b->stream) {
-    BCK(cudaEventRecord(b->admit, inst->stream), "submit");
-    BCK(cudaStreamWaitEvent(b->stream, b->admit, 0), "submit");
+    BCK(cudaStreamSynchronize(inst->stream), "submit");
   }
   int s = -1;
   for (int i = 0; i < (int)b->slots.size(); ++i)
@@ -712,7 +707,6 @@ void dirac_batch_destroy(dirac_batch* b) {
   for (auto& kv : b->classes) free_class(kv.second);
   for (cudaEvent_t e : b->tick_events) cudaEventDestroy(e);
   if (b->fork) cudaEventDestroy(b->fork);
-  if (b->admit) cudaEventDestroy(b->admit);
   if (b->tick_done) cudaEventDestroy(b->tick_done);
   if (b->d_err) cudaFree(b->d_err);
   if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
