@@ -12,7 +12,11 @@ namespace dgb {
 
 // Kernel launch with, if `pdl`, programmatic stream serialization: the kernel may be scheduled
 // while its predecessor in the stream still runs (it calls pdl_wait before it touches memory),
-// and, if cluster > 1, that cluster size.
+// and, if cluster > 1, that cluster size. Loads through the read-only path (__ldg, ld.global.nc)
+// need data that no kernel writes while the loading one is resident, which pdl_wait does not
+// change: a kernel launched with `pdl` takes that path for tables only (coefficients,
+// twiddles, multipliers, instance pointers; their producers are launched without it and are
+// complete before), and reads states and terms by ordinary loads or bulk copies.
 template <typename... P, typename... A>
 inline cudaError_t launch_pdl(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
                               cudaStream_t st, bool pdl, int cluster, A&&... args) {

@@ -106,6 +106,17 @@ __device__ __forceinline__ Q4<float> ld_stream_q4(const Q4<float>* p) {
                : "l"(p));
   return v;
 }
+// The same through the coherent path, for arrays that an earlier kernel of the chain writes (see
+// launch_pdl: this kernel may be resident while that one still runs, so its data is not
+// read-only for this kernel's lifetime, which ld.global.nc asks for).
+__device__ __forceinline__ Q4<float> ld_chain_q4(const Q4<float>* p) {
+  Q4<float> v;
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p)
+               : "memory");
+  return v;
+}
 __device__ __forceinline__ float ld_stream(const float* p) {
   float v;
   asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));

@@ -166,11 +166,11 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
       if constexpr (PHASE == 2) {
         if (a.base) {
 #pragma unroll
-          for (int mm = 0; mm < 4; ++mm) qb[mm] = ld_stream_q4(a.base + gz(g0 + T * mm));
+          for (int mm = 0; mm < 4; ++mm) qb[mm] = ld_chain_q4(a.base + gz(g0 + T * mm));
         }
 #pragma unroll
         for (int mm = 0; mm < 4; ++mm) {
-          const Q4<float> s = ld_stream_q4(a.s_other + gz(g0 + T * mm));
+          const Q4<float> s = ld_chain_q4(a.s_other + gz(g0 + T * mm));
           o[4 * mm] = s.x;
           o[4 * mm + 1] = s.y;
           o[4 * mm + 2] = s.z;
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
         if (a.prev) {
           Q4<float> q[4];
 #pragma unroll
-          for (int mm = 0; mm < 4; ++mm) q[mm] = ld_stream_q4(a.prev + gz(g0 + T * mm));
+          for (int mm = 0; mm < 4; ++mm) q[mm] = ld_chain_q4(a.prev + gz(g0 + T * mm));
 #pragma unroll
           for (int mm = 0; mm < 4; ++mm) {
             o[4 * mm] += a.beta_prev * q[mm].x;
