@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <complex>
@@ -523,31 +524,32 @@ static dirac_status krylov_combine(dirac_ctx* ctx, void* out,
 
 // One Arnoldi step after w = G V_j is in kv[j + 1]: classical Gram-Schmidt twice against V_0..V_j
 // and the norm, everything on the device. dots: h (2 m values), second h (2 m), norm^2, 1/norm.
+// fp64: the sums of complex64 vectors in FP64.
 template <typename T>
-static dirac_status krylov_orthogonalise(dirac_ctx* ctx, int m) {
+static dirac_status krylov_orthogonalise(dirac_ctx* ctx, int m, bool fp64) {
   cudaStream_t st = ctx->stream;
   const size_t np = npts(ctx);
   const auto V = (const Q4<T>* const*)ctx->k_vptr;
   Q4<T>* w = (Q4<T>*)ctx->kv[m];
   double *d0 = ctx->k_dots, *d1 = d0 + 2 * m, *d2 = d1 + 2 * m;
-  CK(launch_gram_schmidt<T>(0, V, m, w, nullptr, np, ctx->k_partials, ctx->k_ticket, d0,
+  CK(launch_gram_schmidt<T>(0, fp64, V, m, w, nullptr, np, ctx->k_partials, ctx->k_ticket, d0,
                             kKrylovBlocks, st),
      "inner products");
   if (m <= 4) {
     // the first combination and the second products in one sweep
-    CK(launch_gram_schmidt<T>(1, V, m, w, d0, np, ctx->k_partials, ctx->k_ticket, d1,
+    CK(launch_gram_schmidt<T>(1, fp64, V, m, w, d0, np, ctx->k_partials, ctx->k_ticket, d1,
                               kKrylovBlocks, st),
        "inner products");
   } else {
-    CK(launch_gram_schmidt<T>(2, V, m, w, d0, np, ctx->k_partials, ctx->k_ticket, d2,
+    CK(launch_gram_schmidt<T>(2, fp64, V, m, w, d0, np, ctx->k_partials, ctx->k_ticket, d2,
                               kKrylovBlocks, st),
        "combination");
-    CK(launch_gram_schmidt<T>(0, V, m, w, nullptr, np, ctx->k_partials, ctx->k_ticket, d1,
+    CK(launch_gram_schmidt<T>(0, fp64, V, m, w, nullptr, np, ctx->k_partials, ctx->k_ticket, d1,
                               kKrylovBlocks, st),
        "inner products");
     ctx->launches += 1;
   }
-  CK(launch_gram_schmidt<T>(2, V, m, w, d1, np, ctx->k_partials, ctx->k_ticket, d2, kKrylovBlocks,
+  CK(launch_gram_schmidt<T>(2, fp64, V, m, w, d1, np, ctx->k_partials, ctx->k_ticket, d2, kKrylovBlocks,
                             st),
      "combination");
   CK(launch_normalise<T>(w, d0, 4 * m + 1, ctx->k_host, np, st), "normalise");
@@ -615,9 +617,16 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
       g[0] = beta;
       int kdim = 0;
       for (int j = 0; j < m; ++j) {
-        CKS(cn_apply<T>(ctx, ctx->kv[j], ctx->kv[j + 1], 0.5 * dt));
-        CKS(krylov_orthogonalise<T>(ctx, j + 1));
-        CKS(krylov_fetch(ctx));
+        // FP32 sums hold |w| up to about 1e19; a larger one (a time step of that many periods of
+        // the fastest mode) overflows them, and the vector is made again with FP64 sums
+        for (bool fp64 : {false, true}) {
+          CKS(cn_apply<T>(ctx, ctx->kv[j], ctx->kv[j + 1], 0.5 * dt));
+          CKS(krylov_orthogonalise<T>(ctx, j + 1, fp64));
+          CKS(krylov_fetch(ctx));
+          if (sizeof(T) == 8 || std::all_of(ctx->k_host, ctx->k_host + 4 * (j + 1) + 1,
+                                            [](double v) { return isfinite(v); }))
+            break;
+        }
         const double* d = ctx->k_host;
         for (int i = 0; i <= j; ++i)
           H[(size_t)i * m + j] = cd(d[2 * i], d[2 * i + 1]) +

@@ -206,8 +206,9 @@ cudaError_t launch_max_b(const double* a1, const double* a2, const double* sxinv
 // kind 1: w -= sum_i coef_i V_i, then dots as for kind 0 (count <= 4);
 // kind 2: w -= sum_i coef_i V_i, then dots[0] = <w, w>, dots[1] = 1 / sqrt(dots[0]) (1 unless
 // dots[0] > 0).
+// fp64: complex64 vectors summed in FP64 too (slower, for squares beyond the FP32 range).
 template <typename T>
-cudaError_t launch_gram_schmidt(int kind, const Q4<T>* const* V, int count, Q4<T>* w,
+cudaError_t launch_gram_schmidt(int kind, bool fp64, const Q4<T>* const* V, int count, Q4<T>* w,
                                 const double* coef, size_t n, double* partials, unsigned* ticket,
                                 double* dots, int n_blocks, cudaStream_t st);
 // v = 2 (rhs - x) (mode 0) or rhs - v (mode 1); dots[0] = <v, v>, dots[1] = <rhs, rhs> (mode 0),

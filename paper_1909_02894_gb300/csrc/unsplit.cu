@@ -164,8 +164,8 @@ struct DotAcc<float> {
     return (threadIdx.x & 31) == 0 ? d + ((double)s + ((double)c + (double)g)) : 0.0;
   }
 };
-template <typename T>
-__device__ __forceinline__ void dot_point(DotAcc<T>& re, DotAcc<T>& im, const Q4<T>& a,
+template <typename A, typename T>
+__device__ __forceinline__ void dot_point(DotAcc<A>& re, DotAcc<A>& im, const Q4<T>& a,
                                           const Q4<T>& b) {
   re.add(a.x, b.x);
   re.add(a.y, b.y);
@@ -232,14 +232,16 @@ constexpr int kChunk = 4;  // vectors whose products a thread accumulates at onc
 
 // KIND 0: dots of the chunk's vectors with w. KIND 1 (one chunk): w -= sum coef_i V_i first.
 // KIND 2 (grid.y = 1): w -= sum coef_i V_i over all `count` vectors, then the norm of w.
-template <typename T, int KIND>
+// Products and norms in accumulators of type A: T's own, or FP64 for complex64 vectors whose
+// squares left the FP32 range.
+template <typename T, typename A, int KIND>
 __global__ void __launch_bounds__(TPB) k_gram_schmidt(const Q4<T>* const* V, int count, Q4<T>* w,
                                                       const double* coef, size_t n,
                                                       double* partials, unsigned* ticket,
                                                       double* dots) {
   const int first = KIND == 0 ? blockIdx.y * kChunk : 0;
   const int c = KIND == 2 ? count : min(kChunk, count - first);
-  DotAcc<T> acc[KIND == 2 ? 1 : 2 * kChunk];  // re, im of each product; the norm
+  DotAcc<A> acc[KIND == 2 ? 1 : 2 * kChunk];  // re, im of each product; the norm
   int since = 0;
   const size_t stride = (size_t)gridDim.x * blockDim.x;
   const bool flushed = n > 8 * stride;
@@ -347,19 +349,29 @@ static int sum_blocks(size_t n, int n_max) {
   return (int)(b < (size_t)n_max ? b : (size_t)n_max);
 }
 
+template <typename T, typename A>
+static void gram_schmidt_as(int kind, const Q4<T>* const* V, int count, Q4<T>* w,
+                            const double* coef, size_t n, double* partials, unsigned* ticket,
+                            double* dots, int n_blocks, cudaStream_t st) {
+  if (kind == 0)
+    k_gram_schmidt<T, A, 0><<<dim3(n_blocks, (count + kChunk - 1) / kChunk), TPB, 0, st>>>(
+        V, count, w, coef, n, partials, ticket, dots);
+  else if (kind == 1)
+    k_gram_schmidt<T, A, 1><<<n_blocks, TPB, 0, st>>>(V, count, w, coef, n, partials, ticket, dots);
+  else
+    k_gram_schmidt<T, A, 2><<<n_blocks, TPB, 0, st>>>(V, count, w, coef, n, partials, ticket, dots);
+}
+
 template <typename T>
-cudaError_t launch_gram_schmidt(int kind, const Q4<T>* const* V, int count, Q4<T>* w,
+cudaError_t launch_gram_schmidt(int kind, bool fp64, const Q4<T>* const* V, int count, Q4<T>* w,
                                 const double* coef, size_t n, double* partials, unsigned* ticket,
                                 double* dots, int n_blocks, cudaStream_t st) {
   if (count < 1 || (kind == 1 && count > kChunk)) return cudaErrorInvalidValue;
   n_blocks = sum_blocks(n, n_blocks);
-  if (kind == 0)
-    k_gram_schmidt<T, 0><<<dim3(n_blocks, (count + kChunk - 1) / kChunk), TPB, 0, st>>>(
-        V, count, w, coef, n, partials, ticket, dots);
-  else if (kind == 1)
-    k_gram_schmidt<T, 1><<<n_blocks, TPB, 0, st>>>(V, count, w, coef, n, partials, ticket, dots);
+  if (fp64)
+    gram_schmidt_as<T, double>(kind, V, count, w, coef, n, partials, ticket, dots, n_blocks, st);
   else
-    k_gram_schmidt<T, 2><<<n_blocks, TPB, 0, st>>>(V, count, w, coef, n, partials, ticket, dots);
+    gram_schmidt_as<T, T>(kind, V, count, w, coef, n, partials, ticket, dots, n_blocks, st);
   return cudaGetLastError();
 }
 
@@ -470,7 +482,7 @@ bool bessel_j_series(double x, int n, double* out) {
       const Q4<T>*, const Q4<T>*, const double*, const double*, const double*, const double*, \
       const double*, const double*, int, int, double, double, const Q4<T>*, double, double,  \
       const Q4<T>*, double, Q4<T>*, cudaStream_t);                                           \
-  template cudaError_t launch_gram_schmidt<T>(int, const Q4<T>* const*, int, Q4<T>*,          \
+  template cudaError_t launch_gram_schmidt<T>(int, bool, const Q4<T>* const*, int, Q4<T>*,    \
                                               const double*, size_t, double*, unsigned*,      \
                                               double*, int, cudaStream_t);                    \
   template cudaError_t launch_residual<T>(int, const Q4<T>*, const Q4<T>*, Q4<T>*, size_t,    \
