@@ -193,7 +193,8 @@ dirac_status dirac_set_poly_degree(dirac_ctx *ctx, int degree);
  * |G~ psi|; 0 = default: 1e-14 for complex128, 3e-7 for complex64), Krylov dimension
  * `restart` (1..100, default 20; restart + 1 state-sized device arrays, allocated on the
  * next dirac_step) and at most max_restarts restarts per step (default 100). A step whose
- * solve does not converge returns DIRAC_ENOCONV and leaves the state invalid. */
+ * solve does not converge returns DIRAC_ENOCONV and leaves the state invalid, and so does
+ * DIRAC_ETIMEOUT when a bounded device wait ran out under the solve. */
 dirac_status dirac_set_krylov(dirac_ctx *ctx, double tol, int restart, int max_restarts);
 
 /* Total Arnoldi steps of Scheme I on this context since its creation. */
@@ -232,11 +233,13 @@ dirac_status dirac_set_launch(dirac_ctx *ctx, int threads_x_pass, int threads_y_
 dirac_status dirac_autotune(dirac_ctx *ctx, int reps, int *threads_x, int *threads_y);
 
 /* Test hook for failure detection: in the next dirac_step -- or, for a context submitted
- * to a batch, in the first tick that steps it -- the team pass's bulk-copy waits
- * expect 16 bytes that never arrive, so each wait runs out after its bound (about 1.5 s),
- * the kernel returns early and the next synchronising call (dirac_synchronize, or
- * dirac_batch_poll / dirac_batch_synchronize) reports DIRAC_ETIMEOUT; the context stays
- * usable (set the state again). No effect on the other launch shapes. */
+ * to a batch, in the first tick that steps it -- the team pass's bulk-copy waits (for the
+ * polynomial schemes and Scheme I those of the first operator application, where its passes
+ * are team passes) expect 16 bytes that never arrive, so each wait runs out after its bound
+ * (about 1.5 s), the kernel returns early and the next synchronising call
+ * (dirac_synchronize, or dirac_batch_poll / dirac_batch_synchronize; Scheme I's dirac_step
+ * itself) reports DIRAC_ETIMEOUT; the context stays usable (set the state again). No effect
+ * on the other launch shapes. */
 dirac_status dirac_test_timeout_next_step(dirac_ctx *ctx);
 
 /* Host-side fault injection for failure-detection tests (no GPU fault involved): with the

@@ -9,6 +9,7 @@
 
 // inner products of one Arnoldi step: 4 per basis vector (at most 100), norms
 constexpr size_t kKrylovHost = 1024;
+constexpr size_t kKrylovErr = kKrylovHost / 2 - 1;  // the device error flag in k_host
 
 struct dirac_ctx {
   int nx = 0, ny = 0;
@@ -61,7 +62,8 @@ struct dirac_ctx {
   double* k_coef = nullptr;         // combination coefficients (device)
   double* k_dots = nullptr;         // inner products (device), kKrylovHost values
   unsigned* k_ticket = nullptr;     // counter of the inner products' last block
-  double* k_host = nullptr;         // pinned: inner products (first half), coefficients (second)
+  double* k_host = nullptr;         // pinned: inner products and the error flag (first half),
+                                    // coefficients (second)
   // complex64 axes of 256 points or more: the step tables (x at dt and dt/2, y) in the
   // order of team_perm, for the team pass
   void *mult_px = nullptr, *mult_py = nullptr, *mult_pxh = nullptr;

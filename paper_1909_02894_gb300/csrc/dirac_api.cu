@@ -315,6 +315,8 @@ static dirac_status unsplit_apply_team(dirac_ctx* ctx, const UnsplitOp& op) {
       a.in = (const Q4<float>*)op.in;
       a.out = (Q4<float>*)ctx->scratch1;
       a.out_in = (Q4<float>*)op.in_t;
+      a.test_extra_tx = ctx->test_timeout_next;
+      ctx->test_timeout_next = 0;
     } else {
       a.in = (const Q4<float>*)op.in_t;
       a.out = (Q4<float>*)op.out;
@@ -340,6 +342,7 @@ static dirac_status unsplit_apply_team(dirac_ctx* ctx, const UnsplitOp& op) {
 template <typename T>
 static dirac_status unsplit_apply(dirac_ctx* ctx, const UnsplitOp& op) {
   cudaStream_t st = ctx->stream;
+  ctx->test_timeout_next = 0;  // no bounded waits here
   LinePassArgs<T> ax = pass_args<T>(ctx, 0), ay = pass_args<T>(ctx, 1);
   ax.in = (const Q4<T>*)op.in;
   ax.out = (Q4<T>*)ctx->scratch1;
@@ -498,9 +501,11 @@ static dirac_status cn_apply(dirac_ctx* ctx, const void* v, void* out, double a)
 }
 
 // Waits until the dot products, which the normalisation writes, are in the pinned host buffer.
+// DIRAC_ETIMEOUT if a bounded wait ran out in the operator's passes: what they left is not to
+// be iterated on.
 static dirac_status krylov_fetch(dirac_ctx* ctx) {
   CK(cudaStreamSynchronize(ctx->stream), "inner products");
-  return DIRAC_OK;
+  return ctx->k_host[kKrylovErr] != 0.0 ? device_error(ctx) : DIRAC_OK;
 }
 
 // out += sum_{i < c.size()} c_i V_i
@@ -552,7 +557,8 @@ static dirac_status krylov_orthogonalise(dirac_ctx* ctx, int m, bool fp64) {
   CK(launch_gram_schmidt<T>(2, fp64, V, m, w, d1, np, ctx->k_partials, ctx->k_ticket, d2, kKrylovBlocks,
                             st),
      "combination");
-  CK(launch_normalise<T>(w, d0, 4 * m + 1, ctx->k_host, np, st), "normalise");
+  CK(launch_normalise<T>(w, d0, 4 * m + 1, ctx->d_err, ctx->k_host, ctx->k_host + kKrylovErr, np,
+                         st), "normalise");
   ctx->launches += 4;
   return DIRAC_OK;
 }
@@ -603,7 +609,8 @@ static dirac_status step_cn(dirac_ctx* ctx, long n, double dt) {
                             (Q4<T>*)v0, np, ctx->k_partials, ctx->k_ticket, ctx->k_dots,
                             kKrylovBlocks, st),
          "residual");
-      CK(launch_normalise<T>((Q4<T>*)v0, ctx->k_dots, 2, ctx->k_host, np, st), "normalise");
+      CK(launch_normalise<T>((Q4<T>*)v0, ctx->k_dots, 2, ctx->d_err, ctx->k_host,
+                             ctx->k_host + kKrylovErr, np, st), "normalise");
       ctx->launches += 2;
       CKS(krylov_fetch(ctx));
       const double beta = sqrt(fmax(ctx->k_host[0], 0.0));

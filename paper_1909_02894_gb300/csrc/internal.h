@@ -217,10 +217,11 @@ template <typename T>
 cudaError_t launch_residual(int mode, const Q4<T>* rhs, const Q4<T>* x, Q4<T>* v, size_t n,
                             double* partials, unsigned* ticket, double* dots, int n_blocks,
                             cudaStream_t st);
-// v *= inv[0] (device memory).
+// v *= dots[at] (device memory); dots[0..at) and the device error flag *err also go to host and
+// *host_err (pinned host memory).
 template <typename T>
-cudaError_t launch_normalise(Q4<T>* v, const double* dots, int at, double* host, size_t n,
-                             cudaStream_t st);
+cudaError_t launch_normalise(Q4<T>* v, const double* dots, int at, const int* err, double* host,
+                             double* host_err, size_t n, cudaStream_t st);
 // out += sum_i coef_i V_i with complex FP64 coef (device array of 2 count doubles).
 template <typename T>
 cudaError_t launch_multi_axpy(Q4<T>* out, const Q4<T>* const* V, const double* coef, int count,

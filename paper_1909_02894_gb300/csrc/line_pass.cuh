@@ -101,6 +101,7 @@ struct UnsplitArgs {
   const Q4<float>* u_store;
   int store_normal;  // 1: out is [n_lines][L], 0: transposed
   int* err;
+  unsigned test_extra_tx;  // test hook, as in LinePassArgs
 };
 
 // Batched launches: a block (or group) of lines belongs to instance `k`; take that

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(TGeo<L, LPC, PAIR>::THREADS, TGeo<L, LPC, PAIR
   };
   auto issue = [&](int unit, int h) {
     fence_proxy_async_smem();
-    mbar_arrive_expect_tx(bar, (uint32_t)(G::LG * L * 16));
+    mbar_arrive_expect_tx(bar, (uint32_t)(G::LG * L * 16) + a.test_extra_tx);
 #pragma unroll 1
     for (int l = 0; l < G::LG; ++l)
       bulk_copy_g2s(tsm + (grp * G::LG + l) * G::LINE_BYTES,

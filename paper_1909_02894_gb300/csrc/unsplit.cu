@@ -310,13 +310,16 @@ __global__ void __launch_bounds__(TPB) k_residual(int mode, const Q4<T>* rhs, co
   grid_sums<2, true>(acc, true, 2, 0, 2, partials, ticket, dots);
 }
 
-// v *= dots[at]; dots[0..at) go to pinned host memory, written from here as a copy of its own
-// behind this kernel delayed the host, which waits for these values (Scheme I at 512^2, 4 steps
-// with set_state and get_state: 1.43 -> 1.31 ms).
+// v *= dots[at]; dots[0..at) and the device error flag go to pinned host memory, written from
+// here as a copy of its own behind this kernel delayed the host, which waits for these values
+// (Scheme I at 512^2, 4 steps with set_state and get_state: 1.43 -> 1.31 ms).
 template <typename T>
-__global__ void k_normalise(Q4<T>* v, const double* dots, int at, double* host, size_t n) {
-  if (blockIdx.x == 0)
+__global__ void k_normalise(Q4<T>* v, const double* dots, int at, const int* err, double* host,
+                            double* host_err, size_t n) {
+  if (blockIdx.x == 0) {
     for (int t = threadIdx.x; t < at; t += TPB) host[t] = dots[t];
+    if (threadIdx.x == 0) *host_err = *err;
+  }
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   const T c = (T)dots[at];
@@ -385,9 +388,9 @@ cudaError_t launch_residual(int mode, const Q4<T>* rhs, const Q4<T>* x, Q4<T>* v
 }
 
 template <typename T>
-cudaError_t launch_normalise(Q4<T>* v, const double* dots, int at, double* host, size_t n,
-                             cudaStream_t st) {
-  k_normalise<T><<<blocks_for(n), TPB, 0, st>>>(v, dots, at, host, n);
+cudaError_t launch_normalise(Q4<T>* v, const double* dots, int at, const int* err, double* host,
+                             double* host_err, size_t n, cudaStream_t st) {
+  k_normalise<T><<<blocks_for(n), TPB, 0, st>>>(v, dots, at, err, host, host_err, n);
   return cudaGetLastError();
 }
 
@@ -487,8 +490,8 @@ bool bessel_j_series(double x, int n, double* out) {
                                               double*, int, cudaStream_t);                    \
   template cudaError_t launch_residual<T>(int, const Q4<T>*, const Q4<T>*, Q4<T>*, size_t,    \
                                           double*, unsigned*, double*, int, cudaStream_t);    \
-  template cudaError_t launch_normalise<T>(Q4<T>*, const double*, int, double*, size_t,       \
-                                           cudaStream_t);                                     \
+  template cudaError_t launch_normalise<T>(Q4<T>*, const double*, int, const int*, double*,   \
+                                           double*, size_t, cudaStream_t);                    \
   template cudaError_t launch_multi_axpy<T>(Q4<T>*, const Q4<T>* const*, const double*, int,  \
                                             size_t, cudaStream_t);
 INST(float)
