@@ -166,11 +166,12 @@ __device__ __forceinline__ Q4<T> apply_u(Q4<T> u, Q4<T> p) {
 // (u10, d11).
 template <typename T>
 __device__ __forceinline__ Q4<T> apply_u_general(Q4<T> r0, Q4<T> r1, Q4<T> p) {
+  // (fused explicitly, as cmul is, so that the kernels of both layouts round alike)
   const T a = p.x, b = p.y, c = p.z, d = p.w;
-  return {a + (r0.x * a - r0.y * b + r0.z * c - r0.w * d),
-          b + (r0.x * b + r0.y * a + r0.z * d + r0.w * c),
-          c + (r1.x * a - r1.y * b + r1.z * c - r1.w * d),
-          d + (r1.x * b + r1.y * a + r1.z * d + r1.w * c)};
+  return {a + fma_t(-r0.w, d, fma_t(r0.z, c, fma_t(r0.x, a, -(r0.y * b)))),
+          b + fma_t(r0.w, c, fma_t(r0.z, d, fma_t(r0.y, a, r0.x * b))),
+          c + fma_t(-r1.w, d, fma_t(r1.z, c, fma_t(r1.x, a, -(r1.y * b)))),
+          d + fma_t(r1.w, c, fma_t(r1.z, d, fma_t(r1.y, a, r1.x * b)))};
 }
 
 }  // namespace dgb

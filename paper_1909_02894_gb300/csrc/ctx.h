@@ -50,7 +50,7 @@ struct dirac_ctx {
   bool pot_use[3] = {false, false, false};  // V, Ax, Ay set
   bool has_pot = false;
   void *ug = nullptr, *ug2 = nullptr;  // U and U^2, two Q4 per point
-  void *ug_t = nullptr, *ug2_t = nullptr;  // the same, transposed (y passes that apply them)
+  bool ug_transposed = false;          // their layout: transposed for y passes that apply them
   // Scheme I: Krylov solver settings and buffers
   double krylov_tol = 0.0;  // 0 = precision default
   int krylov_m = 20, krylov_restarts = 100;

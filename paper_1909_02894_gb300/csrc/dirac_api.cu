@@ -134,9 +134,18 @@ static LinePassArgs<T> pass_args(dirac_ctx* ctx, int axis) {
   return a;
 }
 
+// Scheme II with static potentials: whether the y pass' store applies the half steps that follow
+// it (a team pass). The matrices are then kept in the transposed layout only; the launch shape
+// decides it, so a step remakes them when dirac_set_launch or the autotuner changed that.
+static bool pot_in_y_pass(const dirac_ctx* ctx) {
+  return ctx->has_pot && ctx->scheme == DIRAC_SCHEME_II && ctx->prec == DIRAC_C64 &&
+         team_length(ctx->ny) && pass_opt(ctx, ctx->threads_y, ctx->ny, ctx->nx) == 2;
+}
+
 template <typename T>
 static dirac_status tables_for_dt(dirac_ctx* ctx, double dt) {
   cudaStream_t st = ctx->stream;
+  ctx->dt_cached = 0.0;  // until they are complete
   const bool sym = ctx->scheme == DIRAC_SCHEME_II_SYMMETRIC;
   const bool need_u2n = ctx->scheme != DIRAC_SCHEME_II;  // U^2 applied in the normal layout
   if (sym && !ctx->mult_xh)
@@ -155,18 +164,12 @@ static dirac_status tables_for_dt(dirac_ctx* ctx, double dt) {
   if (ctx->has_pot) {
     if (!ctx->ug) CK(dalloc(ctx, &ctx->ug, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
     if (!ctx->ug2) CK(dalloc(ctx, &ctx->ug2, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
-    const bool tr = ctx->scheme == DIRAC_SCHEME_II && sizeof(T) == 4 && team_length(ctx->ny);
-    if (tr && !ctx->ug_t)
-      CK(dalloc(ctx, &ctx->ug_t, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
-    if (tr && !ctx->ug2_t)
-      CK(dalloc(ctx, &ctx->ug2_t, 2 * npts(ctx) * sizeof(Q4<T>)), "allocate half-step");
+    ctx->ug_transposed = pot_in_y_pass(ctx);
     CK(launch_halfstep_general<T>(ctx->a1, ctx->a2, ctx->meff, ctx->omx, ctx->omy,
                                   ctx->pot_use[0] ? ctx->pot_v : nullptr,
                                   ctx->pot_use[1] ? ctx->pot_ax : nullptr,
                                   ctx->pot_use[2] ? ctx->pot_ay : nullptr, ctx->nx, ctx->ny, dt,
-                                  (Q4<T>*)ctx->ug, (Q4<T>*)ctx->ug2,
-                                  tr ? (Q4<T>*)ctx->ug_t : nullptr,
-                                  tr ? (Q4<T>*)ctx->ug2_t : nullptr, st),
+                                  ctx->ug_transposed, (Q4<T>*)ctx->ug, (Q4<T>*)ctx->ug2, st),
        "half-step matrices with potentials");
     ctx->launches += 1;
   }
@@ -198,9 +201,11 @@ template <typename T>
 static dirac_status apply_half(dirac_ctx* ctx, void* psi, bool squared) {
   const size_t np = npts(ctx);
   if (ctx->has_pot) {
-    CK(launch_apply_ug<T>((Q4<T>*)psi, (const Q4<T>*)(squared ? ctx->ug2 : ctx->ug), np,
-                          ctx->stream),
-       "half step");
+    const Q4<T>* ug = (const Q4<T>*)(squared ? ctx->ug2 : ctx->ug);
+    if (ctx->ug_transposed)
+      CK(launch_apply_ug_t<T>((Q4<T>*)psi, ug, ctx->nx, ctx->ny, ctx->stream), "half step");
+    else
+      CK(launch_apply_ug<T>((Q4<T>*)psi, ug, np, ctx->stream), "half step");
   } else if (!ctx->u_identity) {
     CK(launch_apply_u<T>((Q4<T>*)psi, (const Q4<T>*)(squared ? ctx->u2_n : ctx->u_n), np,
                          ctx->stream),
@@ -709,7 +714,7 @@ static dirac_status step_small(dirac_ctx* ctx, long n, bool* done) {
 
 template <typename T>
 static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
-  if (dt != ctx->dt_cached) {
+  if (dt != ctx->dt_cached || (ctx->has_pot && ctx->ug_transposed != pot_in_y_pass(ctx))) {
     dirac_status s = tables_for_dt<T>(ctx, dt);
     if (s != DIRAC_OK) return s;
   }
@@ -741,7 +746,7 @@ static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
   // that is a team pass, else by their own kernel too
   const bool fused = !ctx->has_pot;
   const int opt_y = pass_opt(ctx, ctx->threads_y, ctx->ny, ctx->nx);
-  const bool fused_pot = !fused && sizeof(T) == 4 && opt_y == 2 && team_length(ctx->ny);
+  const bool fused_pot = !fused && ctx->ug_transposed;
   if (!fused) CKS(apply_half<T>(ctx, ctx->psi, false));
   for (long s = 0; s < n; ++s) {
     ax.u_load = (fused && s == 0 && !ctx->u_identity) ? (const Q4<T>*)ctx->u_n : nullptr;
@@ -751,7 +756,7 @@ static dirac_status step_impl(dirac_ctx* ctx, long n, double dt) {
     ay.u_load = nullptr;
     ay.u_store = (!fused || ctx->u_identity) ? nullptr
                                              : (const Q4<T>*)(s + 1 == n ? ctx->u_t : ctx->u2_t);
-    ay.ug_store = fused_pot ? (const Q4<T>*)(s + 1 == n ? ctx->ug_t : ctx->ug2_t) : nullptr;
+    ay.ug_store = fused_pot ? (const Q4<T>*)(s + 1 == n ? ctx->ug : ctx->ug2) : nullptr;
     CK(launch_line_pass<T>(ay, MODE_STEP, opt_y, ctx->stream), "y pass");
     ctx->launches += 2;
     if (!fused && !fused_pot) CKS(apply_half<T>(ctx, ctx->psi, s + 1 < n));

@@ -135,18 +135,21 @@ cudaError_t launch_team_twiddles(int n, Cx<T>* tw, cudaStream_t st);
 template <typename T>
 cudaError_t launch_deriv_mult(int n, double a, Q4<T>* mult, cudaStream_t st);
 
-// Half step with static potentials: general complex U and U^2 per point (normal layout,
-// two Q4 per point holding U - I: (d00, u01), (u10, d11)) and, where ug_t, ug2_t are not
-// null, the same in the transposed layout; V, Ax, Ay may be null (0).
+// Half step with static potentials: general complex U and U^2 per point (two Q4 per point
+// holding U - I: (d00, u01), (u10, d11)), in the normal or the transposed layout; V, Ax, Ay may
+// be null (0).
 template <typename T>
 cudaError_t launch_halfstep_general(const double* a1, const double* a2, const double* meff,
                                     const double* omx, const double* omy, const double* V,
                                     const double* Ax, const double* Ay, int nx, int ny,
-                                    double dt, Q4<T>* ug, Q4<T>* ug2, Q4<T>* ug_t, Q4<T>* ug2_t,
+                                    double dt, bool transposed, Q4<T>* ug, Q4<T>* ug2,
                                     cudaStream_t st);
-// psi <- U psi for such a general U.
+// psi <- U psi (psi in the normal layout) for such a general U in the normal and in the
+// transposed layout.
 template <typename T>
 cudaError_t launch_apply_ug(Q4<T>* psi, const Q4<T>* ug, size_t n, cudaStream_t st);
+template <typename T>
+cudaError_t launch_apply_ug_t(Q4<T>* psi, const Q4<T>* ug_t, int nx, int ny, cudaStream_t st);
 
 // The team pass for one line length (256..4096; one translation unit each, team_<L>.cu), and
 // one phase (1 or 2) of the unsplit operator.

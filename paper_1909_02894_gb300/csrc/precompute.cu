@@ -237,16 +237,18 @@ __device__ inline void pauli_exp_general(Z v1, Z v2, Z v3, double phi, Z* d) {
   d[3] = zadd(zmul(e, m11), em1);
 }
 
-// U and U^2 with potentials (normal layout), two Q4 per point:
-// (d00.re, d00.im, u01.re, u01.im), (u10.re, u10.im, d11.re, d11.im).
+// U and U^2 with potentials, two Q4 per point: (d00.re, d00.im, u01.re, u01.im), (u10.re,
+// u10.im, d11.re, d11.im), in the normal layout or (transposed) in that of the y pass that applies
+// them. Bound by the FP64 exponentials (1.6 ms for 512 x 2048 points): the transposed writes, whole
+// 32-byte sectors in complex64, hide behind them.
 template <typename T>
 __global__ void k_halfstep_general(const double* a1, const double* a2, const double* meff,
                                    const double* omx, const double* omy, const double* V,
                                    const double* Ax, const double* Ay, int nx, int ny,
-                                   double dt, Q4<T>* ug, Q4<T>* ug2, Q4<T>* ug_t, Q4<T>* ug2_t) {
+                                   double dt, int transposed, Q4<T>* ug, Q4<T>* ug2) {
   const size_t k = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= (size_t)nx * ny) return;
-  const size_t row = k / nx, t = (k - row * nx) * ny + row;  // the point's transposed index
+  const size_t row = k / nx, o = transposed ? (k - row * nx) * ny + row : k;
   // exponent -i dt/2 [meff sigma_z + F], F = -i sum_j a^j Omega_j sigma_j
   //   - sum_j a^j A_j sigma_j + V I
   const Z v1 = {-0.5 * dt * a1[k] * omx[k], Ax ? 0.5 * dt * a1[k] * Ax[k] : 0.0};
@@ -255,29 +257,45 @@ __global__ void k_halfstep_general(const double* a1, const double* a2, const dou
   const double phi = V ? -0.5 * dt * V[k] : 0.0;
   Z d[4];
   pauli_exp_general(v1, v2, v3, phi, d);
-  ug[2 * k] = {(T)d[0].r, (T)d[0].i, (T)d[1].r, (T)d[1].i};
-  ug[2 * k + 1] = {(T)d[2].r, (T)d[2].i, (T)d[3].r, (T)d[3].i};
-  if (ug_t) {
-    ug_t[2 * t] = ug[2 * k];
-    ug_t[2 * t + 1] = ug[2 * k + 1];
-  }
+  ug[2 * o] = {(T)d[0].r, (T)d[0].i, (T)d[1].r, (T)d[1].i};
+  ug[2 * o + 1] = {(T)d[2].r, (T)d[2].i, (T)d[3].r, (T)d[3].i};
   pauli_exp_general(zscale(v1, 2.0), zscale(v2, 2.0), zscale(v3, 2.0), 2.0 * phi, d);
-  ug2[2 * k] = {(T)d[0].r, (T)d[0].i, (T)d[1].r, (T)d[1].i};
-  ug2[2 * k + 1] = {(T)d[2].r, (T)d[2].i, (T)d[3].r, (T)d[3].i};
-  if (ug2_t) {
-    ug2_t[2 * t] = ug2[2 * k];
-    ug2_t[2 * t + 1] = ug2[2 * k + 1];
-  }
+  ug2[2 * o] = {(T)d[0].r, (T)d[0].i, (T)d[1].r, (T)d[1].i};
+  ug2[2 * o + 1] = {(T)d[2].r, (T)d[2].i, (T)d[3].r, (T)d[3].i};
 }
 
 template <typename T>
 cudaError_t launch_halfstep_general(const double* a1, const double* a2, const double* meff,
                                     const double* omx, const double* omy, const double* V,
                                     const double* Ax, const double* Ay, int nx, int ny,
-                                    double dt, Q4<T>* ug, Q4<T>* ug2, Q4<T>* ug_t, Q4<T>* ug2_t,
+                                    double dt, bool transposed, Q4<T>* ug, Q4<T>* ug2,
                                     cudaStream_t st) {
   k_halfstep_general<T><<<nblocks((size_t)nx * ny), TPB, 0, st>>>(
-      a1, a2, meff, omx, omy, V, Ax, Ay, nx, ny, dt, ug, ug2, ug_t, ug2_t);
+      a1, a2, meff, omx, omy, V, Ax, Ay, nx, ny, dt, transposed, ug, ug2);
+  return cudaGetLastError();
+}
+
+// psi <- U psi (normal layout) with a general U in the transposed layout: a block turns a tile of
+// U through shared memory, 512 bytes in a row.
+constexpr int TILE = 16;
+static_assert(TPB == TILE * TILE, "a block makes one tile");
+template <typename T>
+__global__ void k_apply_ug_t(Q4<T>* psi, const Q4<T>* ug_t, int nx, int ny) {
+  __shared__ Q4<T> tile[2][TILE][TILE + 1];
+  const int c = threadIdx.x % TILE, r = threadIdx.x / TILE;
+  const int x0 = (int)(blockIdx.x % (nx / TILE)) * TILE, y0 = (int)(blockIdx.x / (nx / TILE)) * TILE;
+  const size_t t = (size_t)(x0 + r) * ny + y0 + c, k = (size_t)(y0 + r) * nx + x0 + c;
+  const Q4<T> p = psi[k];  // beside the tile: after it cost 2 us at 512 x 2048 (16 against 18)
+  tile[0][r][c] = ug_t[2 * t];
+  tile[1][r][c] = ug_t[2 * t + 1];
+  __syncthreads();
+  psi[k] = apply_u_general(tile[0][c][r], tile[1][c][r], p);
+}
+
+template <typename T>
+cudaError_t launch_apply_ug_t(Q4<T>* psi, const Q4<T>* ug_t, int nx, int ny, cudaStream_t st) {
+  if (nx % TILE || ny % TILE) return cudaErrorInvalidValue;  // axes are powers of two from 16
+  k_apply_ug_t<T><<<nblocks((size_t)nx * ny), TPB, 0, st>>>(psi, ug_t, nx, ny);
   return cudaGetLastError();
 }
 
@@ -484,8 +502,9 @@ cudaError_t launch_transpose(const Q4<T>* in, Q4<T>* out, int rows, int cols, cu
                                           Q4<T>*, Q4<T>*, Q4<T>*, Q4<T>*, cudaStream_t);     \
   template cudaError_t launch_halfstep_general<T>(                                            \
       const double*, const double*, const double*, const double*, const double*,             \
-      const double*, const double*, const double*, int, int, double, Q4<T>*, Q4<T>*,         \
-      Q4<T>*, Q4<T>*, cudaStream_t);                                                         \
+      const double*, const double*, const double*, int, int, double, bool, Q4<T>*, Q4<T>*,   \
+      cudaStream_t);                                                                         \
+  template cudaError_t launch_apply_ug_t<T>(Q4<T>*, const Q4<T>*, int, int, cudaStream_t);    \
   template cudaError_t launch_twiddles<T>(int, int, Cx<T>*, cudaStream_t);                    \
   template cudaError_t launch_step_mult<T>(int, double, double, Q4<T>*, cudaStream_t);        \
   template cudaError_t launch_team_perm<T>(int, const Q4<T>*, Q4<T>*, cudaStream_t);          \
