@@ -76,6 +76,9 @@ class _Obs(C.Structure):
 
 
 _lib = None
+# what each context runs beyond its grid and precision: [scheme, static potentials set], by
+# handle, from dirac_create to dirac_destroy (the autotuner's cache tells contexts apart by it)
+_routes = {}
 
 
 def build(force: bool = False) -> str:
@@ -183,6 +186,7 @@ def dirac_create(nx: int, ny: int, ax: float, ay: float, *, g00=None, g11=None, 
     st = lib().dirac_create(C.byref(_Grid(nx, ny)), C.byref(_Domain(ax, ay)), C.byref(metric),
                             mass, c, C.byref(absorber), precision, stream, C.byref(out))
     _check(st, None)
+    _routes[out.value] = [DIRAC_SCHEME_II, False]
     return out.value
 
 
@@ -241,6 +245,7 @@ def dirac_set_launch(ctx, threads_x: int, threads_y: int):
 
 def dirac_set_scheme(ctx, scheme: int):
     _check(lib().dirac_set_scheme(ctx, int(scheme)), ctx)
+    _routes.setdefault(ctx, [DIRAC_SCHEME_II, False])[0] = int(scheme)
 
 
 def dirac_set_poly_degree(ctx, degree: int):
@@ -264,6 +269,7 @@ def dirac_set_potentials(ctx, V=None, Ax=None, Ay=None, shape=None):
                 raise ValueError(f"potential shape {a.shape} != {tuple(shape)}")
     ptrs = [None if a is None else a.ctypes.data for a in arrs]
     _check(lib().dirac_set_potentials(ctx, *ptrs), ctx)
+    _routes.setdefault(ctx, [DIRAC_SCHEME_II, False])[1] = any(p is not None for p in ptrs)
 
 
 def dirac_launch_count(ctx) -> int:
@@ -404,6 +410,7 @@ def dirac_batch_destroy(batch):
 
 def dirac_destroy(ctx):
     if ctx:
+        _routes.pop(ctx, None)
         lib().dirac_destroy(ctx)
 
 
