@@ -74,8 +74,9 @@ __device__ __forceinline__ void cluster_barrier() {
 }
 
 // One pass over this CTA's lines of L points. src: their points (pitch L + 1); dst[m]: where
-// component c of point j + m L/8 of this line goes (shared::cluster addresses).
-template <int L, int SIGMA>
+// component c of point j + m L/8 of this line goes (shared::cluster addresses). LINES: lines of
+// the CTA, the bound of the debug build's index checks (no code otherwise).
+template <int L, int SIGMA, int LINES>
 __device__ __forceinline__ void small_pass(const Q4<float>* src, const uint32_t (&dst)[8],
                                            Cx<float>* fft, int line, int j, int c,
                                            const float* beta, const Q4<float>* mult,
@@ -83,16 +84,17 @@ __device__ __forceinline__ void small_pass(const Q4<float>* src, const uint32_t 
                                            const Q4<float>* u_store) {
   constexpr int J = L / 8;
   const float sg = c ? -1.f : 1.f;
-  const Cx<float>* in = reinterpret_cast<const Cx<float>*>(src + (size_t)line * (L + 1)) + c;
+  auto at = [&](int i) { return dbg_at(line * L + i, (size_t)LINES * L); };
+  const Cx<float>* in = reinterpret_cast<const Cx<float>*>(src) + c;
   Cx<float>* buf = fft + line * SGeo<L>::STRIDE + c * SGeo<L>::COMP;
   Cx<float> v[8], p[8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const int i = j + m * J;
-    Cx<float> own = in[2 * i];
+    Cx<float> own = in[2 * dbg_at(line * (L + 1) + i, (size_t)LINES * (L + 1))];
     Cx<float> oth = shfl_pair(own);
     if (u_load) {
-      own = apply_u_row(ldg_q4(u_load + line * L + i), own, oth, c);
+      own = apply_u_row(ldg_q4(u_load + at(i)), own, oth, c);
       oth = shfl_pair(own);
     }
     p[m] = own;
@@ -103,7 +105,7 @@ __device__ __forceinline__ void small_pass(const Q4<float>* src, const uint32_t 
   warp_fft<L, false>(v, buf, j, tw);
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
-    const Q4<float> q = mult[j + m * J];
+    const Q4<float> q = mult[dbg_at(j + m * J, (size_t)L)];
     const float vr = v[m].re, vi = v[m].im;
     const float sh = -sg * q.z, sl = -sg * q.w;
     v[m] = {fma_t(q.x, vr, fma_t(-sh, vi, fma_t(-sl, vi, q.y * vr))),
@@ -118,9 +120,9 @@ __device__ __forceinline__ void small_pass(const Q4<float>* src, const uint32_t 
     Cx<float> d;
     if (c == 0) d = cadd_p(dp, dm);
     else d = SIGMA == 0 ? csub_p(dp, dm) : mul_i(csub_p(dp, dm));
-    const float bm1 = beta[line * L + i];
+    const float bm1 = beta[at(i)];
     Cx<float> o = cfma_p(bm1, d, cadd_p(p[m], d));
-    if (u_store) o = apply_u_row(u_store[line * L + i], o, shfl_pair(o), c);
+    if (u_store) o = apply_u_row(u_store[at(i)], o, shfl_pair(o), c);
     st_remote(dst[m], o);
   }
 }
@@ -141,15 +143,16 @@ __global__ void __launch_bounds__(SPlan<LX, LY, NC>::THREADS)
   Cx<float>* fft = reinterpret_cast<Cx<float>*>(sm + S::FFT);
   const int tid = threadIdx.x, rank = (int)cooperative_groups::this_cluster().block_rank();
   const size_t row0 = (size_t)rank * S::ROWS * LX, col0 = (size_t)rank * S::COLS * LY;
+  auto gz = [&](size_t i) { return dbg_at(i, (size_t)LX * LY); };  // points of the global arrays
   pdl_wait();
   pdl_launch_next();
   for (int k = tid; k < S::ROWS * LX; k += S::THREADS) {
-    sa[(k / LX) * S::PX + k % LX] = a.psi[row0 + k];
-    sb1[k] = a.beta1[row0 + k];
+    sa[dbg_at((k / LX) * S::PX + k % LX, S::ROWS * S::PX)] = a.psi[gz(row0 + k)];
+    sb1[k] = a.beta1[gz(row0 + k)];
   }
   for (int k = tid; k < S::COLS * LY; k += S::THREADS) {
-    sb2[k] = a.beta2[col0 + k];
-    if (a.u2_t) su2[k] = a.u2_t[col0 + k];
+    sb2[k] = a.beta2[gz(col0 + k)];
+    if (a.u2_t) su2[k] = a.u2_t[gz(col0 + k)];
   }
   for (int k = tid; k < LX; k += S::THREADS) smx[k] = a.mult_x[k];
   for (int k = tid; k < LY; k += S::THREADS) smy[k] = a.mult_y[k];
@@ -162,24 +165,26 @@ __global__ void __launch_bounds__(SPlan<LX, LY, NC>::THREADS)
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
     const int ix = jx + m * (LX / 8);  // x index of the point: column ix % COLS of CTA ix / COLS
-    dx[m] = shared_of(smem_u32(sb + (ix % S::COLS) * S::PY + rank * S::ROWS + lx) + 8 * c,
-                      ix / S::COLS);
+    dx[m] = shared_of(smem_u32(sb + dbg_at((ix % S::COLS) * S::PY + rank * S::ROWS + lx,
+                                           S::COLS * S::PY)) + 8 * c,
+                      (int)dbg_at(ix / S::COLS, NC));
     const int iy = jy + m * (LY / 8);  // y index: row iy % ROWS of CTA iy / ROWS
-    dy[m] = shared_of(smem_u32(sa + (iy % S::ROWS) * S::PX + rank * S::COLS + ly) + 8 * c,
-                      iy / S::ROWS);
+    dy[m] = shared_of(smem_u32(sa + dbg_at((iy % S::ROWS) * S::PX + rank * S::COLS + ly,
+                                           S::ROWS * S::PX)) + 8 * c,
+                      (int)dbg_at(iy / S::ROWS, NC));
   }
   cluster_barrier();  // every CTA of the cluster runs, its buffers are filled
   for (int s = 0; s < n; ++s) {
-    small_pass<LX, 0>(sa, dx, fft, lx, jx, c, sb1, smx, a.tw_x,
+    small_pass<LX, 0, S::ROWS>(sa, dx, fft, lx, jx, c, sb1, smx, a.tw_x,
                       s == 0 && lead && a.u_n ? a.u_n + row0 : nullptr, nullptr);
     cluster_barrier();
     const Q4<float>* us = a.u2_t ? su2 : nullptr;
     if (s + 1 == n && trail && a.u_t) us = a.u_t + col0;
-    small_pass<LY, 1>(sb, dy, fft, ly, jy, c, sb2, smy, a.tw_y, nullptr, us);
+    small_pass<LY, 1, S::COLS>(sb, dy, fft, ly, jy, c, sb2, smy, a.tw_y, nullptr, us);
     cluster_barrier();
   }
   for (int k = tid; k < S::ROWS * LX; k += S::THREADS)
-    a.psi[row0 + k] = sa[(k / LX) * S::PX + k % LX];
+    a.psi[gz(row0 + k)] = sa[dbg_at((k / LX) * S::PX + k % LX, S::ROWS * S::PX)];
 }
 
 template <int LX, int LY, int NC>
