@@ -206,11 +206,11 @@ long dirac_krylov_iterations(const dirac_ctx *ctx);
  * CTA; complex128: 1 to 4 lines per CTA, 32 to 512 threads), 1024 the radix-16 team pass
  * (complex64, lines of 256..4096 points; L/16 threads per line, the next lines stream into
  * shared memory while the current ones are finished); 0 = the default (complex64: the team
- * pass for lines of 256 points or more, the smaller shape for 128-point lines, else the
- * larger; complex128: the smaller shape for 1024-point lines and lines of 128 points or
- * fewer, else the larger; 512-point lines the smaller when there are fewer than 512; complex64
- * grids whose axes both have 64 or 128 points run whole Scheme II steps, all of a call, in one
- * launch). The
+ * pass for lines of 256 points or more; for shorter ones the smaller shape, but the larger where
+ * lines of 32 points or more have 2^17 points or more together; grids whose axes both have 64 or
+ * 128 points run whole Scheme II steps, all of a call, in one launch. complex128: the smaller
+ * shape for 1024-point lines, for lines of 128 points or fewer and for fewer than 512 lines of
+ * 512 points, else the larger). The
  * smaller shape of lines of 128 points or fewer gives each thread 2 (up to 512 lines) or 4
  * points, the larger takes 16 lines per CTA; 4096-point lines have one shape besides the team
  * pass. 256 or 512 plus

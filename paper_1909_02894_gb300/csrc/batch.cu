@@ -149,8 +149,6 @@ static dirac_status grow_class(dirac_batch* b, Class& c, int need) {
   return DIRAC_OK;
 }
 
-// Fill the host tables of a class for one tick; returns the number of steps any of its
-// contexts takes in this tick.
 // Reads the device error flag (after the work it covers has completed). A bounded wait
 // that ran out leaves every context then in the batch without a valid state: they are
 // marked failed and stop stepping (poll reports DIRAC_ETIMEOUT until they are released),
@@ -174,6 +172,8 @@ static dirac_status batch_device_error(dirac_batch* b, const char* where) {
   return bfail(b, DIRAC_ETIMEOUT, where);
 }
 
+// Fill the host tables of a class for one tick; returns the number of steps any of its
+// contexts takes in this tick.
 template <typename T>
 static int fill_class(dirac_batch* b, Class& c, int K) {
   std::vector<int>& m = c.members;

@@ -94,11 +94,12 @@ static int pass_opt(const dirac_ctx* ctx, int shape, int L, int n_lines) {
   // Default, by measurement: complex64 the team pass for lines of 256 points or more (256^2
   // 0.0109 against 0.0118 ms per step for the radix-8 pass, 1024^2 0.0282 against 0.039); the
   // smaller shape for lines of 128 points or fewer, but for complex64 lines of 32 points or more
-  // only up to 2^17 points (128 x 1024 0.0137 against 0.0139 ms per step, 128 x 2048 0.0201
-  // against 0.0155, 64 x 1024 0.0121 against 0.0117, 32 x 4096 0.0218 against 0.0200), and, in
+  // only below 2^17 points (smaller | larger x pass, ms per step: 32 x 2048 0.0135 | 0.0151, 64 x
+  // 1024 0.0121 | 0.0118, 128 x 512 0.0127 | 0.0125, at 2^17 32 x 4096 0.0218 | 0.0200, 64 x 2048
+  // 0.0170 | 0.0134, 128 x 1024 0.0137 | 0.0138, above it 128 x 2048 0.0202 | 0.0154), and, in
   // complex128, for 1024-point lines (one line per CTA: 1024 CTAs spread over the SMs to within
-  // one line, 0.74 against 0.89 ms per 1024^2 step) and fewer than 512 lines of 512 points (512
-  // x 256: 0.104 against 0.165 ms per step); else the larger.
+  // one line, 0.636 against 0.761 ms per 1024^2 step) and fewer than 512 lines of 512 points (512
+  // x 256: 0.125 against 0.144 ms per step with both passes in one shape); else the larger.
   if (ctx->prec == DIRAC_C64) {
     if (L >= 256) return 2;
     return L >= 32 && (size_t)L * n_lines >= kWideShortLines ? 1 : 0;

@@ -68,8 +68,8 @@ int line_pass_radix(int L);
 // launch options 3 and 4 run it, with a twiddle table of that radix in tw_alt.
 template <typename T>
 int line_pass_radix_alt(int L);
-// Short complex64 lines (32 to 128 points): from this many points the larger shape is the
-// faster one (see pass_opt in dirac_api.cu).
+// Short complex64 lines (32 to 128 points): from this many points on the larger shape is taken
+// (see pass_opt in dirac_api.cu).
 constexpr size_t kWideShortLines = (size_t)1 << 17;
 // Elements per thread of launch option 0 and of the derivative mode for lines of 128 points
 // or fewer (0: longer lines), with a twiddle table of that radix in tw_small.
@@ -194,10 +194,6 @@ cudaError_t launch_unsplit_combine(const Q4<T>* dx, const Q4<T>* dy, const doubl
                                    int ny, double ar, double ai, const Q4<T>* base, double gr,
                                    double gi, const Q4<T>* prev, double beta, Q4<T>* out,
                                    cudaStream_t st);
-// out = c in.
-template <typename T>
-cudaError_t launch_scale(Q4<T>* out, const Q4<T>* in, double cr, double ci, size_t n,
-                         cudaStream_t st);
 // Per-block maxima of |b1|, |b2| into partials[2 * n_blocks].
 cudaError_t launch_max_b(const double* a1, const double* a2, const double* sxinv,
                          const double* syinv, const double* sxinv_im, const double* syinv_im,

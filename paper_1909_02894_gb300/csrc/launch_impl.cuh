@@ -64,10 +64,10 @@ static cudaError_t launch_one(const LinePassArgs<T>& a, cudaStream_t st) {
 //   FP32 (E = 8 from 256 points): 256: 4|8, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1
 //     (256|512 threads, 512|1024 at 2048, 1024 at 4096)
 //   FP64 (E = 16 from 2048 points): 256: 1|2, 512: 2|4, 1024: 1|2, 2048: 1|2, 4096: 1 (64..512 threads).
-//     The FP64 pass is bound by the FP64 units and its CTAs hold 128-162 registers per
-//     thread, so few CTAs fit an SM: small CTAs keep all 152 SMs evenly loaded. Measured on
-//     the strained-graphene grids (ms per step, opt 0 | opt 1): 512^2 0.203 | 0.199, 1024^2
-//     0.741 | 0.886, 2048^2 3.61 | 3.20.
+//     The FP64 pass is bound by the FP64 units and its CTAs hold 96-172 registers per
+//     thread, so few CTAs fit an SM: small CTAs keep all 152 SMs evenly loaded. Measured (ms per
+//     step, opt 0 | opt 1): 256^2 0.0497 | 0.0500, 512^2 0.1717 | 0.1714, 1024^2 0.636 | 0.761,
+//     2048^2 3.21 | 2.82.
 //   both, 128 points or fewer: as few lines as fill a warp or two with radix_small elements per
 //     thread (16 points 4 | 2, 32 points 2 | 1 for E = 4 | 2, 64 and 128 points 1) | 16 lines.
 //     A full GPU prefers the larger shape (100 complex64 128^2 instances: 0.074 ms per step

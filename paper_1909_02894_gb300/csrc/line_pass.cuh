@@ -233,7 +233,7 @@ __device__ __forceinline__ void dft16(Cx<T> (&x)[16], const Cx<T>* __restrict__ 
 }
 
 // ---- FP64 butterflies in fused multiply-adds. The FP64 pass is bound by the number of FP64
-// instructions (the pipe is 85 % busy), so every twiddle w = c (1 + i tau) is applied in two
+// instructions (at 1024^2 the pipe is busy 87 % of the active cycles), so every twiddle w = c (1 + i tau) is applied in two
 // steps that fuse: u = x (1 + i tau) costs two FMAs, and the factor c goes into the additions
 // that follow (Linzer and Feig's scheme). A DFT-4 with three twiddles takes 22 instructions
 // instead of 28, with four 28 instead of 32; DFT-16 144 instead of 160 (its inner twiddles are

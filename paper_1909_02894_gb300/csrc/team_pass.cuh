@@ -19,8 +19,10 @@
 // together as whole 32-byte sectors straight from registers; otherwise the CTA's LPC lines
 // are staged in shared memory and leave in segments of LPC points.
 //
-// What bounds it (4096^2 and 2048^2, ncu): the shared-memory/L1 data pipe (exchanges: 128 B
-// per point) and instruction issue, both about half busy; 16 warps of 128 registers per SM.
+// What bounds it, by ncu (profiles/line_pass_team_*.md): at 4096^2 the shared-memory/L1 data pipe
+// (exchanges: 128 B per point) and instruction issue, both about half busy, with 16 warps of 128
+// registers per SM; at 1024^2, whose 512 pairs of lines make 256 CTAs, latency: 6.4 warps per SM,
+// issue 23..25 % and data pipe 31..35 % busy.
 // Measured per step of two passes, against the design before it (one 1024-thread CTA per SM
 // in radix 8 with one eigencomponent per thread, three exchanges per FFT): 4096^2 0.507 ->
 // 0.370 ms, 2048^2 0.165 -> 0.085, 1024^2 0.0439 -> 0.0291 (all three with programmatic

@@ -11,8 +11,8 @@
 // components of its points, so the 2 x 2 algebra needs no exchange. Bound like the step pass,
 // and by the latency of the coefficient and term loads of the epilogue (up to 52 B per point);
 // phase 1 stores twice as much (two transposed arrays). Measured with the whole scheme around
-// it: Chebyshev of degree 8 at 1024^2 0.52 -> 0.30 ms per step (0.0175 and 0.0257 ms per phase
-// under ncu, against 0.064 for the four launches).
+// it: Chebyshev of degree 8 at 1024^2 0.52 -> 0.29 ms per step (0.0193 and 0.0275 ms per phase
+// under ncu, profiles/unsplit_chebyshev1024.md, against 0.064 for the four launches).
 #pragma once
 #include "team_pass.cuh"
 

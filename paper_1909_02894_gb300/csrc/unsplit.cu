@@ -109,9 +109,8 @@ __global__ void k_max_b(const double* a1, const double* a2, const double* sxinv,
 // remainder (an FMA), and both are added to a sum of three FP32 terms by two-sums (Knuth; the
 // scheme of Ogita, Rump and Oishi's DotK with K = 3, threefold FP32 precision), within 8
 // points of a thread and across the 32 lanes of a warp; everything beyond is added in FP64.
-// Error of a product of unit vectors against the exact sum, 4096 to 2^20 points (noise and wave
-// packets, emulated): at most 2.8e-17, the same as FP64 fused multiply-adds per thread (rms
-// 1.3e-19..1.2e-17 and 1.1e-19..1.2e-17).
+// Error of a product of unit vectors against the exact sum, 4096 to 2^18 points (noise and wave
+// packets, emulated in tests/test_krylov_sums_cpu.py): at most one FP64 rounding, 1.1e-16.
 template <typename T>
 struct DotAcc;
 template <>
