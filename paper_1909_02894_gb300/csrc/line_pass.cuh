@@ -331,7 +331,7 @@ __device__ __forceinline__ void dft8_outer(Cx<double> (&x)[8], Cx<double> e0, Cx
   x[7] = fma_c(kC2, u3, e3);
 }
 // R-point butterfly with the pass's twiddles (tw: this k's first slot, step between slots):
-// the slots hold the pairs that the twiddle kernel's tan_pair gives.
+// the slots hold the pairs that the twiddle kernel's tan_half gives.
 template <int R, bool INV>
 __device__ __forceinline__ void tw_dft(Cx<double> (&x)[R], const Cx<double>* __restrict__ tw,
                                        int step) {

@@ -317,36 +317,52 @@ __device__ inline void split(double v, T* hi, T* lo) {
   *lo = (T)(v - (double)h);
 }
 
-// Per-pass twiddle blocks (layout in line_pass.cuh, tw_offset) for E elements per
-// thread: for every pass after the first, span NS (E, E^2, ...) and radix R (E, or the
-// remaining radix for the last pass), entries [(t - 1) NS + k] = exp(-2 pi i t k/(NS R)).
-// Computed in FP64.
-// Slot i (0..r-2) of the FP64 butterflies' twiddles w_t = exp(-2 pi i t phase) = c_t (1 + i
-// tau_t), see tw_dft: groups of a DFT-4 with x0 untwiddled, factors t1..t3: (tau1, tau2), (tau3,
-// c2), (c1, c3/c1); with four factors: (tau0, tau1), (tau2, tau3), (c2/c0, c3/c1), (c0, c1).
-__device__ inline double2 tan_pair(int r, int i, double phase) {
+// One half of slot i (0..r-2) of the FP64 butterflies' twiddles w_t = exp(-2 pi i t phase) = c_t
+// (1 + i tau_t), see tw_dft: groups of a DFT-4 with x0 untwiddled, factors t1..t3: (tau1, tau2),
+// (tau3, c2), (c1, c3/c1); with four factors: (tau0, tau1), (tau2, tau3), (c2/c0, c3/c1), (c0,
+// c1). Every half is a sine or cosine over a cosine (or 1).
+__device__ inline double tan_half(int r, int i, int half, double phase) {
   auto c = [&](int t) {
     const double v = cospi(2.0 * t * phase), least = 8.673617379884035e-19;  // 2^-60
     return fabs(v) < least ? copysign(least, v) : v;
   };
-  auto tau = [&](int t) { return -sinpi(2.0 * t * phase) / c(t); };
-  if (r == 2) return make_double2(tau(1), c(1));
-  // stride between the factors of a group, first group's t1
-  const int d = r / 4;
-  if (i < 3)
-    return i == 0   ? make_double2(tau(d), tau(2 * d))
-           : i == 1 ? make_double2(tau(3 * d), c(2 * d))
-                    : make_double2(c(d), c(3 * d) / c(d));
-  const int g = (i - 3) / 4 + 1, s = (i - 3) % 4;  // group g: factors g, g + d, g + 2 d, g + 3 d
-  return s == 0   ? make_double2(tau(g), tau(g + d))
-         : s == 1 ? make_double2(tau(g + 2 * d), tau(g + 3 * d))
-         : s == 2 ? make_double2(c(g + 2 * d) / c(g), c(g + 3 * d) / c(g + d))
-                  : make_double2(c(g), c(g + d));
+  int tau = 0, num = 0, den = 0;  // tau_t: -sin_t / c_t; else c_num / c_den (den = 0: c_num)
+  if (r == 2) {
+    if (half) num = 1;
+    else tau = 1;
+  } else {
+    // stride between the factors of a group; group g: factors g, g + d, g + 2 d, g + 3 d
+    const int d = r / 4, g = i < 3 ? 0 : (i - 3) / 4 + 1;
+    const int kind = i < 3 ? i : (i - 3) % 4, a = g + half * d;
+    if (i < 3) {
+      if (kind == 0) tau = (1 + half) * d;
+      else if (kind == 1) (half ? num : tau) = half ? 2 * d : 3 * d;
+      else if (half) num = 3 * d, den = d;
+      else num = d;
+    } else if (kind < 2) {
+      tau = a + kind * 2 * d;
+    } else if (kind == 2) {
+      num = a + 2 * d;
+      den = a;
+    } else {
+      num = a;
+    }
+  }
+  const double n = tau ? -sinpi(2.0 * tau * phase) : c(num);
+  const int q = tau ? tau : den;
+  return q ? n / c(q) : n;
 }
 
+// Per-pass twiddle blocks (layout in line_pass.cuh, tw_offset) for E elements per
+// thread: for every pass after the first, span NS (E, E^2, ...) and radix R (E, or the
+// remaining radix for the last pass), entries [(t - 1) NS + k] = exp(-2 pi i t k/(NS R)).
+// Computed in FP64. complex128: a thread makes half an entry, since one thread's chain of up to
+// eight sines and cosines and two quotients made creating a context up to 5 % dearer (512 x 16:
+// 564 -> 594 us against entries of one sine and cosine; now 541).
 template <typename T>
 __global__ void k_twiddles(int n, int e, Cx<T>* tw) {
-  const int m = blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr int PARTS = sizeof(T) == 8 ? 2 : 1;
+  const int id = blockIdx.x * blockDim.x + threadIdx.x, m = id / PARTS;
   if (m >= n) return;
   int log2n = 0, log2e = 0;
   while ((1 << log2n) < n) ++log2n;
@@ -358,24 +374,24 @@ __global__ void k_twiddles(int n, int e, Cx<T>* tw) {
     const int cnt = (r - 1) * ns;
     if (m < off + cnt) {
       const int t = (m - off) / ns + 1, k = (m - off) % ns;
-      if constexpr (sizeof(T) == 8) {
-        const double2 p = tan_pair(r, t - 1, (double)k / ((double)ns * r));
-        tw[m] = {(T)p.x, (T)p.y};
-        return;
+      if constexpr (PARTS == 2) {
+        reinterpret_cast<T*>(tw)[id] = tan_half(r, t - 1, id & 1, (double)k / ((double)ns * r));
+      } else {
+        double s, c;
+        sincospi(2.0 * (double)t * k / ((double)ns * r), &s, &c);
+        tw[m] = {(T)c, (T)(-s)};
       }
-      double s, c;
-      sincospi(2.0 * (double)t * k / ((double)ns * r), &s, &c);
-      tw[m] = {(T)c, (T)(-s)};
       return;
     }
     off += cnt;
   }
-  tw[m] = {(T)1, (T)0};  // unused entries
+  if constexpr (PARTS == 2) reinterpret_cast<T*>(tw)[id] = id & 1 ? T(0) : T(1);
+  else tw[m] = {(T)1, (T)0};  // unused entries
 }
 
 template <typename T>
 cudaError_t launch_twiddles(int n, int e, Cx<T>* tw, cudaStream_t st) {
-  k_twiddles<T><<<nblocks(n), TPB, 0, st>>>(n, e, tw);
+  k_twiddles<T><<<nblocks((size_t)n * (sizeof(T) == 8 ? 2 : 1)), TPB, 0, st>>>(n, e, tw);
   return cudaGetLastError();
 }
 
