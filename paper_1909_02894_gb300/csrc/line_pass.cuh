@@ -239,7 +239,8 @@ __device__ __forceinline__ void dft16(Cx<T> (&x)[16], const Cx<T>* __restrict__ 
 // instead of 28, with four 28 instead of 32; DFT-16 144 instead of 160 (its inner twiddles are
 // constants), 186 instead of 220 with its 15 outer ones. Where |c| < 2^-60 the table holds
 // 2^-60: u is then at most 2^60 |x|, and what is lost is below the rounding of x w. Rounding
-// errors are those of the usual product (each is relative to |x|).
+// errors are those of the usual product (each is relative to |x|). Amplitudes above about 1e290
+// overflow in u; their norm, |psi|^2, has left the FP64 range long before (from 1e154).
 __device__ __forceinline__ Cx<double> fma_c(double s, Cx<double> a, Cx<double> b) {  // s a + b
   return {fma(s, a.re, b.re), fma(s, a.im, b.im)};
 }
